@@ -204,8 +204,14 @@ int ep_cost(ep_schedule *s, int64_t *loads, int64_t *vertex_cut, void *stream);
  *     With tau = 0, x is unchanged and out = flux(x).
  *   EP_KERNEL_SPMV (bipartite schedule): x float[n] (read), w float[m],
  *     out float[n] = y (written), D = 1, steps = 1, tau ignored.
+ * A flux run of two or more steps under the default kernel organisation
+ * (ep_set_pipeline 2..8, EP_CACHE_SMEM, no halo) is one cooperative launch that
+ * keeps the mesh on the chip, one part of it per SM, when the parts fit shared
+ * memory (for D = 5 on mesh-like graphs up to about a million vertices) and no
+ * vertex is in more than 192 tasks; other runs launch one edge kernel a step.
+ * Both give the same results up to FP32 rounding order.
  * Uses schedule-owned device workspace (allocated on first use: make the
- * first call before any stream capture).  Every kernel stages a whole
+ * first call before any stream capture).  Every step kernel stages a whole
  * schedule block in shared memory: EP_EINVAL (nothing launched) when the
  * largest block does not fit, i.e. C too large for the graph and D (for
  * D = 5 on mesh-like graphs, C up to a few thousand tasks fits).
@@ -357,7 +363,9 @@ int ep_batch(ep_schedule *const *parts, int32_t count, ep_schedule **out);
  * its own stream; ep_timing_read() waits for the recorded events and returns
  * the summed device time and launch count of one kernel class since the last
  * reset:
- *   EP_T_EDGE_FWD  flux edge kernel (forward)      EP_T_BND   shared-vertex update
+ *   EP_T_EDGE_FWD  flux edge kernel (forward; one launch per step, or per
+ *                  run where ep_run keeps the mesh on the chip)
+ *   EP_T_BND       shared-vertex update
  *   EP_T_EDGE_ADJ  flux edge kernel (adjoint)      EP_T_SPMV  SpMV edge kernel
  *   EP_T_LAYOUT    layout / weight permutations    EP_T_COST  cost kernels
  * enable = 0 turns timing off; enable = 2 clears the totals and keeps it on.
@@ -437,7 +445,8 @@ int ep_pipeline_info(ep_schedule *s, int32_t D, int32_t adjoint, int32_t *grid, 
  * Reads and clears the error word of the pipelined kernels (synchronises
  * `stream`): every wait inside them is bounded, and an expired wait sets a
  * bit here instead of hanging (bit 0: waiting for data, bit 1: waiting for a
- * free stage).  *code = 0 and EP_OK when clean, else EP_ETIMEOUT.
+ * free stage, bit 2: waiting for another part's boundary values in a run kept
+ * on the chip).  *code = 0 and EP_OK when clean, else EP_ETIMEOUT.
  */
 int ep_check_errors(ep_schedule *s, int32_t *code, void *stream);
 
@@ -465,7 +474,9 @@ int ep_set_cache(ep_schedule *s, int32_t mode);
  * nothing arrives), so the consumers' bounded wait for it expires: the
  * launch returns early with bit 0 set in the error word, its results are
  * invalid, and ep_check_errors() reports EP_ETIMEOUT and resets the
- * accumulators.  -1 (default) turns the hook off.
+ * accumulators.  In a run kept on the chip part 0 leaves after that many
+ * steps (at least one), so the wait of its neighbours expires (bit 2).  -1
+ * (default) turns the hook off.
  */
 int ep_debug_stall(ep_schedule *s, int32_t block_index);
 

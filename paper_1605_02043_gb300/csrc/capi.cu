@@ -138,7 +138,7 @@ struct ep_schedule {
   int tpb_adj = 352;  // consumer threads of the adjoint kernels
   bool bacc_dirty = true;
   // device copy of the schedule
-  DBuf d_desc, d_flist, d_ylist, d_ent, d_perm, d_wmap, d_rec, d_xrec, d_yrec, d_bptr, d_eu,
+  DBuf d_desc, d_flist, d_ylist, d_ent, d_wmap, d_rec, d_xrec, d_yrec, d_bptr, d_eu,
       d_ev;
   DBuf d_sidx, d_soff, d_sid, d_gslot, d_frec, d_fsid;  // flux layout
   // workspace
@@ -147,7 +147,7 @@ struct ep_schedule {
   // vertex-ordered maps for inputs read from host memory (built on first use):
   // records of every vertex (CSR) and the weight slots of every task (2 each)
   DBuf d_hptr, d_hrec, d_tslot;
-  bool host_maps = false;
+  bool host_maps = false, task_slots = false;
   // shard halo (ep_set_halo): shared id of every halo vertex here, -1 if untouched
   std::vector<int32_t> hmap;
   DBuf d_hmap;
@@ -169,6 +169,16 @@ struct ep_schedule {
   // steps inside a stream capture only enqueue work
   ep::dev::TmaPlan plans[EP_MAX_D + 1][2];
   int plan_key[EP_MAX_D + 1][2] = {};
+  // resident runs of several steps (march.h): the host layout until it is
+  // uploaded, its device copy, the run's workspace and the launch plans
+  ep::MarchLayout ml;
+  bool march = false, march_up = false;
+  bool march_dirty = true;  // the exchange records and the parts' counts need clearing
+  int32_t march_D = 0;      // state width they were last used with
+  DBuf d_mpart, d_mhalo, d_mnbr, d_moff, d_ment, d_mwmap, d_mrec;
+  DBuf ws_mx, ws_mw, ws_mout, ws_mex, ws_mflag;
+  ep::dev::MarchPlan mplans[EP_MAX_D + 1];
+  bool mplan_set[EP_MAX_D + 1] = {};
 };
 
 namespace {
@@ -176,12 +186,13 @@ namespace {
 bool bipartite(const ep_schedule* s) { return (s->h.flags & EP_BIPARTITE) != 0; }
 
 constexpr int kCtlWords = 4;
+constexpr int32_t kMarchParts = 152;  // one part per SM of the GPU the library is built for
 
 #define CU(call)                                                                          \
   do {                                                                                    \
     cudaError_t e_ = (call);                                                              \
     if (e_ != cudaSuccess) {                                                              \
-      s->bacc_dirty = true;                                                               \
+      s->bacc_dirty = s->march_dirty = true;                                              \
       return fail(EP_ECUDA, "%s: %s (%s:%d)", #call, cudaGetErrorString(e_), __FILE__, __LINE__); \
     }                                                                                     \
   } while (0)
@@ -201,16 +212,6 @@ int ensure_device(ep_schedule* s) {
     return EP_OK;
   }
   const ep::HostSchedule& h = s->h;
-  std::vector<int32_t> eu(h.m), ev(h.m);
-  for (int64_t i = 0; i < h.m; ++i) {
-    const int32_t e = h.edge_perm[i];
-    eu[i] = bipartite(s) ? (int32_t)(h.n + h.src[e]) : h.src[e];
-    ev[i] = h.dst[e];
-  }
-  CU(upload(s->d_eu, eu));
-  CU(upload(s->d_ev, ev));
-  CU(upload(s->d_bptr, h.block_ptr));
-  CU(upload(s->d_perm, h.edge_perm));
   if (bipartite(s)) {
     CU(upload(s->d_desc, h.sdesc));
     CU(upload(s->d_flist, h.xlist));
@@ -249,9 +250,27 @@ const void* host_mapped(const void* p) {
 }
 
 // Maps for reading inputs in vertex / task order: every record of a vertex
-// (CSR over the data vertices) and the weight slots of every task.
+// (CSR over the data vertices, flux schedules) and the weight slots of every
+// task (for weights in host memory).
 int ensure_host_maps(ep_schedule* s) {
-  if (s->host_maps) return EP_OK;
+  if (s->host_maps || bipartite(s)) return EP_OK;
+  const ep::HostSchedule& h = s->h;
+  std::vector<int32_t> ptr(h.nd + 1, 0), rec;
+  for (int32_t v : h.vrec)
+    if (v >= 0) ++ptr[v + 1];
+  for (int64_t v = 0; v < h.nd; ++v) ptr[v + 1] += ptr[v];
+  rec.resize(ptr[h.nd]);
+  std::vector<int32_t> fill(ptr.begin(), ptr.end() - 1);
+  for (size_t r = 0; r < h.vrec.size(); ++r)
+    if (h.vrec[r] >= 0) rec[fill[h.vrec[r]]++] = (int32_t)r;
+  CU(upload(s->d_hptr, ptr));
+  CU(upload(s->d_hrec, rec));
+  s->host_maps = true;
+  return EP_OK;
+}
+
+int ensure_task_slots(ep_schedule* s) {
+  if (s->task_slots) return EP_OK;
   const ep::HostSchedule& h = s->h;
   std::vector<int32_t> tslot(2 * (size_t)h.m, -1);
   for (size_t j = 0; j < h.wmap.size(); ++j) {
@@ -260,20 +279,8 @@ int ensure_host_maps(ep_schedule* s) {
     int32_t* sl = &tslot[2 * (size_t)t];
     (sl[0] < 0 ? sl[0] : sl[1]) = (int32_t)j;
   }
-  if (!bipartite(s)) {
-    std::vector<int32_t> ptr(h.nd + 1, 0), rec;
-    for (int32_t v : h.vrec)
-      if (v >= 0) ++ptr[v + 1];
-    for (int64_t v = 0; v < h.nd; ++v) ptr[v + 1] += ptr[v];
-    rec.resize(ptr[h.nd]);
-    std::vector<int32_t> fill(ptr.begin(), ptr.end() - 1);
-    for (size_t r = 0; r < h.vrec.size(); ++r)
-      if (h.vrec[r] >= 0) rec[fill[h.vrec[r]]++] = (int32_t)r;
-    CU(upload(s->d_hptr, ptr));
-    CU(upload(s->d_hrec, rec));
-  }
   CU(upload(s->d_tslot, tslot));
-  s->host_maps = true;
+  s->task_slots = true;
   return EP_OK;
 }
 
@@ -412,6 +419,92 @@ int ensure_bacc(ep_schedule* s, int32_t D, cudaStream_t st) {
     s->bacc_dirty = false;
   }
   return EP_OK;
+}
+
+int ensure_ctl(ep_schedule* s, cudaStream_t st) {
+  if (s->ws_ctl.p) return EP_OK;
+  CU(s->ws_ctl.ensure(kCtlWords * sizeof(int)));
+  CU(cudaMemsetAsync(s->ws_ctl.p, 0, kCtlWords * sizeof(int), st));
+  return EP_OK;
+}
+
+// Plan, device copy and workspace of resident runs at state width D; P.parts
+// stays 0 where a run cannot be resident: the graph does not suit the layout,
+// a part does not fit an SM, the GPU has fewer SMs than parts, or another
+// kernel organisation was asked for (one block per kernel block, read-only
+// cache, a shard's halo).
+int ensure_march(ep_schedule* s, int32_t D, ep::dev::MarchPlan& P, cudaStream_t st) {
+  P.parts = 0;
+  if (!s->march || s->stages == 0 || s->cache != EP_CACHE_SMEM || !s->h.halo.empty()) return EP_OK;
+  const ep::MarchLayout& L = s->ml;
+  if (!s->mplan_set[D]) {
+    int dev = 0, optin = 0, sms = 0, coop = 0;
+    CU(cudaGetDevice(&dev));
+    CU(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    CU(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+    ep::dev::MarchPlan& Q = s->mplans[D];
+    const int smem_max = optin - 512;  // less the kernel's static shared memory
+    Q = ep::dev::march_plan({L.parts, L.max_pos, L.max_col, L.max_nsl}, D, smem_max);
+    if (!coop || sms < L.parts) Q.parts = 0;
+    if (Q.parts) {
+      const void* k = ep::dev::march_kernel_ptr(D, Q.resident);
+      CU(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
+      int per_sm = 0;
+      CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, Q.threads, Q.smem));
+      if (per_sm < 1) Q.parts = 0;
+    }
+    s->mplan_set[D] = true;
+  }
+  P = s->mplans[D];
+  if (!P.parts) return EP_OK;
+  if (!s->march_up) {
+    CU(upload(s->d_mpart, L.part));
+    CU(upload(s->d_mhalo, L.halo));
+    CU(upload(s->d_mnbr, L.nbr));
+    CU(upload(s->d_moff, L.moff));
+    CU(upload(s->d_ment, L.ent));
+    CU(upload(s->d_mwmap, L.wmap));
+    CU(upload(s->d_mrec, L.rec_of));
+    s->march_up = true;
+    s->march_dirty = true;
+  }
+  CU(s->ws_mx.ensure((size_t)L.n_rec * D * sizeof(float)));
+  CU(s->ws_mw.ensure((size_t)L.n_col * 64 * sizeof(float)));
+  const size_t ex_bytes = 2 * (size_t)L.n_rec * ep::dev::ex_chunks(D) * 16;
+  if (ex_bytes > s->ws_mex.bytes || D != s->march_D) s->march_dirty = true;  // other records
+  s->march_D = D;
+  CU(s->ws_mex.ensure(ex_bytes));
+  CU(s->ws_mflag.ensure((size_t)L.parts * sizeof(uint32_t)));
+  if (s->march_dirty) {  // no stale tag: every record cleared, counts from 0
+    CU(cudaMemsetAsync(s->ws_mflag.p, 0, s->ws_mflag.bytes, st));
+    CU(cudaMemsetAsync(s->ws_mex.p, 0, s->ws_mex.bytes, st));
+    s->march_dirty = false;
+  }
+  return ensure_ctl(s, st);
+}
+
+ep::dev::MarchArgs march_args(ep_schedule* s, const float* w, const float* x_in, float* x_out, float* out,
+                              int32_t steps, float tau) {
+  ep::dev::MarchArgs a = {};
+  a.part = s->d_mpart.as<ep::MarchPart>();
+  a.halo = s->d_mhalo.as<int32_t>();
+  a.nbr = s->d_mnbr.as<int32_t>();
+  a.moff = s->d_moff.as<uint16_t>();
+  a.ent = s->d_ment.as<uint32_t>();
+  a.w = w;
+  a.x_in = x_in;
+  a.x_out = x_out;
+  a.out = out;
+  a.every = 1;
+  a.ex = s->ws_mex.as<float>();
+  a.flag = s->ws_mflag.as<uint32_t>();
+  a.err = s->ws_ctl.as<int>() + 2;
+  a.n_rec = s->ml.n_rec;
+  a.steps = steps;
+  a.tau = tau;
+  a.stall = s->stall;
+  return a;
 }
 
 // The one-block kernels stage a whole schedule block in shared memory.
@@ -563,7 +656,7 @@ int weights_to_ws(ep_schedule* s, const float* w, bool from_host, cudaStream_t s
     s->zeroed_w = nullptr;
     return EP_OK;
   }
-  if (int rc = ensure_host_maps(s)) return rc;
+  if (int rc = ensure_task_slots(s)) return rc;
   if (s->zeroed_w != s->ws_w.p) {
     CU(cudaMemsetAsync(s->ws_w.p, 0, s->ws_w.bytes, st));
     s->zeroed_w = s->ws_w.p;
@@ -640,6 +733,7 @@ int fill_partition(ep_schedule* s, const int32_t* src, const int32_t* dst, int64
     if (stop && stop->load()) return fail(EP_ECANCELED, "partition cancelled");
     std::string err = ep::build_schedule(h, threads);
     if (!err.empty()) return fail(EP_EINVAL, "%s", err.c_str());
+    s->march = ep::build_march(h, kMarchParts, threads, s->ml);
   } catch (const std::bad_alloc&) {
     return fail(EP_ENOMEM, "out of host memory");
   }
@@ -872,6 +966,7 @@ int ep_batch(ep_schedule* const* parts, int32_t count, ep_schedule** out) {
       delete s;
       return fail(EP_EINVAL, "%s", err.c_str());
     }
+    s->march = ep::build_march(h, kMarchParts, 0, s->ml);
   } catch (const std::bad_alloc&) {
     delete s;
     return fail(EP_ENOMEM, "out of host memory");
@@ -917,6 +1012,18 @@ int ep_cost(ep_schedule* s, int64_t* loads, int64_t* vertex_cut, void* stream) {
   if (!s) return fail(EP_EINVAL, "null schedule");
   if (int rc = ensure_device(s)) return rc;
   cudaStream_t st = as_stream(stream);
+  if (!s->d_bptr.p) {  // endpoints in schedule order, on first use (nothing else reads them)
+    const ep::HostSchedule& h = s->h;
+    std::vector<int32_t> eu(h.m), ev(h.m);
+    for (int64_t i = 0; i < h.m; ++i) {
+      const int32_t e = h.edge_perm[i];
+      eu[i] = bipartite(s) ? (int32_t)(h.n + h.src[e]) : h.src[e];
+      ev[i] = h.dst[e];
+    }
+    CU(upload(s->d_eu, eu));
+    CU(upload(s->d_ev, ev));
+    CU(upload(s->d_bptr, h.block_ptr));
+  }
   CU(s->ws_flags.ensure((size_t)s->h.nd));
   CU(s->ws_cnt.ensure(2 * sizeof(unsigned long long)));
   ep::dev::CostArgs a;
@@ -1105,6 +1212,32 @@ int ep_run(ep_schedule* s, int32_t kernel, float* x, const float* w, float* out,
 
 namespace {
 
+// A resident run: the state in and out through the march layout's records.
+int run_march(ep_schedule* s, const ep::dev::MarchPlan& P, int32_t D, int32_t steps, float tau, float* x,
+              const float* w, float* out, bool from_host, cudaStream_t st) {
+  const ep::MarchLayout& L = s->ml;
+  const int32_t* rec = s->d_mrec.as<int32_t>();
+  float *mx = s->ws_mx.as<float>(), *mw = s->ws_mw.as<float>(), *mout = out ? s->ws_mout.as<float>() : nullptr;
+  if (from_host) {  // each weight crosses the host link once
+    CU(s->ws_hw.ensure((size_t)s->h.m * sizeof(float)));
+    CU(cudaMemcpyAsync(s->ws_hw.p, w, (size_t)s->h.m * sizeof(float), cudaMemcpyDefault, st));
+    w = s->ws_hw.as<float>();
+  }
+  CU(ep::dev::layout_in(rec, s->h.nd, L.n_rec, D, x, mx, st, s->t()));
+  CU(ep::dev::gather(s->d_mwmap.as<int32_t>(), 64 * L.n_col, w, mw, st, s->t()));
+  if (mout && s->h.touched < s->h.nd) CU(cudaMemsetAsync(mout, 0, (size_t)L.n_rec * D * sizeof(float), st));
+  {
+    ep::dev::Timer* t = s->t();
+    if (t) t->begin(ep::dev::T_EDGE_FWD, st);
+    const cudaError_t e = ep::dev::march_fwd(march_args(s, mw, mx, mx, mout, steps, tau), P, D, st);
+    if (t) t->end(ep::dev::T_EDGE_FWD, st);
+    CU(e);
+  }
+  CU(ep::dev::layout_out(rec, s->h.nd, L.n_rec, D, mx, x, st, s->t()));
+  if (out) CU(ep::dev::layout_out(rec, s->h.nd, L.n_rec, D, mout, out, st, s->t()));
+  return EP_OK;
+}
+
 // ep_run's flux part: x, w and out in the caller's layout, device addresses.
 // from_host: x and w are read in vertex / task order (host memory the GPU
 // reads over the host link).
@@ -1119,6 +1252,14 @@ int run_flux(ep_schedule* s, int32_t D, int32_t steps, float tau, float* x, cons
   }
   fresh_state(s);
   if (int rc = ensure_bacc(s, D, st)) return rc;
+  // every workspace of either path now, whatever `steps`: a later call inside
+  // a stream capture may take the other one
+  ep::dev::MarchPlan P;
+  if (int rc = ensure_march(s, D, P, st)) return rc;
+  if (P.parts && out) CU(s->ws_mout.ensure((size_t)s->ml.n_rec * D * sizeof(float)));
+  CU(s->ws_w.ensure((size_t)wlen_of(s) * sizeof(float)));
+  if (int rc = ensure_host_maps(s)) return rc;
+  if (P.parts && steps > 1) return run_march(s, P, D, steps, tau, x, w, out, from_host, st);
   if (s->zeroed_x != s->ws_x.p) {  // records of no vertex stay zero
     CU(cudaMemsetAsync(s->ws_x.p, 0, s->ws_x.bytes, st));
     s->zeroed_x = s->ws_x.p;
@@ -1312,6 +1453,7 @@ int ep_check_errors(ep_schedule* s, int32_t* code, void* stream) {
   if (v) {
     CU(cudaMemsetAsync(s->ws_ctl.as<int>() + 2, 0, sizeof(int), st));
     s->bacc_dirty = true;  // an interrupted launch may have left partial sums
+    s->march_dirty = true;  // and the parts' counts apart
     return fail(EP_ETIMEOUT, "a pipelined kernel gave up waiting (code %d)", v);
   }
   return EP_OK;
@@ -1363,7 +1505,7 @@ int ep_set_halo(ep_schedule* s, const int32_t* halo, int64_t nh) {
     for (int& k : row) k = 0;
   s->pending[0] = s->pending[1] = false;
   s->bacc_dirty = true;
-  s->host_maps = false;
+  s->host_maps = s->task_slots = false;
   s->zeroed_x = s->zeroed_w = nullptr;
   return EP_OK;
 }

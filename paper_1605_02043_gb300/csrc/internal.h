@@ -5,6 +5,7 @@
 #include <climits>
 #include <cstddef>
 #include <cstdint>
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -135,7 +136,9 @@ bool partition_edges(const int32_t* src, const int32_t* dst, int64_t m, int64_t 
 
 // schedule.cpp: everything after the partition (Definition 4, vertex lists,
 // cpack, cost, kernel layout).  Returns an empty string or an error message.
-std::string build_schedule(HostSchedule& s, int threads);
+// `ordered`, if given, is called once the schedule itself stands (everything
+// but the kernel layout).
+std::string build_schedule(HostSchedule& s, int threads, const std::function<void()>& ordered = {});
 // The flux layout again (after `halo` changed); non-bipartite schedules only.
 std::string rebuild_flux_layout(HostSchedule& s);
 

@@ -6,6 +6,7 @@
 #include <cstdint>
 
 #include "internal.h"
+#include "march.h"
 
 namespace ep {
 namespace dev {
@@ -96,6 +97,43 @@ cudaError_t flux_fwd_tma(const FluxArgs& a, const TmaPlan& P, int D, cudaStream_
 cudaError_t flux_adj_tma(const FluxArgs& a, const TmaPlan& P, int D, float* lam, float* gw,
                          cudaStream_t st);
 const void* flux_tma_kernel_ptr(int D, bool adjoint);
+
+// Resident runs of several steps (march.cu): one CUDA block per part.
+struct MarchArgs {
+  const MarchPart* part;
+  const int32_t* halo;
+  const int32_t* nbr;
+  const uint16_t* moff;
+  const uint32_t* ent;
+  const float* w;      // weights in the layout's slots
+  const float* x_in;   // planar state of n_rec records
+  float* x_out;        // may equal x_in when steps > 1
+  float* out;          // flux of the last step, or nullptr
+  float* ckpt;         // states before steps 0, every, 2 every, ...; or nullptr
+  float* ex;           // 2 x n_rec exchange records (ex_chunks(D) chunks)
+  uint32_t* flag;      // steps published so far by every part
+  int* err;
+  int64_t n_rec;
+  int every, steps;
+  float tau;
+  int stall;           // test hook: part 0 leaves after publishing this many steps (-1: off)
+  int npos, off_moff, off_ent, off_w;
+  uint32_t hold_cols, tmem_cols;
+};
+// 16-byte chunks of one exchange record: three components and a tag each
+__host__ __device__ constexpr int ex_chunks(int D) { return (D + 2) / 3; }
+struct MarchSizes {
+  int32_t parts, max_pos, max_col, max_nsl;
+};
+struct MarchPlan {
+  int parts;  // 0: does not fit
+  int threads, npos, off_moff, off_ent, off_w, hold_cols, tmem_cols;
+  bool resident;  // slots and weights stay in shared memory too
+  size_t smem;
+};
+MarchPlan march_plan(const MarchSizes& z, int D, int smem_max);
+const void* march_kernel_ptr(int D, bool resident);
+cudaError_t march_fwd(const MarchArgs& a, const MarchPlan& P, int D, cudaStream_t st);
 
 cudaError_t flux_step(const FluxArgs& a, int D, cudaStream_t st);
 // read-only-cache variant (no staging); needs max_np <= 4096

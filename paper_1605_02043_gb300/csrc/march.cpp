@@ -1,0 +1,312 @@
+// march.cpp -- host side of the resident run kernels' layout (march.h).
+#include "march.h"
+
+#include <algorithm>
+#include <atomic>
+#include <thread>
+
+namespace ep {
+namespace {
+
+// A vertex's slots are walked by one lane: past this degree the lane would be
+// on its own for longer than a whole step of an ordinary part takes (about
+// 3 us), and every other lane of its slice would carry as many unused slots.
+constexpr int32_t kMarchMaxDegree = 192;
+// Vertices per part below which more parts only add neighbours to wait for.
+constexpr int64_t kMarchMinPart = 64;
+
+template <typename F>
+void parallel_for(int64_t n, int threads, F f) {
+  threads = (int)std::max<int64_t>(1, std::min<int64_t>(threads, n));
+  std::atomic<int64_t> next{0};
+  auto work = [&](int t) {
+    for (int64_t i; (i = next.fetch_add(1)) < n;) f(t, i);
+  };
+  std::vector<std::thread> pool;
+  for (int t = 1; t < threads; ++t) pool.emplace_back(work, t);
+  work(0);
+  for (auto& th : pool) th.join();
+}
+
+struct Entry {
+  int32_t o;  // position of the other endpoint
+  int32_t e;  // task
+  bool src;
+};
+
+// Columns of one slice: lane l's entries ents[lo[l] .. hi[l]) spread over K
+// columns so that the 32 lanes of a column read their other positions from
+// different shared-memory banks as far as the lists allow (a 16-byte load is
+// served 8 lanes at a time, 4 banks each; a 4-byte load 32 lanes at a time).
+// Unused slots name the lane's own position; put(column, lane, entry or null).
+template <typename Put>
+void spread_slice(std::vector<Entry>& ents, const int32_t* lo0, const int32_t* hi, int32_t p0, int32_t K, Put put) {
+  int32_t lo[32];
+  std::copy(lo0, lo0 + 32, lo);
+  for (int32_t c = 0; c < K; ++c) {
+    uint32_t used32 = 0, used8[4] = {0, 0, 0, 0};
+    auto score = [&](int l, int32_t o) {
+      return 2 * (int)((used8[l >> 3] >> (o & 7)) & 1u) + (int)((used32 >> (o & 31)) & 1u);
+    };
+    auto take = [&](int l, int32_t o) {
+      used8[l >> 3] |= 1u << (o & 7);
+      used32 |= 1u << (o & 31);
+    };
+    uint32_t forced_mask = 0;  // lanes with an entry for every remaining column go first
+    for (int l = 0; l < 32; ++l) forced_mask |= (uint32_t)(hi[l] - lo[l] == K - c) << l;
+    for (int pass = 0; pass < 2; ++pass)
+      for (int l = 0; l < 32; ++l) {
+        const bool forced = (forced_mask >> l) & 1u;
+        if ((pass == 0) != forced) continue;
+        int32_t best = -1, bs = forced ? 4 : score(l, p0 + l) + 1;
+        for (int32_t i = lo[l]; i < hi[l] && bs > 0; ++i) {
+          const int sc = score(l, ents[i].o);
+          if (sc < bs) best = i, bs = sc;
+        }
+        if (best < 0) {
+          put(c, l, (const Entry*)nullptr);
+          take(l, p0 + l);
+        } else {
+          std::swap(ents[lo[l]], ents[best]);
+          put(c, l, &ents[lo[l]]);
+          take(l, ents[lo[l]++].o);
+        }
+      }
+  }
+}
+
+// The first block that touches a vertex is not always the part most of its
+// neighbours are in, and the parts' cuts fall anywhere: passes over the
+// vertices move each one to the part that most of its neighbours are in, as
+// long as no part gets more than 3% above equal work (a step takes as long as
+// its largest part) or a third below it (which lets the few parts that hold
+// the partition's scattered remainders dissolve: they have the largest halo,
+// and it sets the shared memory).  1M-point mesh, 152 parts: mean halo 2478 ->
+// 1607 records, largest 5147 -> 2396.
+constexpr int kSmoothPasses = 2;
+void smooth_parts(const std::vector<int32_t>& ptr, const std::vector<int32_t>& nb, int32_t P, int64_t total,
+                  std::vector<int32_t>& part_of) {
+  if (P < 2) return;
+  const int64_t n = (int64_t)part_of.size();
+  std::vector<int64_t> load(P, 0);
+  for (int64_t v = 0; v < n; ++v) load[part_of[v]] += 4 + ptr[v + 1] - ptr[v];
+  const int64_t hi = total / P + total / P / 33 + 16, lo = total / P - total / P / 3 - 16;
+  for (int pass = 0; pass < kSmoothPasses; ++pass)
+    for (int64_t v = 0; v < n; ++v) {
+      const int32_t q = part_of[v], deg = ptr[v + 1] - ptr[v];
+      int32_t cand[8], cnt[8], nc = 0, mine = 0;
+      for (int32_t j = ptr[v]; j < ptr[v + 1]; ++j) {
+        const int32_t po = part_of[nb[j]];
+        if (po == q) {
+          mine += nb[j] != v;
+          continue;
+        }
+        int32_t i = 0;
+        while (i < nc && cand[i] != po) ++i;
+        if (i == nc) {
+          if (nc == 8) continue;
+          cand[nc] = po, cnt[nc++] = 0;
+        }
+        ++cnt[i];
+      }
+      int32_t best = -1, bc = mine;
+      for (int32_t i = 0; i < nc; ++i)
+        if (cnt[i] > bc && load[cand[i]] + 4 + deg <= hi) best = cand[i], bc = cnt[i];
+      if (best < 0 || load[q] - 4 - deg < lo) continue;
+      load[q] -= 4 + deg, load[best] += 4 + deg, part_of[v] = best;
+    }
+}
+
+}  // namespace
+
+// Vertices go by their cpack rank throughout (neighbours are near each other
+// in it), tasks in schedule order.
+bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLayout& L) {
+  if (s.flags & 1u) return false;
+  if (threads <= 0) threads = (int)std::max(1u, std::thread::hardware_concurrency());
+  const int64_t nd = s.nd, m = s.m, n = s.touched;
+  threads = (int)std::max<int64_t>(1, std::min<int64_t>(threads, m / 8192));  // a thread costs about 50 us
+  std::vector<int32_t> ru(m), rv(m);  // endpoint ranks in schedule order
+  constexpr int64_t kChunk = 1 << 14;
+  parallel_for((m + kChunk - 1) / kChunk, threads, [&](int, int64_t c) {
+    for (int64_t i = c * kChunk; i < std::min(m, (c + 1) * kChunk); ++i) {
+      const int32_t e = s.edge_perm[i];
+      ru[i] = s.relabel[s.src[e]];
+      rv[i] = s.relabel[s.dst[e]];
+    }
+  });
+  // incidence lists: the neighbour and the task's place in schedule order,
+  // negative (~i) where the vertex is the task's second endpoint
+  std::vector<int32_t> ptr(n + 1, 0);
+  for (int64_t i = 0; i < m; ++i) {
+    ++ptr[ru[i] + 1];
+    if (rv[i] != ru[i]) ++ptr[rv[i] + 1];
+  }
+  for (int64_t v = 0; v < n; ++v) {
+    if (ptr[v + 1] > kMarchMaxDegree) return false;
+    ptr[v + 1] += ptr[v];
+  }
+  std::vector<int32_t> nb(ptr[n]), inc(ptr[n]);
+  {
+    std::vector<int32_t> cur(ptr.begin(), ptr.end() - 1);
+    for (int64_t i = 0; i < m; ++i) {
+      const int32_t u = ru[i], v = rv[i];
+      nb[cur[u]] = v, inc[cur[u]++] = (int32_t)i;
+      if (v != u) nb[cur[v]] = u, inc[cur[v]++] = ~(int32_t)i;
+    }
+  }
+  // contiguous parts of equal slot work (a position costs about as much as
+  // four slots: its own load, its store, its share of the exchange)
+  const int32_t P = (int32_t)std::max<int64_t>(1, std::min<int64_t>(max_parts, n / kMarchMinPart));
+  const int64_t total = (int64_t)ptr[n] + 4 * n;
+  std::vector<int32_t> part_of(n, 0), rec(n, -1), order(n);  // order: the ranks part by part
+  std::vector<int64_t> cut(P + 1, 0);
+  {
+    int64_t sum = 0;
+    int32_t q = 0;
+    for (int64_t v = 0; v < n; ++v) {
+      while (q + 1 < P && sum * P >= total * (q + 1)) ++q;
+      part_of[v] = q;
+      sum += 4 + ptr[v + 1] - ptr[v];
+    }
+  }
+  smooth_parts(ptr, nb, P, total, part_of);
+  {
+    for (int64_t v = 0; v < n; ++v) ++cut[part_of[v] + 1];
+    for (int32_t q = 0; q < P; ++q) cut[q + 1] += cut[q];
+    std::vector<int64_t> at(cut.begin(), cut.end() - 1);
+    for (int64_t v = 0; v < n; ++v) order[at[part_of[v]]++] = (int32_t)v;
+  }
+  L = MarchLayout();
+  L.parts = P;
+  L.part.assign(P, MarchPart{});
+  int64_t next = 0;
+  for (int32_t q = 0; q < P; ++q) {
+    MarchPart& d = L.part[q];
+    d.lo = (int32_t)next;
+    d.own = (int32_t)(cut[q + 1] - cut[q]);
+    d.nsl = (d.own + 31) / 32;
+    d.hbase = (d.own + 3) & ~3;
+    next += d.hbase;
+  }
+  const int64_t run = next;
+  // positions: boundary vertices first, then by descending degree
+  parallel_for(P, threads, [&](int, int64_t q) {
+    MarchPart& d = L.part[q];
+    std::vector<std::pair<int32_t, int32_t>> key(d.own);  // (class and degree, place)
+    for (int32_t i = 0; i < d.own; ++i) {
+      const int32_t v = order[cut[q] + i];
+      bool bnd = false;
+      for (int32_t j = ptr[v]; j < ptr[v + 1] && !bnd; ++j) bnd = part_of[nb[j]] != q;
+      d.nb += bnd;
+      key[i] = {-((bnd ? 2 * kMarchMaxDegree : 0) + ptr[v + 1] - ptr[v]), i};
+    }
+    std::sort(key.begin(), key.end());
+    for (int32_t p = 0; p < d.own; ++p) rec[order[cut[q] + key[p].second]] = d.lo + p;
+  });
+  // halo lists, then the slots
+  struct Piece {
+    std::vector<int32_t> halo, nbr, wmap;
+    std::vector<uint16_t> moff;
+    std::vector<uint32_t> ent;
+  };
+  std::vector<Piece> piece(P);
+  L.gslot.assign(m, -1);
+  std::atomic<bool> ok{true};
+  parallel_for(P, threads, [&](int, int64_t q) {
+    MarchPart& d = L.part[q];
+    Piece& t = piece[q];
+    std::vector<int32_t> vert(d.own);
+    for (int64_t r = cut[q]; r < cut[q + 1]; ++r) vert[rec[order[r]] - d.lo] = order[r];
+    for (int32_t p = 0; p < d.nb; ++p)
+      for (int32_t j = ptr[vert[p]]; j < ptr[vert[p] + 1]; ++j) {
+        const int32_t o = nb[j];
+        if (part_of[o] != q) t.halo.push_back(rec[o]), t.nbr.push_back(part_of[o]);
+      }
+    for (auto* l : {&t.halo, &t.nbr}) {
+      std::sort(l->begin(), l->end());
+      l->erase(std::unique(l->begin(), l->end()), l->end());
+    }
+    d.nh = (int32_t)t.halo.size();
+    d.ng = (int32_t)t.nbr.size();
+    if (d.hbase + d.nh > (int32_t)kSlotPos) {
+      ok = false;
+      return;
+    }
+    t.moff.push_back(0);
+    int32_t cols = 0;
+    for (int32_t j = 0; j < d.nsl; ++j) {
+      int32_t K = 0;
+      for (int32_t p = 32 * j; p < std::min(d.own, 32 * j + 32); ++p) K = std::max(K, ptr[vert[p] + 1] - ptr[vert[p]]);
+      cols += (K + 1) / 2;
+      t.moff.push_back((uint16_t)cols);
+    }
+    if (cols > 0xffff) {
+      ok = false;
+      return;
+    }
+    d.ncol = cols;
+    t.ent.assign((size_t)cols * 32, 0);
+    t.wmap.assign((size_t)cols * 64, -1);
+    std::vector<Entry> ents;
+    for (int32_t j = 0; j < d.nsl; ++j) {
+      int32_t lo[32], hi[32];
+      ents.clear();
+      for (int l = 0; l < 32; ++l) {
+        lo[l] = (int32_t)ents.size();
+        const int32_t p = 32 * j + l;
+        if (p < d.own)
+          for (int32_t i = ptr[vert[p]]; i < ptr[vert[p] + 1]; ++i) {
+            const int32_t o = nb[i], e = s.edge_perm[inc[i] < 0 ? ~inc[i] : inc[i]];
+            const int32_t po = part_of[o] == q ? rec[o] - d.lo
+                                               : d.hbase + (int32_t)(std::lower_bound(t.halo.begin(), t.halo.end(), rec[o]) -
+                                                                     t.halo.begin());
+            ents.push_back(Entry{po, e, inc[i] >= 0});
+          }
+        hi[l] = (int32_t)ents.size();
+      }
+      const int32_t c0 = t.moff[j], K = 2 * (t.moff[j + 1] - c0);
+      spread_slice(ents, lo, hi, 32 * j, K, [&](int32_t c, int l, const Entry* x) {
+        const size_t at = (size_t)32 * (c0 + c / 2) + l;
+        const uint32_t v = x ? (uint32_t)x->o | (x->src ? kSlotSrc : 0u) : (uint32_t)(32 * j + l);
+        t.ent[at] |= v << (16 * (c & 1));
+        if (x) t.wmap[2 * at + (c & 1)] = x->e;
+      });
+    }
+    while (t.halo.size() % 4) t.halo.push_back(0);
+    while (t.moff.size() % 8) t.moff.push_back(0);
+  });
+  if (!ok) return false;
+  int64_t nh = 0, ng = 0, nq = 0, nc = 0;
+  for (int32_t q = 0; q < P; ++q) {
+    MarchPart& d = L.part[q];
+    d.h0 = (int32_t)nh, d.g0 = (int32_t)ng, d.q0 = (int32_t)nq, d.s0 = (int32_t)nc;
+    nh += (int64_t)piece[q].halo.size(), ng += d.ng, nq += (int64_t)piece[q].moff.size(), nc += d.ncol;
+    L.max_pos = std::max(L.max_pos, std::max(d.hbase + d.nh, 32 * d.nsl));
+    L.max_nh = std::max(L.max_nh, d.nh);
+    L.max_col = std::max(L.max_col, d.ncol);
+    L.max_nsl = std::max(L.max_nsl, d.nsl);
+  }
+  if (nc > INT32_MAX / 64 || run > INT32_MAX / 2) return false;
+  L.n_col = nc;
+  L.halo.resize(nh), L.nbr.resize(ng), L.moff.resize(nq), L.ent.resize(32 * nc), L.wmap.resize(64 * nc);
+  parallel_for(P, threads, [&](int, int64_t q) {
+    const MarchPart& d = L.part[q];
+    const Piece& t = piece[q];
+    std::copy(t.halo.begin(), t.halo.end(), L.halo.begin() + d.h0);
+    std::copy(t.nbr.begin(), t.nbr.end(), L.nbr.begin() + d.g0);
+    std::copy(t.moff.begin(), t.moff.end(), L.moff.begin() + d.q0);
+    std::copy(t.ent.begin(), t.ent.end(), L.ent.begin() + 32 * (int64_t)d.s0);
+    std::copy(t.wmap.begin(), t.wmap.end(), L.wmap.begin() + 64 * (int64_t)d.s0);
+    for (int64_t i = 0; i < 64 * (int64_t)d.ncol; ++i)
+      if (t.wmap[i] >= 0 && ((t.ent[i / 2] >> (16 * (i & 1))) & kSlotSrc))
+        L.gslot[t.wmap[i]] = (int32_t)(64 * (int64_t)d.s0 + i);
+  });
+  L.rec_of.resize(nd);
+  for (int64_t v = 0; v < nd; ++v)  // untouched vertices after the parts
+    L.rec_of[v] = s.relabel[v] < n ? rec[s.relabel[v]] : (int32_t)next++;
+  L.n_rec = (next + 3) & ~(int64_t)3;
+  return true;
+}
+
+}  // namespace ep

@@ -1,0 +1,58 @@
+// march.h -- layout of the resident run kernels (internal to libepcache).
+//
+// A run of several explicit steps keeps the whole mesh on the chip: the data
+// vertices, in the order of first appearance over the schedule's blocks
+// (cpack, Section 4.1, the locality the partition made), are cut into one
+// contiguous part per CUDA block.  A part owns its vertices: it computes the
+// whole flux of each of them (pull form, every task at both endpoints, as the
+// step kernels do), so nothing is accumulated across parts; what a part needs
+// from the others is the value of the neighbours it does not own (its halo).
+#pragma once
+
+#include <cstdint>
+#include <string>
+#include <vector>
+
+#include "internal.h"
+
+namespace ep {
+
+// One part.  Positions [0, own): its vertices, the boundary ones (in some
+// other part's halo) first, each class by descending degree; position p is
+// the state record lo + p.  Positions [hbase, hbase + nh): the halo, record
+// halo[h0 + j] (ascending).  Slices of 32 positions; slice j has
+// moff[q0 + j + 1] - moff[q0 + j] pair columns, each 32 lanes of two slots:
+// entry pair 32 * (s0 + column) + lane holds two 16-bit entries (position of
+// the other endpoint, kSlotSrc on the task's first endpoint) and two weights.
+// An unused slot names the lane's own position with weight 0 (its difference
+// is zero by itself).
+struct MarchPart {
+  int32_t lo, own, nb, nsl;
+  int32_t hbase, nh, h0, q0;
+  int32_t s0, ncol;  // pair columns [s0, s0 + ncol)
+  int32_t g0, ng;    // parts that share a boundary: nbr[g0 .. g0 + ng)
+  int32_t pad[4];
+};
+static_assert(sizeof(MarchPart) == 64, "MarchPart layout");
+
+struct MarchLayout {
+  int32_t parts = 0;
+  int64_t n_rec = 0;               // records per plane of a state (multiple of 4)
+  int64_t n_col = 0;               // pair columns in all (64 weights each)
+  std::vector<MarchPart> part;
+  std::vector<int32_t> rec_of;     // data vertex -> record (untouched vertices after the parts)
+  std::vector<int32_t> halo;       // records, each part's list padded to 4
+  std::vector<int32_t> nbr;        // neighbouring parts
+  std::vector<uint16_t> moff;      // pair-column offsets, each part's table padded to 8
+  std::vector<uint32_t> ent;       // entry pairs
+  std::vector<int32_t> wmap;       // weight slot (pair column, lane, which) -> task, -1 unused
+  std::vector<int32_t> gslot;      // task -> weight slot at its first endpoint
+  int32_t max_pos = 0, max_nh = 0, max_col = 0, max_nsl = 0;
+};
+
+// Builds the layout for at most `max_parts` parts.  False when the graph does
+// not suit it (a vertex of very large degree, whose slots one lane would walk
+// alone, or more positions in a part than an entry can name).
+bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLayout& out);
+
+}  // namespace ep

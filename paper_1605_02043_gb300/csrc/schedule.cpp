@@ -15,6 +15,7 @@
 //                    and the copy lists of the shared vertices; SpMV: row
 //                    lists over x records staged by owner and foreign ids.
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <thread>
 
@@ -184,7 +185,17 @@ void place_slice(HostSchedule& s, const FluxDesc& d, int32_t j, const std::vecto
   }
 }
 
-std::string flux_layout_blocks(HostSchedule& s) {
+// f(lo, hi) over contiguous ranges of [0, n), one host thread each
+template <typename F>
+void parallel_blocks(int64_t n, int threads, F f) {
+  threads = (int)std::max<int64_t>(1, std::min<int64_t>(threads, n / 16));
+  std::vector<std::thread> pool;
+  for (int t = 1; t < threads; ++t) pool.emplace_back([&f, n, t, threads] { f(n * t / threads, n * (t + 1) / threads); });
+  f(0, n / threads);
+  for (auto& th : pool) th.join();
+}
+
+std::string flux_layout_blocks(HostSchedule& s, int threads) {
   std::vector<int32_t> p, owner;
   usage(s, p, owner);
   // halo vertices of a shard (touched by other shards' tasks too) take the
@@ -193,9 +204,6 @@ std::string flux_layout_blocks(HostSchedule& s) {
   for (int32_t v : s.halo)
     if (v >= 0 && v < s.nd && p[v] == 1) p[v] = 2;
   auto align4 = [](int64_t v) { return (v + 3) & ~(int64_t)3; };
-  auto pad_to = [](auto& v, size_t mult, auto fill) {
-    while (v.size() % mult) v.push_back(fill);
-  };
   // shared ids in order of first appearance over the kernel blocks
   std::vector<int32_t> sid(s.nd, -1);
   int64_t n_sh = 0;
@@ -207,90 +215,107 @@ std::string flux_layout_blocks(HostSchedule& s) {
   s.n_sh = n_sh;
   s.fdesc.assign(s.k, FluxDesc{});
   s.rec_of.assign(s.nd, -1);
-  s.sid_list.clear();
-  s.sidx.clear();
-  s.soff.clear();
-  s.wmap.clear();
   s.gslot.assign(s.m, -1);
   s.max_nv = s.max_nslot = s.max_nsh = s.max_nsl = 0;
-  std::vector<std::vector<int32_t>> copies(n_sh);
-  std::vector<int32_t> deg(s.nd, 0), ord, pos(s.nd, -1), cls, col, ent_ptr;
-  std::vector<SlotEntry> ents;
-  int64_t next = 0;  // next free record
+  std::vector<int32_t> order(s.vert_list.size());     // positions of every block, vert_ptr offsets
+  std::vector<uint16_t> cols(s.vert_list.size() + s.k);  // slice offsets, vert_ptr[b] + b
+  std::atomic<const char*> err{nullptr};
+  // every block by itself: its positions (interior vertices, then shared
+  // ones, each by descending degree) and its slices' columns
+  parallel_blocks(s.k, threads, [&](int64_t lo, int64_t hi) {
+    std::vector<int32_t> deg(s.nd, 0), ord, cls;
+    for (int64_t b = lo; b < hi; ++b) {
+      FluxDesc& d = s.fdesc[b];
+      d.ne = (int32_t)(s.block_ptr[b + 1] - s.block_ptr[b]);
+      block_degrees(s, b, deg);
+      class_order(s, b, deg, [&](int32_t v) { return p[v] == 1; }, ord);
+      d.ni = (int32_t)ord.size();
+      class_order(s, b, deg, [&](int32_t v) { return p[v] > 1; }, cls);
+      ord.insert(ord.end(), cls.begin(), cls.end());
+      d.nv = (int32_t)ord.size();
+      std::copy(ord.begin(), ord.end(), order.begin() + s.vert_ptr[b]);
+      // slices of 32 positions; columns = largest degree in the slice
+      d.nsl = (d.nv + 31) / 32;
+      uint16_t* off = &cols[s.vert_ptr[b] + b];
+      int32_t c = off[0] = 0;
+      for (int32_t j = 0; j < d.nsl; ++j) {
+        int32_t K = 0;
+        for (int32_t q = 32 * j; q < std::min(d.nv, 32 * j + 32); ++q) K = std::max(K, deg[ord[q]]);
+        c += K;
+        if (c > 0xffff) {
+          err = "block has too many incidence entries";
+          break;
+        }
+        off[j + 1] = (uint16_t)c;
+      }
+      if (d.nv > (int32_t)kSlotPos) err = "block touches too many vertices";
+      d.nslot = 32 * c;
+      for (int64_t i = s.vert_ptr[b]; i < s.vert_ptr[b + 1]; ++i) deg[s.vert_list[i]] = 0;
+      if (err.load()) return;
+    }
+  });
+  if (err.load()) return err.load();
+  // where every block's segments start (16-byte boundaries)
+  int64_t next = 0, n_sid = 0, n_off = 0, n_slot = 0;
   for (int64_t b = 0; b < s.k; ++b) {
     FluxDesc& d = s.fdesc[b];
-    d.ne = (int32_t)(s.block_ptr[b + 1] - s.block_ptr[b]);
-    block_degrees(s, b, deg);
-    // positions: interior vertices, then shared ones, each by descending degree
-    class_order(s, b, deg, [&](int32_t v) { return p[v] == 1; }, ord);
-    d.ni = (int32_t)ord.size();
-    class_order(s, b, deg, [&](int32_t v) { return p[v] > 1; }, cls);
-    ord.insert(ord.end(), cls.begin(), cls.end());
-    d.nv = (int32_t)ord.size();
-    if (d.nv > (int32_t)kSlotPos) return "block touches too many vertices";
     next = align4(next);
     d.rec_lo = (int32_t)next;
-    for (int32_t q = 0; q < d.nv; ++q) {
-      const int32_t v = ord[q];
-      pos[v] = q;
-      const int32_t r = (int32_t)(next + q);
-      if (owner[v] == b) s.rec_of[v] = r;  // first copy of a shared vertex
-      if (q >= d.ni) copies[sid[v]].push_back(r);
-    }
+    d.h0 = (int32_t)n_sid;
+    d.q0 = (int32_t)n_off;
+    d.s0 = (int32_t)n_slot;  // a multiple of 32
     next += d.nv;
-    // shared ids of positions [ni, nv); the first copy of each shared vertex
-    // (in its first block) carries kSidFirst
-    pad_to(s.sid_list, 4, (int32_t)0);
-    d.h0 = (int32_t)s.sid_list.size();
-    for (int32_t q = d.ni; q < d.nv; ++q)
-      s.sid_list.push_back(sid[ord[q]] | (owner[ord[q]] == b ? kSidFirst : 0));
-    pad_to(s.sid_list, 4, (int32_t)0);
-    // slices of 32 positions; columns = largest degree in the slice
-    d.nsl = (d.nv + 31) / 32;
-    pad_to(s.soff, 8, (uint16_t)0);
-    d.q0 = (int32_t)s.soff.size();
-    int32_t cols = 0;
-    s.soff.push_back(0);
-    for (int32_t j = 0; j < d.nsl; ++j) {
-      int32_t K = 0;
-      for (int32_t q = 32 * j; q < std::min(d.nv, 32 * j + 32); ++q) K = std::max(K, deg[ord[q]]);
-      cols += K;
-      if (cols > 0xffff) return "block has too many incidence entries";
-      s.soff.push_back((uint16_t)cols);
-    }
-    pad_to(s.soff, 8, (uint16_t)0);
-    d.s0 = (int32_t)s.sidx.size();  // a multiple of 32
-    d.nslot = 32 * cols;
-    s.sidx.resize(s.sidx.size() + d.nslot, 0);
-    s.wmap.resize(s.sidx.size(), -1);
-    // the entries of every position: each task at both endpoints (a self
-    // loop once), the source side flagged
-    ent_ptr.assign(d.nv + 1, 0);
-    for (int64_t i = s.block_ptr[b]; i < s.block_ptr[b + 1]; ++i) {
-      int32_t u, v;
-      task_ends(s, s.edge_perm[i], u, v);
-      ++ent_ptr[pos[u] + 1];
-      if (v != u) ++ent_ptr[pos[v] + 1];
-    }
-    for (int32_t q = 0; q < d.nv; ++q) ent_ptr[q + 1] += ent_ptr[q];
-    ents.resize(ent_ptr[d.nv]);
-    col.assign(ent_ptr.begin(), ent_ptr.end() - 1);
-    for (int64_t i = s.block_ptr[b]; i < s.block_ptr[b + 1]; ++i) {
-      const int32_t e = s.edge_perm[i];
-      int32_t u, v;
-      task_ends(s, e, u, v);
-      const int32_t pu = pos[u], pv = pos[v];
-      ents[col[pu]++] = SlotEntry{pv, e, true};
-      if (v != u) ents[col[pv]++] = SlotEntry{pu, e, false};
-    }
-    for (int32_t j = 0; j < d.nsl; ++j) place_slice(s, d, j, ent_ptr, ents);
-    for (int64_t i = s.vert_ptr[b]; i < s.vert_ptr[b + 1]; ++i) deg[s.vert_list[i]] = 0;
+    n_sid += align4(d.nv - d.ni);
+    n_off += (d.nsl + 1 + 7) & ~7;
+    n_slot += d.nslot;
     s.max_nv = std::max(s.max_nv, d.nv);
     s.max_nslot = std::max(s.max_nslot, d.nslot);
     s.max_nsh = std::max(s.max_nsh, d.nv - d.ni);
     s.max_nsl = std::max(s.max_nsl, d.nsl);
-    if (s.sidx.size() >= (size_t)INT32_MAX || next >= INT32_MAX / 2) return "schedule too large";
+    if (n_slot >= INT32_MAX || next >= INT32_MAX / 2) return "schedule too large";
   }
+  s.sid_list.assign(n_sid, 0);
+  s.soff.assign(n_off, 0);
+  s.sidx.assign(n_slot, 0);
+  s.wmap.assign(n_slot, -1);
+  parallel_blocks(s.k, threads, [&](int64_t blo, int64_t bhi) {
+    std::vector<int32_t> pos(s.nd), ent_ptr, col;
+    std::vector<SlotEntry> ents;
+    for (int64_t b = blo; b < bhi; ++b) {
+      const FluxDesc& d = s.fdesc[b];
+      const int32_t* ord = &order[s.vert_ptr[b]];
+      // shared ids of positions [ni, nv); the first copy of each shared vertex
+      // (in its first block) carries kSidFirst and is the vertex's record
+      for (int32_t q = 0; q < d.nv; ++q) {
+        const int32_t v = ord[q];
+        pos[v] = q;
+        if (owner[v] == b) s.rec_of[v] = d.rec_lo + q;
+        if (q >= d.ni) s.sid_list[d.h0 + q - d.ni] = sid[v] | (owner[v] == b ? kSidFirst : 0);
+      }
+      std::copy_n(&cols[s.vert_ptr[b] + b], d.nsl + 1, s.soff.begin() + d.q0);
+      // the entries of every position: each task at both endpoints (a self
+      // loop once), the source side flagged
+      ent_ptr.assign(d.nv + 1, 0);
+      for (int64_t i = s.block_ptr[b]; i < s.block_ptr[b + 1]; ++i) {
+        int32_t u, v;
+        task_ends(s, s.edge_perm[i], u, v);
+        ++ent_ptr[pos[u] + 1];
+        if (v != u) ++ent_ptr[pos[v] + 1];
+      }
+      for (int32_t q = 0; q < d.nv; ++q) ent_ptr[q + 1] += ent_ptr[q];
+      ents.resize(ent_ptr[d.nv]);
+      col.assign(ent_ptr.begin(), ent_ptr.end() - 1);
+      for (int64_t i = s.block_ptr[b]; i < s.block_ptr[b + 1]; ++i) {
+        const int32_t e = s.edge_perm[i];
+        int32_t u, v;
+        task_ends(s, e, u, v);
+        const int32_t pu = pos[u], pv = pos[v];
+        ents[col[pu]++] = SlotEntry{pv, e, true};
+        if (v != u) ents[col[pv]++] = SlotEntry{pu, e, false};
+      }
+      for (int32_t j = 0; j < d.nsl; ++j) place_slice(s, d, j, ent_ptr, ents);
+    }
+  });
   s.n_run = align4(next);
   next = s.n_run;
   for (int64_t v = 0; v < s.nd; ++v)
@@ -308,12 +333,14 @@ std::string flux_layout_blocks(HostSchedule& s) {
       s.fold_sid.push_back(s.sid_list[d.h0 + q - d.ni]);
     }
   }
+  // the copies of every shared vertex, in block order (fold_rec is)
   s.cptr.assign(n_sh + 1, 0);
-  s.crec.clear();
-  s.crec.reserve(s.vert_ptr.back());
-  for (int64_t h = 0; h < n_sh; ++h) {
-    s.crec.insert(s.crec.end(), copies[h].begin(), copies[h].end());
-    s.cptr[h + 1] = (int32_t)s.crec.size();
+  for (int32_t h : s.fold_sid) ++s.cptr[(h & kSidMask) + 1];
+  for (int64_t h = 0; h < n_sh; ++h) s.cptr[h + 1] += s.cptr[h];
+  s.crec.resize(s.fold_rec.size());
+  {
+    std::vector<int32_t> cur(s.cptr.begin(), s.cptr.end() - 1);
+    for (size_t i = 0; i < s.fold_sid.size(); ++i) s.crec[cur[s.fold_sid[i] & kSidMask]++] = s.fold_rec[i];
   }
   for (int64_t v = 0; v < s.nd; ++v)  // every copy of a shared vertex maps back to it
     if (sid[v] >= 0)
@@ -390,7 +417,7 @@ bool cut_large_blocks(const HostSchedule& s, Pieces& out) {
   return true;
 }
 
-std::string flux_layout(HostSchedule& s) {
+std::string flux_layout(HostSchedule& s, int threads) {
   Pieces pc;
   const bool cut = cut_large_blocks(s, pc);
   if (cut) {
@@ -399,7 +426,7 @@ std::string flux_layout(HostSchedule& s) {
     s.vert_ptr.swap(pc.vert_ptr);
     s.vert_list.swap(pc.vert_list);
   }
-  std::string err = flux_layout_blocks(s);
+  std::string err = flux_layout_blocks(s, threads);
   if (cut) {  // the schedule itself is the uncut one
     std::swap(s.k, pc.k);
     s.block_ptr.swap(pc.block_ptr);
@@ -533,9 +560,11 @@ std::string spmv_layout(HostSchedule& s) {
 
 }  // namespace
 
-std::string rebuild_flux_layout(HostSchedule& s) { return flux_layout(s); }
+std::string rebuild_flux_layout(HostSchedule& s) {
+  return flux_layout(s, (int)std::max(1u, std::thread::hardware_concurrency()));
+}
 
-std::string build_schedule(HostSchedule& s, int threads) {
+std::string build_schedule(HostSchedule& s, int threads, const std::function<void()>& ordered) {
   if (threads <= 0) threads = (int)std::max(1u, std::thread::hardware_concurrency());
   threads = (int)std::max<int64_t>(1, std::min<int64_t>(threads, s.k));
   // reconstruction (Definition 4): counting sort by block keeps ascending ids
@@ -553,7 +582,8 @@ std::string build_schedule(HostSchedule& s, int threads) {
   }
   vertex_lists(s, threads);
   cpack(s);
-  return (s.flags & 1u) ? spmv_layout(s) : flux_layout(s);
+  if (ordered) ordered();
+  return (s.flags & 1u) ? spmv_layout(s) : flux_layout(s, threads);
 }
 
 }  // namespace ep

@@ -1,0 +1,129 @@
+"""Resident runs of several steps (march.cu) against the oracle (GPU only).
+
+Sizes where the layout has its edges: one part, parts of a few vertices, the
+last slice partly filled, a halo larger than the part (default order), slots
+kept in shared memory and slots read from the L2, every state width, isolated
+vertices, self loops and repeated pairs.  Tolerances: parity.py.
+"""
+import numpy as np
+import pytest
+
+import oracle as O
+import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import paper_1605_02043_gb300 as E  # noqa: E402
+from paper_1605_02043_gb300._lib import EpError  # noqa: E402
+from parity import check_field, check_state  # noqa: E402
+
+
+def cuda(a):
+    return torch.from_numpy(np.ascontiguousarray(a, np.float32)).cuda()
+
+
+def run_against_oracle(S, src, dst, n, D, steps, seed, tau=1e-2):
+    x0, w = W.flux_state(n, D, seed), W.flux_weights(src.size, seed)
+    x = cuda(x0)
+    out = torch.full_like(x, 7.0)
+    S.timing(2)
+    S.run(x, cuda(w), out, steps=steps, tau=tau)
+    launches = S.timing_read(E.T_EDGE_FWD)[1]
+    S.timing(0)
+    assert S.check_errors() == 0
+    xT, fT = O.flux_steps(src, dst, x0, w, steps, tau)
+    check_field(out, fT, "out")
+    check_state(x, xT, x0, steps, "x")
+    return launches
+
+
+@pytest.mark.parametrize("n,C,D,steps,default_order", [
+    (40, 16, 5, 3, False), (129, 64, 1, 2, False), (300, 64, 5, 9, True), (1025, 256, 3, 4, False),
+    (4096, 256, 2, 5, False), (4096, 1000, 4, 5, True), (9999, 512, 6, 3, False), (9999, 512, 7, 4, True),
+    (20011, 512, 8, 3, False), (50021, 1024, 5, 6, False), (50021, 512, 5, 2, True), (200003, 512, 1, 3, False),
+])
+def test_runs_match_oracle(n, C, D, steps, default_order):
+    src, dst = W.knn_mesh(n, 4, 1)
+    S = E.Schedule.partition(src, dst, n, C, default_order=default_order)
+    assert run_against_oracle(S, src, dst, n, D, steps, n) == 1  # one launch for the whole run
+    # again on the same schedule: the step counters go on from where they stand
+    assert run_against_oracle(S, src, dst, n, D, steps + 1, n + 1) == 1
+
+
+def test_slots_in_shared_memory_and_from_l2():
+    # widths from 1 to 8 on one mesh: with D = 1 a part's slots fit beside its
+    # state, with D = 8 they do not
+    n = 320000
+    src, dst = W.knn_mesh(n, 4, 2)
+    S = E.Schedule.partition(src, dst, n, 1024)
+    for D in (1, 5, 8):
+        assert run_against_oracle(S, src, dst, n, D, 2, D) == 1
+
+
+def test_loops_pairs_and_isolated_vertices():
+    rng = np.random.default_rng(4)
+    n = 3000
+    src = rng.integers(0, 2000, 7777).astype(np.int32)
+    dst = ((src + rng.integers(1, 30, 7777)) % 2000).astype(np.int32)
+    src[:50] = dst[:50]
+    src[50:100], dst[50:100] = src[100:150], dst[100:150]
+    S = E.Schedule.partition(src, dst, n, 100)
+    assert run_against_oracle(S, src, dst, n, 5, 4, 3) == 1
+
+
+def test_hub_takes_the_step_kernels():
+    # one vertex in every task: its slots would be one lane's
+    n = 2000
+    src, dst = np.zeros(n - 1, np.int32), np.arange(1, n, dtype=np.int32)
+    S = E.Schedule.partition(src, dst, n, 128)
+    assert run_against_oracle(S, src, dst, n, 3, 3, 3, tau=1e-4) == 3
+
+
+def test_two_streams_and_graph_replay():
+    """Runs of two schedules on two streams, then captured and replayed."""
+    n = 30011
+    src, dst = W.knn_mesh(n, 4, 5)
+    Ss = [E.Schedule.partition(src, dst, n, C) for C in (256, 512)]
+    x0, w = W.flux_state(n, 5, 1), W.flux_weights(src.size, 1)
+    xT, _ = O.flux_steps(src, dst, x0, w, 20, 1e-3)
+    streams = [torch.cuda.Stream() for _ in Ss]
+    wd, xs = cuda(w), [cuda(x0) for _ in Ss]
+    torch.cuda.synchronize()
+    for _ in range(2):
+        for S, st, x in zip(Ss, streams, xs):
+            with torch.cuda.stream(st):
+                S.run(x, wd, None, steps=10, tau=1e-3)
+    torch.cuda.synchronize()
+    for S, x in zip(Ss, xs):
+        assert S.check_errors() == 0
+        check_state(x, xT, x0, 20, "x")
+    x = cuda(x0)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        Ss[0].run(x, wd, None, steps=5, tau=1e-3)
+    for _ in range(4):
+        g.replay()
+    torch.cuda.synchronize()
+    assert Ss[0].check_errors() == 0
+    check_state(x, xT, x0, 20, "x (graph)")
+
+
+def test_wait_for_a_neighbour_expires_then_recovers():
+    """Part 0 leaves after its first published step (ep_debug_stall): the others' bounded
+    wait runs out, the error is reported, and the next run is correct."""
+    n = 30011
+    src, dst = W.knn_mesh(n, 4, 5)
+    S = E.Schedule.partition(src, dst, n, 512)
+    x0, w = W.flux_state(n, 5, 2), W.flux_weights(src.size, 2)
+    S.debug_stall(1)
+    S.run(cuda(x0), cuda(w), None, steps=4, tau=1e-3)
+    with pytest.raises(EpError) as ei:
+        S.check_errors()
+    assert ei.value.code == -4
+    S.debug_stall(-1)
+    assert run_against_oracle(S, src, dst, n, 5, 4, 2, tau=1e-3) == 1
