@@ -346,6 +346,37 @@ int ep_adjoint_step_pending(ep_schedule *s, int32_t D, const float *x_lay, const
 int ep_adjoint_finish(ep_schedule *s, int32_t D, float *lam, float tau, void *stream);
 
 /*
+ * No counterpart in the paper: a run and its reverse sweep for a training
+ * step, each one launch that keeps the mesh on the chip (see ep_run), in a
+ * layout of their own.  ep_grad_sizes gives the floats of a state buffer and
+ * of a weight buffer in that layout, or 0 and 0 where such runs do not apply
+ * (as for ep_run; the sweep holds state and cotangent, so about half as many
+ * vertices fit).  All layout buffers are 16-byte aligned device memory.
+ *   ep_grad_state_in / _out      x (float[D][n]) <-> x_lay
+ *   ep_grad_weights_in           w_lay <- w (float[m])
+ *   ep_grad_weights_out          grad_w (float[m]) <- gw_lay, overwritten
+ *   ep_grad_forward              xT_lay <- `steps` explicit steps from x_lay
+ *                                (may be the same buffer when steps > 1); ckpt
+ *                                receives the states before steps 0, every,
+ *                                2 every, ... (ceil(steps / every) states)
+ *   ep_grad_backward             lam_out <- dL/dx_0 from lam_in = dL/dx_T (may
+ *                                be the same buffer when steps > 1), gw_lay <-
+ *                                dL/dw, from ep_grad_forward's ckpt; hist:
+ *                                scratch of every - 1 states (may be NULL when
+ *                                every <= 2)
+ */
+int ep_grad_sizes(ep_schedule *s, int32_t D, int64_t *state_floats, int64_t *weight_floats);
+int ep_grad_state_in(ep_schedule *s, int32_t D, const float *x, float *x_lay, void *stream);
+int ep_grad_state_out(ep_schedule *s, int32_t D, const float *x_lay, float *x, void *stream);
+int ep_grad_weights_in(ep_schedule *s, int32_t D, const float *w, float *w_lay, void *stream);
+int ep_grad_weights_out(ep_schedule *s, int32_t D, const float *gw_lay, float *grad_w, void *stream);
+int ep_grad_forward(ep_schedule *s, int32_t D, const float *x_lay, float *xT_lay, const float *w_lay,
+                    float *ckpt, int32_t steps, int32_t every, float tau, void *stream);
+int ep_grad_backward(ep_schedule *s, int32_t D, const float *ckpt, float *hist, const float *w_lay,
+                     const float *lam_in, float *lam_out, float *gw_lay, int32_t steps,
+                     int32_t every, float tau, void *stream);
+
+/*
  * No counterpart in the paper (a build-side pattern of this library): the
  * union of balanced edge partitions of disjoint affinity graphs (Definition 1)
  * is an edge partition of their union, and its cost (Eq. 1) is the sum of the

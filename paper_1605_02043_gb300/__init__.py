@@ -291,6 +291,38 @@ class Schedule:
         """Brings the shared copies of a pending state up to date (ep_finish)."""
         check(lib().ep_finish(self._h, D, _vp(x_lay), tau, _stream(stream)))
 
+    # ------------------------------------------ runs kept on the chip, with gradient
+    def grad_sizes(self, D: int):
+        """Floats of a state and of a weight buffer of the grad_* calls (ep_grad_sizes);
+        (0, 0) where such runs do not apply."""
+        a, b = ctypes.c_int64(), ctypes.c_int64()
+        check(lib().ep_grad_sizes(self._h, D, ctypes.byref(a), ctypes.byref(b)))
+        return a.value, b.value
+
+    def grad_state_in(self, x, x_lay, stream=None):
+        check(lib().ep_grad_state_in(self._h, int(x.shape[0]), _vp(x), _vp(x_lay), _stream(stream)))
+
+    def grad_state_out(self, x_lay, x, stream=None):
+        check(lib().ep_grad_state_out(self._h, int(x.shape[0]), _vp(x_lay), _vp(x), _stream(stream)))
+
+    def grad_weights_in(self, D: int, w, w_lay, stream=None):
+        check(lib().ep_grad_weights_in(self._h, D, _vp(w), _vp(w_lay), _stream(stream)))
+
+    def grad_weights_out(self, D: int, gw_lay, grad_w, stream=None):
+        check(lib().ep_grad_weights_out(self._h, D, _vp(gw_lay), _vp(grad_w), _stream(stream)))
+
+    def grad_forward(self, D: int, x_lay, xT_lay, w_lay, ckpt, steps: int, every: int, tau: float = 1e-3,
+                     stream=None):
+        """A run in one launch that keeps its checkpoints (ep_grad_forward)."""
+        check(lib().ep_grad_forward(self._h, D, _vp(x_lay), _vp(xT_lay), _vp(w_lay), _vp(ckpt), steps, every,
+                                    tau, _stream(stream)))
+
+    def grad_backward(self, D: int, ckpt, hist, w_lay, lam_in, lam_out, gw_lay, steps: int, every: int,
+                      tau: float = 1e-3, stream=None):
+        """Its reverse sweep in one launch (ep_grad_backward)."""
+        check(lib().ep_grad_backward(self._h, D, _vp(ckpt), _vp(hist), _vp(w_lay), _vp(lam_in), _vp(lam_out),
+                                     _vp(gw_lay), steps, every, tau, _stream(stream)))
+
     # ------------------------------------------------------------ shard halo
     def set_halo(self, ids):
         """Declares the data vertices other shards touch too (ep_set_halo); rebuilds

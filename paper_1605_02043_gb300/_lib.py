@@ -48,6 +48,13 @@ SIGNATURES = {
     "ep_adjoint_step": (ctypes.c_int, [P, I32, P, P, P, P, F32, P]),
     "ep_adjoint_step_pending": (ctypes.c_int, [P, I32, P, P, P, P, F32, P]),
     "ep_adjoint_finish": (ctypes.c_int, [P, I32, P, F32, P]),
+    "ep_grad_sizes": (ctypes.c_int, [P, I32, P, P]),
+    "ep_grad_state_in": (ctypes.c_int, [P, I32, P, P, P]),
+    "ep_grad_state_out": (ctypes.c_int, [P, I32, P, P, P]),
+    "ep_grad_weights_in": (ctypes.c_int, [P, I32, P, P, P]),
+    "ep_grad_weights_out": (ctypes.c_int, [P, I32, P, P, P]),
+    "ep_grad_forward": (ctypes.c_int, [P, I32, P, P, P, P, I32, I32, F32, P]),
+    "ep_grad_backward": (ctypes.c_int, [P, I32, P, P, P, P, P, P, I32, I32, F32, P]),
     "ep_spmv_x_in": (ctypes.c_int, [P, P, P, P]),
     "ep_spmv_y_out": (ctypes.c_int, [P, P, P, P]),
     "ep_spmv": (ctypes.c_int, [P, P, P, P, P]),

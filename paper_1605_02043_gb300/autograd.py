@@ -7,7 +7,9 @@ forward kernel, then runs the hand-written adjoint kernel (same schedule, same
 access pattern) step by step back to the checkpoint.  Gradients flow to x0 and
 to the task weights w.  Steps leave the copies of shared vertices pending
 (one launch per step); a state is finished where it is stored or read whole
-(checkpoints, recomputed states, the results).
+(checkpoints, recomputed states, the results).  Where the mesh fits the chip
+(Schedule.grad_sizes) the forward run and the whole reverse sweep are one launch
+each instead, with the same checkpoints and the same recomputation.
 """
 from __future__ import annotations
 
@@ -22,8 +24,23 @@ class FluxSteps(torch.autograd.Function):
         D = int(x0.shape[0])
         x0 = x0.contiguous()
         w = w.contiguous()
-        xl = torch.empty(sched.layout_floats(D), device=x0.device, dtype=torch.float32)
-        wl = torch.empty(sched.weights_floats(), device=x0.device, dtype=torch.float32)
+        f32 = dict(device=x0.device, dtype=torch.float32)
+        ctx.sched, ctx.steps, ctx.tau, ctx.every, ctx.D = sched, steps, tau, every, D
+        ns, nw = sched.grad_sizes(D) if steps > 0 and every > 0 else (0, 0)
+        ctx.on_chip = ns > 0
+        if ctx.on_chip:
+            xl, wl = torch.empty(ns, **f32), torch.empty(nw, **f32)
+            xo = xl if steps > 1 else torch.empty_like(xl)
+            ckpt = torch.empty(-(-steps // every), ns, **f32)
+            sched.grad_state_in(x0, xl)
+            sched.grad_weights_in(D, w, wl)
+            sched.grad_forward(D, xl, xo, wl, ckpt, steps, every, tau)
+            xT = torch.empty_like(x0)
+            sched.grad_state_out(xo, xT)
+            ctx.save_for_backward(wl, ckpt)
+            return xT
+        xl = torch.empty(sched.layout_floats(D), **f32)
+        wl = torch.empty(sched.weights_floats(), **f32)
         sched.layout_in(x0, xl)
         sched.weights_in(w, wl)
         ckpts = []
@@ -36,7 +53,6 @@ class FluxSteps(torch.autograd.Function):
         sched.finish(D, xl, tau)
         xT = torch.empty_like(x0)
         sched.layout_out(xl, xT)
-        ctx.sched, ctx.steps, ctx.tau, ctx.every, ctx.D = sched, steps, tau, every, D
         ctx.save_for_backward(wl, *ckpts)
         return xT
 
@@ -45,6 +61,21 @@ class FluxSteps(torch.autograd.Function):
         sched, steps, tau, every, D = ctx.sched, ctx.steps, ctx.tau, ctx.every, ctx.D
         wl, *ckpts = ctx.saved_tensors
         g = g.contiguous()
+        if ctx.on_chip:
+            ckpt = ckpts[0]
+            ns = ckpt.shape[1]
+            # images between two checkpoints: every - 1 at most, and no more than the run has
+            hist = torch.empty(max(min(every, steps) - 2, 0), ns, device=g.device, dtype=torch.float32)
+            lam = torch.empty(ns, device=g.device, dtype=torch.float32)
+            lo = lam if steps > 1 else torch.empty_like(lam)
+            gwl = torch.empty_like(wl)
+            sched.grad_state_in(g, lam)
+            sched.grad_backward(D, ckpt, hist if hist.numel() else None, wl, lam, lo, gwl, steps, every, tau)
+            dx0 = torch.empty_like(g)
+            sched.grad_state_out(lo, dx0)
+            dw = torch.empty(sched.m, device=g.device, dtype=torch.float32)
+            sched.grad_weights_out(D, gwl, dw)
+            return dx0, dw, None, None, None, None
         lam = torch.empty_like(ckpts[0])
         sched.layout_in(g, lam)
         gwl = torch.zeros_like(wl)
@@ -84,7 +115,11 @@ class FluxRunner:
     def __init__(self, sched: Schedule, D: int, steps: int, tau: float = 1e-3, every: int = 5,
                  device="cuda"):
         self.s, self.D, self.steps, self.tau, self.every = sched, D, steps, tau, every
-        nl, nw = sched.layout_floats(D), sched.weights_floats()
+        # runs kept on the chip where they apply, else one launch per step
+        ns, nw = sched.grad_sizes(D) if steps > 1 and every > 0 else (0, 0)
+        self.on_chip = ns > 0
+        nl = ns if self.on_chip else sched.layout_floats(D)
+        nw = nw if self.on_chip else sched.weights_floats()
         f32 = dict(device=device, dtype=torch.float32)
         self.x0l = torch.zeros(nl, **f32)
         self.gl = torch.zeros(nl, **f32)
@@ -93,16 +128,24 @@ class FluxRunner:
         self.wl = torch.zeros(nw, **f32)
         self.gwl = torch.zeros(nw, **f32)
         nseg = (steps + every - 1) // every
-        self.ckpt = [torch.zeros(nl, **f32) for _ in range(nseg)]
-        self.hist = [torch.zeros(nl, **f32) for _ in range(max(every - 1, 0))]
+        self.ckpt = torch.zeros(nseg, nl, **f32)
+        self.hist = torch.zeros(max(every - 1, 0), nl, **f32)
 
     def load(self, x0, w, g):
+        if self.on_chip:
+            self.s.grad_state_in(x0.contiguous(), self.x0l)
+            self.s.grad_weights_in(self.D, w.contiguous(), self.wl)
+            self.s.grad_state_in(g.contiguous(), self.gl)
+            return
         self.s.layout_in(x0.contiguous(), self.x0l)
         self.s.weights_in(w.contiguous(), self.wl)
         self.s.layout_in(g.contiguous(), self.gl)
 
     def forward(self):
         s, D, tau = self.s, self.D, self.tau
+        if self.on_chip:
+            s.grad_forward(D, self.x0l, self.xl, self.wl, self.ckpt, self.steps, self.every, tau)
+            return
         self.xl.copy_(self.x0l)
         for t in range(self.steps):
             if t % self.every == 0:
@@ -114,11 +157,15 @@ class FluxRunner:
 
     def backward(self):
         s, D, tau = self.s, self.D, self.tau
+        if self.on_chip:
+            s.grad_backward(D, self.ckpt, self.hist if self.hist.numel() else None, self.wl, self.gl, self.lam,
+                            self.gwl, self.steps, self.every, tau)
+            return
         self.lam.copy_(self.gl)
         self.gwl.zero_()
         for seg in range(len(self.ckpt) - 1, -1, -1):
             T = min(self.every, self.steps - seg * self.every)
-            states = [self.ckpt[seg]] + self.hist[: T - 1]
+            states = [self.ckpt[seg], *self.hist[: T - 1]]
             for t in range(T - 1):
                 s.step(D, states[t], states[t + 1], self.wl, None, tau)
             for t in range(T - 1, -1, -1):
@@ -130,10 +177,16 @@ class FluxRunner:
         self.backward()
 
     def results(self, x_like, m: int):
-        xT = torch.empty_like(x_like)
-        self.s.layout_out(self.xl, xT)
-        dx0 = torch.empty_like(x_like)
-        self.s.layout_out(self.lam, dx0)
+        s = self.s
+        xT, dx0 = torch.empty_like(x_like), torch.empty_like(x_like)
+        if self.on_chip:
+            dw = torch.empty(m, device=x_like.device, dtype=torch.float32)
+            s.grad_state_out(self.xl, xT)
+            s.grad_state_out(self.lam, dx0)
+            s.grad_weights_out(self.D, self.gwl, dw)
+            return xT, dx0, dw
+        s.layout_out(self.xl, xT)
+        s.layout_out(self.lam, dx0)
         dw = torch.zeros(m, device=x_like.device, dtype=torch.float32)
-        self.s.weights_out_add(self.gwl, dw)
+        s.weights_out_add(self.gwl, dw)
         return xT, dx0, dw

@@ -175,10 +175,10 @@ struct ep_schedule {
   bool march = false, march_up = false;
   bool march_dirty = true;  // the exchange records and the parts' counts need clearing
   int32_t march_D = 0;      // state width they were last used with
-  DBuf d_mpart, d_mhalo, d_mnbr, d_moff, d_ment, d_mwmap, d_mrec;
+  DBuf d_mpart, d_mhalo, d_mtab, d_ment, d_mwmap, d_mrec, d_mgslot;
   DBuf ws_mx, ws_mw, ws_mout, ws_mex, ws_mflag;
-  ep::dev::MarchPlan mplans[EP_MAX_D + 1];
-  bool mplan_set[EP_MAX_D + 1] = {};
+  ep::dev::MarchPlan mplans[EP_MAX_D + 1][2];  // [0] forward run, [1] reverse sweep
+  bool mplan_set[EP_MAX_D + 1][2] = {};
 };
 
 namespace {
@@ -428,49 +428,55 @@ int ensure_ctl(ep_schedule* s, cudaStream_t st) {
   return EP_OK;
 }
 
-// Plan, device copy and workspace of resident runs at state width D; P.parts
-// stays 0 where a run cannot be resident: the graph does not suit the layout,
-// a part does not fit an SM, the GPU has fewer SMs than parts, or another
-// kernel organisation was asked for (one block per kernel block, read-only
-// cache, a shard's halo).
-int ensure_march(ep_schedule* s, int32_t D, ep::dev::MarchPlan& P, cudaStream_t st) {
+// Launch plan of a resident run (grad: of its reverse sweep) at state width D;
+// P.parts stays 0 where it cannot be resident: the graph does not suit the
+// layout, a part does not fit an SM, or the GPU has fewer SMs than parts.
+int march_plan_of(ep_schedule* s, int32_t D, bool grad, ep::dev::MarchPlan& P) {
   P.parts = 0;
-  if (!s->march || s->stages == 0 || s->cache != EP_CACHE_SMEM || !s->h.halo.empty()) return EP_OK;
+  if (!s->march) return EP_OK;
   const ep::MarchLayout& L = s->ml;
-  if (!s->mplan_set[D]) {
+  ep::dev::MarchPlan& Q = s->mplans[D][grad];
+  if (!s->mplan_set[D][grad]) {
     int dev = 0, optin = 0, sms = 0, coop = 0;
     CU(cudaGetDevice(&dev));
     CU(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     CU(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
-    ep::dev::MarchPlan& Q = s->mplans[D];
-    const int smem_max = optin - 512;  // less the kernel's static shared memory
-    Q = ep::dev::march_plan({L.parts, L.max_pos, L.max_col, L.max_nsl}, D, smem_max);
+    const int smem_max = optin - 512;  // less the kernels' static shared memory
+    Q = ep::dev::march_plan({L.parts, L.warps, L.max_pos, L.max_col, L.max_nsl}, D, grad, smem_max);
     if (!coop || sms < L.parts) Q.parts = 0;
     if (Q.parts) {
-      const void* k = ep::dev::march_kernel_ptr(D, Q.resident);
+      const void* k = ep::dev::march_kernel_ptr(D, grad, Q.resident);
       CU(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
       int per_sm = 0;
       CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, Q.threads, Q.smem));
       if (per_sm < 1) Q.parts = 0;
     }
-    s->mplan_set[D] = true;
+    s->mplan_set[D][grad] = true;
   }
-  P = s->mplans[D];
-  if (!P.parts) return EP_OK;
+  P = Q;
+  return EP_OK;
+}
+
+// Whether runs may be resident under the schedule's settings (another kernel
+// organisation, the read-only cache and a shard's halo keep the step kernels).
+bool march_wanted(const ep_schedule* s) {
+  return s->march && s->stages != 0 && s->cache == EP_CACHE_SMEM && s->h.halo.empty();
+}
+
+// Device copy of the layout, and the exchange records.
+int ensure_march(ep_schedule* s, int32_t D, cudaStream_t st) {
+  const ep::MarchLayout& L = s->ml;
   if (!s->march_up) {
     CU(upload(s->d_mpart, L.part));
     CU(upload(s->d_mhalo, L.halo));
-    CU(upload(s->d_mnbr, L.nbr));
-    CU(upload(s->d_moff, L.moff));
+    CU(upload(s->d_mtab, L.tab));
     CU(upload(s->d_ment, L.ent));
     CU(upload(s->d_mwmap, L.wmap));
     CU(upload(s->d_mrec, L.rec_of));
     s->march_up = true;
     s->march_dirty = true;
   }
-  CU(s->ws_mx.ensure((size_t)L.n_rec * D * sizeof(float)));
-  CU(s->ws_mw.ensure((size_t)L.n_col * 64 * sizeof(float)));
   const size_t ex_bytes = 2 * (size_t)L.n_rec * ep::dev::ex_chunks(D) * 16;
   if (ex_bytes > s->ws_mex.bytes || D != s->march_D) s->march_dirty = true;  // other records
   s->march_D = D;
@@ -484,27 +490,38 @@ int ensure_march(ep_schedule* s, int32_t D, ep::dev::MarchPlan& P, cudaStream_t 
   return ensure_ctl(s, st);
 }
 
-ep::dev::MarchArgs march_args(ep_schedule* s, const float* w, const float* x_in, float* x_out, float* out,
-                              int32_t steps, float tau) {
+int ensure_march_grad(ep_schedule* s) {
+  if (!s->d_mgslot.p) CU(upload(s->d_mgslot, s->ml.gslot));
+  return EP_OK;
+}
+
+ep::dev::MarchArgs march_args(ep_schedule* s, const float* w, int32_t steps, int32_t every, float tau) {
   ep::dev::MarchArgs a = {};
   a.part = s->d_mpart.as<ep::MarchPart>();
   a.halo = s->d_mhalo.as<int32_t>();
-  a.nbr = s->d_mnbr.as<int32_t>();
-  a.moff = s->d_moff.as<uint16_t>();
+  a.tab = s->d_mtab.as<uint16_t>();
   a.ent = s->d_ment.as<uint32_t>();
   a.w = w;
-  a.x_in = x_in;
-  a.x_out = x_out;
-  a.out = out;
-  a.every = 1;
   a.ex = s->ws_mex.as<float>();
   a.flag = s->ws_mflag.as<uint32_t>();
   a.err = s->ws_ctl.as<int>() + 2;
   a.n_rec = s->ml.n_rec;
   a.steps = steps;
+  a.every = every;
   a.tau = tau;
   a.stall = s->stall;
   return a;
+}
+
+int march_launch(ep_schedule* s, const ep::dev::MarchPlan& P, const ep::dev::MarchArgs& a, int32_t D, bool grad,
+                 cudaStream_t st) {
+  ep::dev::Timer* t = s->t();
+  const int cls = grad ? ep::dev::T_EDGE_ADJ : ep::dev::T_EDGE_FWD;
+  if (t) t->begin(cls, st);
+  const cudaError_t e = ep::dev::march_run(a, P, D, grad, st);
+  if (t) t->end(cls, st);
+  CU(e);
+  return EP_OK;
 }
 
 // The one-block kernels stage a whole schedule block in shared memory.
@@ -1226,13 +1243,10 @@ int run_march(ep_schedule* s, const ep::dev::MarchPlan& P, int32_t D, int32_t st
   CU(ep::dev::layout_in(rec, s->h.nd, L.n_rec, D, x, mx, st, s->t()));
   CU(ep::dev::gather(s->d_mwmap.as<int32_t>(), 64 * L.n_col, w, mw, st, s->t()));
   if (mout && s->h.touched < s->h.nd) CU(cudaMemsetAsync(mout, 0, (size_t)L.n_rec * D * sizeof(float), st));
-  {
-    ep::dev::Timer* t = s->t();
-    if (t) t->begin(ep::dev::T_EDGE_FWD, st);
-    const cudaError_t e = ep::dev::march_fwd(march_args(s, mw, mx, mx, mout, steps, tau), P, D, st);
-    if (t) t->end(ep::dev::T_EDGE_FWD, st);
-    CU(e);
-  }
+  ep::dev::MarchArgs a = march_args(s, mw, steps, 1, tau);
+  a.x_in = a.x_out = mx;
+  a.out = mout;
+  if (int rc = march_launch(s, P, a, D, false, st)) return rc;
   CU(ep::dev::layout_out(rec, s->h.nd, L.n_rec, D, mx, x, st, s->t()));
   if (out) CU(ep::dev::layout_out(rec, s->h.nd, L.n_rec, D, mout, out, st, s->t()));
   return EP_OK;
@@ -1255,8 +1269,15 @@ int run_flux(ep_schedule* s, int32_t D, int32_t steps, float tau, float* x, cons
   // every workspace of either path now, whatever `steps`: a later call inside
   // a stream capture may take the other one
   ep::dev::MarchPlan P;
-  if (int rc = ensure_march(s, D, P, st)) return rc;
-  if (P.parts && out) CU(s->ws_mout.ensure((size_t)s->ml.n_rec * D * sizeof(float)));
+  P.parts = 0;
+  if (march_wanted(s))
+    if (int rc = march_plan_of(s, D, false, P)) return rc;
+  if (P.parts) {
+    if (int rc = ensure_march(s, D, st)) return rc;
+    CU(s->ws_mx.ensure((size_t)s->ml.n_rec * D * sizeof(float)));
+    CU(s->ws_mw.ensure((size_t)s->ml.n_col * 64 * sizeof(float)));
+    if (out) CU(s->ws_mout.ensure((size_t)s->ml.n_rec * D * sizeof(float)));
+  }
   CU(s->ws_w.ensure((size_t)wlen_of(s) * sizeof(float)));
   if (int rc = ensure_host_maps(s)) return rc;
   if (P.parts && steps > 1) return run_march(s, P, D, steps, tau, x, w, out, from_host, st);
@@ -1329,6 +1350,57 @@ int ep_run_host(ep_schedule* s, int32_t kernel, float* x, const float* w, float*
   return EP_OK;
 }
 
+namespace {
+
+// Records of untouched vertices, which no part holds: carried over as they are.
+int carry_untouched(ep_schedule* s, int32_t D, const float* in, float* out, cudaStream_t st) {
+  const int64_t nr = s->ml.n_rec;
+  if (in == out || s->h.touched == s->h.nd) return EP_OK;
+  const int64_t lo = s->ml.n_run;
+  int32_t first[4], width[4];
+  const int np = ep::planes_of(D, first, width);
+  for (int k = 0; k < np; ++k) {
+    const size_t off = (size_t)first[k] * nr + (size_t)lo * width[k];
+    CU(cudaMemcpyAsync(out + off, in + off, (size_t)(nr - lo) * width[k] * sizeof(float), cudaMemcpyDeviceToDevice, st));
+  }
+  return EP_OK;
+}
+
+// ep_run_adjoint as one resident sweep over one segment.
+int run_adjoint_march(ep_schedule* s, const ep::dev::MarchPlan& P, const float* x0, const float* w, float* lam,
+                      float* grad_w, int32_t D, int32_t steps, float tau, cudaStream_t st) {
+  const ep::MarchLayout& L = s->ml;
+  const size_t state = (size_t)L.n_rec * D, wl = (size_t)L.n_col * 64;
+  if (int rc = ensure_march(s, D, st)) return rc;
+  if (int rc = ensure_march_grad(s)) return rc;
+  CU(s->ws_hist.ensure(state * std::max(2, steps) * sizeof(float)));  // the checkpoint, then the states between
+  CU(s->ws_mx.ensure(state * sizeof(float)));
+  CU(s->ws_lam.ensure(state * sizeof(float)));
+  CU(s->ws_mw.ensure(wl * sizeof(float)));
+  CU(s->ws_gw.ensure(wl * sizeof(float)));
+  const int32_t* rec = s->d_mrec.as<int32_t>();
+  CU(ep::dev::layout_in(rec, s->h.nd, L.n_rec, D, x0, s->ws_mx.as<float>(), st, s->t()));
+  CU(ep::dev::layout_in(rec, s->h.nd, L.n_rec, D, lam, s->ws_lam.as<float>(), st, s->t()));
+  CU(ep::dev::gather(s->d_mwmap.as<int32_t>(), (int64_t)wl, w, s->ws_mw.as<float>(), st, s->t()));
+  CU(cudaMemsetAsync(s->ws_gw.p, 0, wl * sizeof(float), st));
+  ep::dev::MarchArgs a = march_args(s, s->ws_mw.as<float>(), steps, steps, tau);
+  a.x_in = s->ws_mx.as<float>();
+  a.ckpt = s->ws_hist.as<float>();
+  a.hist = a.ckpt + state;
+  a.lam_in = a.lam_out = s->ws_lam.as<float>();
+  a.gw = s->ws_gw.as<float>();
+  if (steps == 1) {  // no exchange orders a neighbour's reads before the result is written
+    a.lam_out = s->ws_hist.as<float>() + state;
+    if (int rc = carry_untouched(s, D, a.lam_in, a.lam_out, st)) return rc;
+  }
+  if (int rc = march_launch(s, P, a, D, true, st)) return rc;
+  CU(ep::dev::layout_out(rec, s->h.nd, L.n_rec, D, a.lam_out, lam, st, s->t()));
+  CU(ep::dev::gather_add(s->d_mgslot.as<int32_t>(), s->h.m, s->ws_gw.as<float>(), grad_w, st, s->t()));
+  return EP_OK;
+}
+
+}  // namespace
+
 int ep_run_adjoint(ep_schedule* s, const float* x0, const float* w, float* lam, float* grad_w,
                    int32_t D, int32_t steps, float tau, void* stream) {
   g_error.clear();
@@ -1346,6 +1418,11 @@ int ep_run_adjoint(ep_schedule* s, const float* x0, const float* w, float* lam, 
   CU(s->ws_gw.ensure((size_t)wlen_of(s) * sizeof(float)));
   fresh_state(s);
   if (int rc = ensure_bacc(s, D, st)) return rc;
+  ep::dev::MarchPlan P;
+  P.parts = 0;
+  if (march_wanted(s) && s->stall < 0)
+    if (int rc = march_plan_of(s, D, true, P)) return rc;
+  if (P.parts) return run_adjoint_march(s, P, x0, w, lam, grad_w, D, steps, tau, st);
   float* hist = s->ws_hist.as<float>();
   if (int rc = layout_in_state(s, D, x0, hist, st)) return rc;
   CU(ep::dev::gather(wmap_of(s), wlen_of(s), w, s->ws_w.as<float>(), st, s->t()));
@@ -1364,6 +1441,118 @@ int ep_run_adjoint(ep_schedule* s, const float* x0, const float* w, float* lam, 
   CU(ep::dev::layout_out(s->d_rec.as<int32_t>(), h.nd, h.n_rec, D, s->ws_lam.as<float>(), lam, st, s->t()));
   CU(ep::dev::gather_add(s->d_gslot.as<int32_t>(), h.m, s->ws_gw.as<float>(), grad_w, st, s->t()));
   return EP_OK;
+}
+
+int ep_grad_sizes(ep_schedule* s, int32_t D, int64_t* state_floats, int64_t* weight_floats) {
+  g_error.clear();
+  if (int rc = check_flux(s, D)) return rc;
+  if (!state_floats || !weight_floats) return fail(EP_EINVAL, "null argument");
+  *state_floats = *weight_floats = 0;
+  if (int rc = ensure_device(s)) return rc;
+  if (!march_wanted(s) || s->stall >= 0) return EP_OK;
+  ep::dev::MarchPlan F, B;
+  if (int rc = march_plan_of(s, D, false, F)) return rc;
+  if (int rc = march_plan_of(s, D, true, B)) return rc;
+  if (!F.parts || !B.parts) return EP_OK;
+  *state_floats = s->ml.n_rec * D;
+  *weight_floats = s->ml.n_col * 64;
+  return EP_OK;
+}
+
+namespace {
+// common checks of the resident-gradient calls; P: the plan of the kernel used
+int grad_checks(ep_schedule* s, int32_t D, const void* a, const void* b, const void* c, const void* d, bool grad,
+                ep::dev::MarchPlan& P, cudaStream_t st) {
+  g_error.clear();
+  if (int rc = check_flux(s, D)) return rc;
+  if (!a || !b || !c || !d) return fail(EP_EINVAL, "null argument");
+  if (misaligned(a) || misaligned(b) || misaligned(c) || misaligned(d))
+    return fail(EP_EINVAL, "buffers in the resident layout must be 16-byte aligned");
+  if (int rc = ensure_device(s)) return rc;
+  if (int rc = march_plan_of(s, D, grad, P)) return rc;
+  if (!P.parts || !s->h.halo.empty())
+    return fail(EP_EINVAL, "this schedule's runs are not resident (ep_grad_sizes gives 0)");
+  if (int rc = ensure_march(s, D, st)) return rc;
+  return ensure_march_grad(s);
+}
+}  // namespace
+
+int ep_grad_state_in(ep_schedule* s, int32_t D, const float* x, float* x_lay, void* stream) {
+  ep::dev::MarchPlan P;
+  cudaStream_t st = as_stream(stream);
+  if (int rc = grad_checks(s, D, x_lay, x_lay, x_lay, x_lay, false, P, st)) return rc;
+  if (!x) return fail(EP_EINVAL, "null argument");
+  CU(ep::dev::layout_in(s->d_mrec.as<int32_t>(), s->h.nd, s->ml.n_rec, D, x, x_lay, st, s->t()));
+  return EP_OK;
+}
+
+int ep_grad_state_out(ep_schedule* s, int32_t D, const float* x_lay, float* x, void* stream) {
+  ep::dev::MarchPlan P;
+  cudaStream_t st = as_stream(stream);
+  if (int rc = grad_checks(s, D, x_lay, x_lay, x_lay, x_lay, false, P, st)) return rc;
+  if (!x) return fail(EP_EINVAL, "null argument");
+  CU(ep::dev::layout_out(s->d_mrec.as<int32_t>(), s->h.nd, s->ml.n_rec, D, x_lay, x, st, s->t()));
+  return EP_OK;
+}
+
+int ep_grad_weights_in(ep_schedule* s, int32_t D, const float* w, float* w_lay, void* stream) {
+  ep::dev::MarchPlan P;
+  cudaStream_t st = as_stream(stream);
+  if (int rc = grad_checks(s, D, w_lay, w_lay, w_lay, w_lay, false, P, st)) return rc;
+  if (!w) return fail(EP_EINVAL, "null argument");
+  CU(ep::dev::gather(s->d_mwmap.as<int32_t>(), 64 * s->ml.n_col, w, w_lay, st, s->t()));
+  return EP_OK;
+}
+
+int ep_grad_weights_out(ep_schedule* s, int32_t D, const float* gw_lay, float* grad_w, void* stream) {
+  ep::dev::MarchPlan P;
+  cudaStream_t st = as_stream(stream);
+  if (int rc = grad_checks(s, D, gw_lay, gw_lay, gw_lay, gw_lay, false, P, st)) return rc;
+  if (!grad_w) return fail(EP_EINVAL, "null argument");
+  CU(ep::dev::gather(s->d_mgslot.as<int32_t>(), s->h.m, gw_lay, grad_w, st, s->t()));
+  return EP_OK;
+}
+
+int ep_grad_forward(ep_schedule* s, int32_t D, const float* x_lay, float* xT_lay, const float* w_lay, float* ckpt,
+                    int32_t steps, int32_t every, float tau, void* stream) {
+  ep::dev::MarchPlan P;
+  cudaStream_t st = as_stream(stream);
+  if (steps < 1 || every < 1) {
+    g_error.clear();
+    return fail(EP_EINVAL, "steps and every must be >= 1");
+  }
+  if (int rc = grad_checks(s, D, x_lay, xT_lay, w_lay, ckpt, false, P, st)) return rc;
+  if (steps == 1 && x_lay == xT_lay) return fail(EP_EINVAL, "one step cannot be made in place");
+  if (int rc = carry_untouched(s, D, x_lay, xT_lay, st)) return rc;
+  ep::dev::MarchArgs a = march_args(s, w_lay, steps, every, tau);
+  a.x_in = x_lay;
+  a.x_out = xT_lay;
+  a.ckpt = ckpt;
+  return march_launch(s, P, a, D, false, st);
+}
+
+int ep_grad_backward(ep_schedule* s, int32_t D, const float* ckpt, float* hist, const float* w_lay,
+                     const float* lam_in, float* lam_out, float* gw_lay, int32_t steps, int32_t every, float tau,
+                     void* stream) {
+  ep::dev::MarchPlan P;
+  cudaStream_t st = as_stream(stream);
+  if (steps < 1 || every < 1) {
+    g_error.clear();
+    return fail(EP_EINVAL, "steps and every must be >= 1");
+  }
+  if (int rc = grad_checks(s, D, ckpt, w_lay, lam_in, lam_out, true, P, st)) return rc;
+  if (!gw_lay || misaligned(gw_lay) || misaligned(hist)) return fail(EP_EINVAL, "null or unaligned buffer");
+  if (!hist && std::min(steps, every) > 2) return fail(EP_EINVAL, "null history buffer");
+  if (steps == 1 && lam_in == lam_out) return fail(EP_EINVAL, "one step cannot be made in place");
+  if (int rc = carry_untouched(s, D, lam_in, lam_out, st)) return rc;
+  CU(cudaMemsetAsync(gw_lay, 0, (size_t)s->ml.n_col * 64 * sizeof(float), st));
+  ep::dev::MarchArgs a = march_args(s, w_lay, steps, every, tau);
+  a.ckpt = const_cast<float*>(ckpt);  // only read: x_in is null
+  a.hist = hist;
+  a.lam_in = lam_in;
+  a.lam_out = lam_out;
+  a.gw = gw_lay;
+  return march_launch(s, P, a, D, true, st);
 }
 
 int ep_timing(ep_schedule* s, int32_t enable) {

@@ -102,14 +102,17 @@ const void* flux_tma_kernel_ptr(int D, bool adjoint);
 struct MarchArgs {
   const MarchPart* part;
   const int32_t* halo;
-  const int32_t* nbr;
-  const uint16_t* moff;
+  const uint16_t* tab;
   const uint32_t* ent;
   const float* w;      // weights in the layout's slots
-  const float* x_in;   // planar state of n_rec records
+  const float* x_in;   // planar state of n_rec records, the owners' ones written
   float* x_out;        // may equal x_in when steps > 1
   float* out;          // flux of the last step, or nullptr
-  float* ckpt;         // states before steps 0, every, 2 every, ...; or nullptr
+  float* ckpt;         // images of the states before steps 0, every, 2 every, ...; or nullptr
+  const float* lam_in; // gradient: cotangent in and out, images between two
+  float* lam_out;      // checkpoints (every - 1), weight gradient slots (added to)
+  float* hist;
+  float* gw;
   float* ex;           // 2 x n_rec exchange records (ex_chunks(D) chunks)
   uint32_t* flag;      // steps published so far by every part
   int* err;
@@ -117,23 +120,24 @@ struct MarchArgs {
   int every, steps;
   float tau;
   int stall;           // test hook: part 0 leaves after publishing this many steps (-1: off)
-  int npos, off_moff, off_ent, off_w;
+  int warps, npos, off_lam, off_tab, off_ent, off_w;
   uint32_t hold_cols, tmem_cols;
 };
 // 16-byte chunks of one exchange record: three components and a tag each
 __host__ __device__ constexpr int ex_chunks(int D) { return (D + 2) / 3; }
 struct MarchSizes {
-  int32_t parts, max_pos, max_col, max_nsl;
+  int32_t parts, warps, max_pos, max_col, max_nsl;
 };
 struct MarchPlan {
   int parts;  // 0: does not fit
-  int threads, npos, off_moff, off_ent, off_w, hold_cols, tmem_cols;
+  int threads, warps, npos, off_lam, off_tab, off_ent, off_w, hold_cols, tmem_cols;
   bool resident;  // slots and weights stay in shared memory too
   size_t smem;
 };
-MarchPlan march_plan(const MarchSizes& z, int D, int smem_max);
-const void* march_kernel_ptr(int D, bool resident);
-cudaError_t march_fwd(const MarchArgs& a, const MarchPlan& P, int D, cudaStream_t st);
+// grad: the reverse sweep (state and cotangent on the chip), else the forward run
+MarchPlan march_plan(const MarchSizes& z, int D, bool grad, int smem_max);
+const void* march_kernel_ptr(int D, bool grad, bool resident);
+cudaError_t march_run(const MarchArgs& a, const MarchPlan& P, int D, bool grad, cudaStream_t st);
 
 cudaError_t flux_step(const FluxArgs& a, int D, cudaStream_t st);
 // read-only-cache variant (no staging); needs max_np <= 4096

@@ -38,7 +38,8 @@ struct Entry {
 // columns so that the 32 lanes of a column read their other positions from
 // different shared-memory banks as far as the lists allow (a 16-byte load is
 // served 8 lanes at a time, 4 banks each; a 4-byte load 32 lanes at a time).
-// Unused slots name the lane's own position; put(column, lane, entry or null).
+// Unused slots name the lane's own position; put(column, lane, position, entry
+// or null).
 template <typename Put>
 void spread_slice(std::vector<Entry>& ents, const int32_t* lo0, const int32_t* hi, int32_t p0, int32_t K, Put put) {
   int32_t lo[32];
@@ -64,11 +65,11 @@ void spread_slice(std::vector<Entry>& ents, const int32_t* lo0, const int32_t* h
           if (sc < bs) best = i, bs = sc;
         }
         if (best < 0) {
-          put(c, l, (const Entry*)nullptr);
+          put(c, l, p0 + l, (const Entry*)nullptr);
           take(l, p0 + l);
         } else {
           std::swap(ents[lo[l]], ents[best]);
-          put(c, l, &ents[lo[l]]);
+          put(c, l, ents[lo[l]].o, &ents[lo[l]]);
           take(l, ents[lo[l]++].o);
         }
       }
@@ -180,16 +181,14 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
   L = MarchLayout();
   L.parts = P;
   L.part.assign(P, MarchPart{});
-  int64_t next = 0;
   for (int32_t q = 0; q < P; ++q) {
     MarchPart& d = L.part[q];
-    d.lo = (int32_t)next;
     d.own = (int32_t)(cut[q + 1] - cut[q]);
     d.nsl = (d.own + 31) / 32;
     d.hbase = (d.own + 3) & ~3;
-    next += d.hbase;
+    L.max_nsl = std::max(L.max_nsl, d.nsl);
   }
-  const int64_t run = next;
+  L.warps = std::max(4, std::min(32, (L.max_nsl + 3) / 4 * 4));
   // positions: boundary vertices first, then by descending degree
   parallel_for(P, threads, [&](int, int64_t q) {
     MarchPart& d = L.part[q];
@@ -202,44 +201,59 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
       key[i] = {-((bnd ? 2 * kMarchMaxDegree : 0) + ptr[v + 1] - ptr[v]), i};
     }
     std::sort(key.begin(), key.end());
-    for (int32_t p = 0; p < d.own; ++p) rec[order[cut[q] + key[p].second]] = d.lo + p;
+    for (int32_t p = 0; p < d.own; ++p) rec[order[cut[q] + key[p].second]] = p;
+    // (rec: position so far; its part's first record is added below)
   });
-  // halo lists, then the slots
+  // halo lists (by vertex, then sorted by record once the runs have a place)
   struct Piece {
-    std::vector<int32_t> halo, nbr, wmap;
-    std::vector<uint16_t> moff;
+    std::vector<int32_t> halo, wmap;
+    std::vector<uint16_t> tab;
     std::vector<uint32_t> ent;
   };
   std::vector<Piece> piece(P);
+  parallel_for(P, threads, [&](int, int64_t q) {
+    std::vector<int32_t>& halo = piece[q].halo;
+    for (int64_t i = cut[q]; i < cut[q + 1]; ++i)
+      for (int32_t j = ptr[order[i]]; j < ptr[order[i] + 1]; ++j)
+        if (part_of[nb[j]] != q) halo.push_back(nb[j]);
+    std::sort(halo.begin(), halo.end());
+    halo.erase(std::unique(halo.begin(), halo.end()), halo.end());
+    L.part[q].nh = (int32_t)halo.size();
+  });
+  int64_t next = 0;
+  for (MarchPart& d : L.part) {
+    if (d.hbase + d.nh > (int32_t)kSlotPos) return false;
+    d.lo = (int32_t)next;
+    next += d.hbase + ((d.nh + 3) & ~3);
+    if (next > INT32_MAX / 2) return false;
+  }
+  for (int64_t v = 0; v < n; ++v) rec[v] += L.part[part_of[v]].lo;
+  // the slots
   L.gslot.assign(m, -1);
   std::atomic<bool> ok{true};
   parallel_for(P, threads, [&](int, int64_t q) {
     MarchPart& d = L.part[q];
     Piece& t = piece[q];
+    for (int32_t& v : t.halo) v = rec[v];
+    std::sort(t.halo.begin(), t.halo.end());
     std::vector<int32_t> vert(d.own);
     for (int64_t r = cut[q]; r < cut[q + 1]; ++r) vert[rec[order[r]] - d.lo] = order[r];
-    for (int32_t p = 0; p < d.nb; ++p)
-      for (int32_t j = ptr[vert[p]]; j < ptr[vert[p] + 1]; ++j) {
-        const int32_t o = nb[j];
-        if (part_of[o] != q) t.halo.push_back(rec[o]), t.nbr.push_back(part_of[o]);
-      }
-    for (auto* l : {&t.halo, &t.nbr}) {
-      std::sort(l->begin(), l->end());
-      l->erase(std::unique(l->begin(), l->end()), l->end());
-    }
-    d.nh = (int32_t)t.halo.size();
-    d.ng = (int32_t)t.nbr.size();
-    if (d.hbase + d.nh > (int32_t)kSlotPos) {
-      ok = false;
-      return;
-    }
-    t.moff.push_back(0);
+    std::vector<std::pair<int32_t, int32_t>> hpos(d.nh);  // record, position
+    for (int32_t i = 0; i < d.nh; ++i) hpos[i] = {t.halo[i], d.hbase + i};
+    auto halo_index = [&](int32_t r) {
+      return (int32_t)(std::lower_bound(hpos.begin(), hpos.end(), std::make_pair(r, (int32_t)-1)) - hpos.begin());
+    };
+    auto pos_of = [&](int32_t o) { return part_of[o] == q ? rec[o] - d.lo : hpos[halo_index(rec[o])].second; };
+    const int32_t W = L.warps;
+    std::vector<int32_t> kcol(d.nsl), c0(d.nsl);
+    for (int32_t j = 0; j < d.nsl; ++j)
+      for (int32_t p = 32 * j; p < std::min(d.own, 32 * j + 32); ++p)
+        kcol[j] = std::max(kcol[j], (ptr[vert[p] + 1] - ptr[vert[p]] + 1) / 2);
     int32_t cols = 0;
-    for (int32_t j = 0; j < d.nsl; ++j) {
-      int32_t K = 0;
-      for (int32_t p = 32 * j; p < std::min(d.own, 32 * j + 32); ++p) K = std::max(K, ptr[vert[p] + 1] - ptr[vert[p]]);
-      cols += (K + 1) / 2;
-      t.moff.push_back((uint16_t)cols);
+    t.tab.resize(W + d.nsl);
+    for (int32_t v = 0; v < W; ++v) {
+      t.tab[v] = (uint16_t)cols;
+      for (int32_t j = v; j < d.nsl; j += W) c0[j] = cols, cols += kcol[j], t.tab[W + j] = (uint16_t)kcol[j];
     }
     if (cols > 0xffff) {
       ok = false;
@@ -258,50 +272,44 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
         if (p < d.own)
           for (int32_t i = ptr[vert[p]]; i < ptr[vert[p] + 1]; ++i) {
             const int32_t o = nb[i], e = s.edge_perm[inc[i] < 0 ? ~inc[i] : inc[i]];
-            const int32_t po = part_of[o] == q ? rec[o] - d.lo
-                                               : d.hbase + (int32_t)(std::lower_bound(t.halo.begin(), t.halo.end(), rec[o]) -
-                                                                     t.halo.begin());
-            ents.push_back(Entry{po, e, inc[i] >= 0});
+            ents.push_back(Entry{pos_of(o), e, inc[i] >= 0});
           }
         hi[l] = (int32_t)ents.size();
       }
-      const int32_t c0 = t.moff[j], K = 2 * (t.moff[j + 1] - c0);
-      spread_slice(ents, lo, hi, 32 * j, K, [&](int32_t c, int l, const Entry* x) {
-        const size_t at = (size_t)32 * (c0 + c / 2) + l;
-        const uint32_t v = x ? (uint32_t)x->o | (x->src ? kSlotSrc : 0u) : (uint32_t)(32 * j + l);
+      spread_slice(ents, lo, hi, 32 * j, 2 * kcol[j], [&](int32_t c, int l, int32_t o, const Entry* x) {
+        const size_t at = (size_t)32 * (c0[j] + c / 2) + l;
+        const uint32_t v = (uint32_t)o | (x && x->src ? kSlotSrc : 0u);
         t.ent[at] |= v << (16 * (c & 1));
         if (x) t.wmap[2 * at + (c & 1)] = x->e;
       });
     }
-    while (t.halo.size() % 4) t.halo.push_back(0);
-    while (t.moff.size() % 8) t.moff.push_back(0);
+    while (t.tab.size() % 8) t.tab.push_back(0);
   });
   if (!ok) return false;
-  int64_t nh = 0, ng = 0, nq = 0, nc = 0;
+  int64_t nh = 0, nq = 0, nc = 0;
   for (int32_t q = 0; q < P; ++q) {
     MarchPart& d = L.part[q];
-    d.h0 = (int32_t)nh, d.g0 = (int32_t)ng, d.q0 = (int32_t)nq, d.s0 = (int32_t)nc;
-    nh += (int64_t)piece[q].halo.size(), ng += d.ng, nq += (int64_t)piece[q].moff.size(), nc += d.ncol;
-    L.max_pos = std::max(L.max_pos, std::max(d.hbase + d.nh, 32 * d.nsl));
-    L.max_nh = std::max(L.max_nh, d.nh);
+    d.h0 = (int32_t)nh, d.q0 = (int32_t)nq, d.s0 = (int32_t)nc;
+    nh += d.nh, nq += (int64_t)piece[q].tab.size(), nc += d.ncol;
+    L.max_pos = std::max(L.max_pos, std::max(d.hbase + ((d.nh + 3) & ~3), 32 * d.nsl));
     L.max_col = std::max(L.max_col, d.ncol);
-    L.max_nsl = std::max(L.max_nsl, d.nsl);
   }
-  if (nc > INT32_MAX / 64 || run > INT32_MAX / 2) return false;
+  nc += kMarchAhead;
+  if (nc > INT32_MAX / 64) return false;
   L.n_col = nc;
-  L.halo.resize(nh), L.nbr.resize(ng), L.moff.resize(nq), L.ent.resize(32 * nc), L.wmap.resize(64 * nc);
+  L.halo.resize(nh), L.tab.resize(nq), L.ent.resize(32 * nc, 0), L.wmap.resize(64 * nc, -1);
   parallel_for(P, threads, [&](int, int64_t q) {
     const MarchPart& d = L.part[q];
     const Piece& t = piece[q];
     std::copy(t.halo.begin(), t.halo.end(), L.halo.begin() + d.h0);
-    std::copy(t.nbr.begin(), t.nbr.end(), L.nbr.begin() + d.g0);
-    std::copy(t.moff.begin(), t.moff.end(), L.moff.begin() + d.q0);
+    std::copy(t.tab.begin(), t.tab.end(), L.tab.begin() + d.q0);
     std::copy(t.ent.begin(), t.ent.end(), L.ent.begin() + 32 * (int64_t)d.s0);
     std::copy(t.wmap.begin(), t.wmap.end(), L.wmap.begin() + 64 * (int64_t)d.s0);
     for (int64_t i = 0; i < 64 * (int64_t)d.ncol; ++i)
       if (t.wmap[i] >= 0 && ((t.ent[i / 2] >> (16 * (i & 1))) & kSlotSrc))
         L.gslot[t.wmap[i]] = (int32_t)(64 * (int64_t)d.s0 + i);
   });
+  L.n_run = next;
   L.rec_of.resize(nd);
   for (int64_t v = 0; v < nd; ++v)  // untouched vertices after the parts
     L.rec_of[v] = s.relabel[v] < n ? rec[s.relabel[v]] : (int32_t)next++;

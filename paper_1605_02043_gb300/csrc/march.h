@@ -18,36 +18,41 @@
 namespace ep {
 
 // One part.  Positions [0, own): its vertices, the boundary ones (in some
-// other part's halo) first, each class by descending degree; position p is
-// the state record lo + p.  Positions [hbase, hbase + nh): the halo, record
-// halo[h0 + j] (ascending).  Slices of 32 positions; slice j has
-// moff[q0 + j + 1] - moff[q0 + j] pair columns, each 32 lanes of two slots:
-// entry pair 32 * (s0 + column) + lane holds two 16-bit entries (position of
-// the other endpoint, kSlotSrc on the task's first endpoint) and two weights.
-// An unused slot names the lane's own position with weight 0 (its difference
-// is zero by itself).
+// other part's halo) first, each class by descending degree; positions
+// [hbase, hbase + nh): the halo, ascending by record.  Position p is the state
+// record lo + p, own or halo, so a part's image is one run of records; halo[h0
+// + j] is the record where halo position j is its owner's.  Slices of 32
+// positions are dealt to `warps` warps, slice j to warp j % warps; the pair
+// columns (32 lanes of two slots each) of one warp's slices follow each other,
+// so that a warp reads its columns as one stream: warp v's start at column s0 +
+// tab[q0 + v], and slice j has tab[q0 + warps + j] of them.  Entry pair 32 *
+// column + lane holds two 16-bit entries (position of the other endpoint,
+// kSlotSrc on the task's first endpoint) and two weights.  An unused slot names
+// the lane's own position with weight 0 (its difference is zero by itself).
 struct MarchPart {
   int32_t lo, own, nb, nsl;
   int32_t hbase, nh, h0, q0;
   int32_t s0, ncol;  // pair columns [s0, s0 + ncol)
-  int32_t g0, ng;    // parts that share a boundary: nbr[g0 .. g0 + ng)
-  int32_t pad[4];
+  int32_t pad[6];
 };
 static_assert(sizeof(MarchPart) == 64, "MarchPart layout");
 
+// Columns past the last one that a stream's read-ahead may touch.
+constexpr int kMarchAhead = 2;
+
 struct MarchLayout {
-  int32_t parts = 0;
+  int32_t parts = 0, warps = 0;
   int64_t n_rec = 0;               // records per plane of a state (multiple of 4)
-  int64_t n_col = 0;               // pair columns in all (64 weights each)
+  int64_t n_run = 0;               // records [0, n_run) are the parts' images
+  int64_t n_col = 0;               // pair columns in all, kMarchAhead unused ones included
   std::vector<MarchPart> part;
-  std::vector<int32_t> rec_of;     // data vertex -> record (untouched vertices after the parts)
-  std::vector<int32_t> halo;       // records, each part's list padded to 4
-  std::vector<int32_t> nbr;        // neighbouring parts
-  std::vector<uint16_t> moff;      // pair-column offsets, each part's table padded to 8
+  std::vector<int32_t> rec_of;     // data vertex -> its own record (untouched vertices after the parts)
+  std::vector<int32_t> halo;       // owners' records
+  std::vector<uint16_t> tab;       // stream starts and slice columns, each part's padded to 8
   std::vector<uint32_t> ent;       // entry pairs
-  std::vector<int32_t> wmap;       // weight slot (pair column, lane, which) -> task, -1 unused
+  std::vector<int32_t> wmap;       // weight slot (64 column + 2 lane + which) -> task, -1 unused
   std::vector<int32_t> gslot;      // task -> weight slot at its first endpoint
-  int32_t max_pos = 0, max_nh = 0, max_col = 0, max_nsl = 0;
+  int32_t max_pos = 0, max_col = 0, max_nsl = 0;
 };
 
 // Builds the layout for at most `max_parts` parts.  False when the graph does

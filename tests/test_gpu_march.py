@@ -83,6 +83,40 @@ def test_hub_takes_the_step_kernels():
     assert run_against_oracle(S, src, dst, n, 3, 3, 3, tau=1e-4) == 3
 
 
+@pytest.mark.parametrize("n,C,D,steps,every,default_order", [
+    (40, 16, 5, 3, 2, False), (129, 64, 1, 1, 1, False), (300, 64, 3, 7, 3, True), (4096, 256, 2, 6, 6, False),
+    (9999, 512, 5, 10, 1, False), (20011, 512, 8, 4, 3, False), (50021, 1024, 5, 5, 9, False),
+    (9999, 512, 6, 2, 2, True), (120011, 512, 4, 5, 2, False), (200003, 1024, 7, 3, 5, False),
+])
+def test_gradients_match_oracle(n, C, D, steps, every, default_order):
+    """Forward run and reverse sweep in one launch each (autograd and ep_run_adjoint);
+    isolated vertices keep their state and cotangent."""
+    from paper_1605_02043_gb300.autograd import flux_steps
+
+    src, dst = W.knn_mesh(n, 4, 1)
+    n += 3  # untouched
+    S = E.Schedule.partition(src, dst, n, C, default_order=default_order)
+    assert S.grad_sizes(D)[0] > 0
+    x0, w, g, tau = W.flux_state(n, D, n), W.flux_weights(src.size, n), W.loss_weights(n, D, 1), 1e-2
+    xT_ref, _ = O.flux_steps(src, dst, x0, w, steps, tau)
+    dx_ref, dw_ref = O.flux_adjoint(src, dst, x0, w, steps, tau, g)
+    for _ in range(2):
+        x, wt = cuda(x0).requires_grad_(True), cuda(w).requires_grad_(True)
+        S.timing(2)
+        xT = flux_steps(x, wt, S, steps, tau, every)
+        xT.backward(cuda(g))
+        assert (S.timing_read(E.T_EDGE_FWD)[1], S.timing_read(E.T_EDGE_ADJ)[1]) == (1, 1)
+        S.timing(0)
+        check_state(xT, xT_ref, x0, steps, "xT")
+        check_state(x.grad, dx_ref, g, steps, "dx0")
+        check_field(wt.grad, dw_ref, "dw")
+    lam, gw = cuda(g), torch.full((src.size,), 2.0, device="cuda")
+    S.run_adjoint(cuda(x0), cuda(w), lam, gw, steps=steps, tau=tau)
+    check_state(lam, dx_ref, g, steps, "dx0 (ep_run_adjoint)")
+    check_field(gw, 2.0 + dw_ref, "accumulated dw (ep_run_adjoint)")
+    assert S.check_errors() == 0
+
+
 def test_two_streams_and_graph_replay():
     """Runs of two schedules on two streams, then captured and replayed."""
     n = 30011
