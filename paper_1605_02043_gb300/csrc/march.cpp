@@ -34,45 +34,179 @@ struct Entry {
   bool src;
 };
 
-// Columns of one slice: lane l's entries ents[lo[l] .. hi[l]) spread over K
-// columns so that the 32 lanes of a column read their other positions from
-// different shared-memory banks as far as the lists allow (a 16-byte load is
-// served 8 lanes at a time, 4 banks each; a 4-byte load 32 lanes at a time).
-// Unused slots name the lane's own position; put(column, lane, position, entry
-// or null).
-template <typename Put>
-void spread_slice(std::vector<Entry>& ents, const int32_t* lo0, const int32_t* hi, int32_t p0, int32_t K, Put put) {
-  int32_t lo[32];
-  std::copy(lo0, lo0 + 32, lo);
-  for (int32_t c = 0; c < K; ++c) {
-    uint32_t used32 = 0, used8[4] = {0, 0, 0, 0};
-    auto score = [&](int l, int32_t o) {
-      return 2 * (int)((used8[l >> 3] >> (o & 7)) & 1u) + (int)((used32 >> (o & 31)) & 1u);
-    };
-    auto take = [&](int l, int32_t o) {
-      used8[l >> 3] |= 1u << (o & 7);
-      used32 |= 1u << (o & 31);
-    };
-    uint32_t forced_mask = 0;  // lanes with an entry for every remaining column go first
-    for (int l = 0; l < 32; ++l) forced_mask |= (uint32_t)(hi[l] - lo[l] == K - c) << l;
-    for (int pass = 0; pass < 2; ++pass)
-      for (int l = 0; l < 32; ++l) {
-        const bool forced = (forced_mask >> l) & 1u;
-        if ((pass == 0) != forced) continue;
-        int32_t best = -1, bs = forced ? 4 : score(l, p0 + l) + 1;
-        for (int32_t i = lo[l]; i < hi[l] && bs > 0; ++i) {
-          const int sc = score(l, ents[i].o);
-          if (sc < bs) best = i, bs = sc;
+// Shared-memory banks.  A column of a slice is one load per plane: a 16-byte
+// load is served 8 lanes at a time, each record covering the 4 banks of its
+// position mod 8; a 4-byte load 32 lanes at a time, position mod 32.  Two
+// things are free: the order of the 8 vertices of an octet of positions (the
+// residues its neighbours see), and which column a slot goes to.  Both are
+// chosen here; greedy columns alone left 8.3 wavefronts per 16-byte column on
+// the 1M-point mesh (4 is the least), and the gathers were what a step waited
+// for (11 us of 14).
+
+// Residues: swaps inside octets of [lo, hi) (aligned to 8) that even out, for
+// every reading octet, how many of its slots fall on each residue (sum of
+// squares).  readers(p): positions whose slots name position p; cnt: [octet][8].
+// swapped(a, b) carries the swap out.
+template <typename Readers, typename Swapped>
+void even_residues(int32_t lo, int32_t hi, int32_t keep, std::vector<int32_t>& cnt, Readers readers, Swapped swapped) {
+  auto shift = [&](int32_t p, int from, int to) {  // cost change when p's residue moves
+    int32_t c = 0;
+    for (int32_t q : readers(p)) {
+      int32_t* n = &cnt[(q >> 3) * 8];
+      c += 1 - 2 * n[from]--;
+      c += 1 + 2 * n[to]++;
+    }
+    return c;
+  };
+  for (int pass = 0; pass < 2; ++pass)
+    for (int32_t o = lo; o < hi; o += 8)
+      for (int32_t i = o; i < std::min(hi, o + 8); ++i)
+        for (int32_t j = i + 1; j < std::min(hi, o + 8); ++j) {
+          if ((i < keep) != (j < keep)) continue;  // a boundary position stays one
+          const int32_t c = shift(i, i & 7, j & 7) + shift(j, j & 7, i & 7);
+          if (c < 0) {
+            swapped(i, j);
+          } else {
+            shift(i, j & 7, i & 7);
+            shift(j, i & 7, j & 7);
+          }
         }
-        if (best < 0) {
-          put(c, l, p0 + l, (const Entry*)nullptr);
-          take(l, p0 + l);
-        } else {
-          std::swap(ents[lo[l]], ents[best]);
-          put(c, l, ents[lo[l]].o, &ents[lo[l]]);
-          take(l, ents[lo[l]++].o);
+}
+
+// Columns of one octet: lane l's entries (n[l] <= K of them, residues in
+// res[l]) get different columns, and entries of one residue different columns
+// too as far as there are no more than K of them: an edge colouring of the
+// bipartite lane-residue graph, by alternating paths (Koenig).  col[l][i]
+// receives the column of entry i.
+struct OctetColumns {
+  std::vector<int16_t> lane_at, res_at;  // [8][K]: entry of a lane / lane of a residue in a column
+  void run(const int32_t* n, const uint8_t* const* res, int32_t K, int16_t* const* col) {
+    lane_at.assign(8 * (size_t)K, -1);
+    res_at.assign(8 * (size_t)K, -1);
+    for (int l = 0; l < 8; ++l)
+      for (int32_t i = 0; i < n[l]; ++i) {
+        const int r = res[l][i];
+        int32_t a = -1, b = -1, both = -1;
+        for (int32_t c = 0; c < K && both < 0; ++c) {
+          const bool fl = lane_at[l * K + c] < 0, fr = res_at[r * K + c] < 0;
+          if (fl && fr) both = c;
+          if (fl && a < 0) a = c;
+          if (fr && b < 0) b = c;
         }
+        if (both < 0 && b >= 0) {  // a is free at the lane, b at the residue: swap a and b along the path from r
+          int rr = r;
+          const int32_t x = a, y = b;
+          int path_l[8], n_path = 0;  // residue -x- lane -y- residue -x- ...
+          while (n_path < 8) {
+            const int ll = res_at[rr * K + x];
+            if (ll < 0) break;
+            path_l[n_path++] = ll;
+            const int16_t e2 = lane_at[ll * K + y];
+            if (e2 < 0) break;
+            rr = res[ll][e2];
+            if (res_at[rr * K + y] != ll) break;  // an overflowing entry ends the path
+          }
+          auto mark = [&](int k, bool on) {
+            const int ll = path_l[k];
+            for (int32_t c : {x, y}) {
+              const int16_t e2 = lane_at[ll * K + c];
+              if (e2 < 0) continue;
+              int16_t& at = res_at[res[ll][e2] * K + c];
+              if (on ? at < 0 : at == ll) at = on ? (int16_t)ll : (int16_t)-1;
+            }
+          };
+          for (int k = 0; k < n_path; ++k) mark(k, false);
+          for (int k = 0; k < n_path; ++k) std::swap(lane_at[path_l[k] * K + x], lane_at[path_l[k] * K + y]);
+          for (int k = 0; k < n_path; ++k) mark(k, true);
+          both = a;
+        }
+        const int32_t c = both >= 0 ? both : a;
+        lane_at[l * K + c] = (int16_t)i;
+        if (res_at[r * K + c] < 0) res_at[r * K + c] = (int16_t)l;
       }
+    for (int l = 0; l < 8; ++l)
+      for (int32_t c = 0; c < K; ++c)
+        if (lane_at[l * K + c] >= 0) col[l][lane_at[l * K + c]] = (int16_t)c;
+  }
+};
+
+// The slots of one slice: lane l's entries ents[lo[l] .. hi[l]) over K columns,
+// octet by octet; an octet's columns are then ordered so that the four octets'
+// positions mod 32 differ where they can.  An unused slot names the lane's own
+// position or one of its neighbours, whichever falls on a bank that is free or
+// read there anyway (its weight is 0 and its term zero whenever the lane's
+// used slots are finite); put(column, lane, position, entry or null).
+template <typename Put>
+void spread_slice(const std::vector<Entry>& ents, const int32_t* lo, const int32_t* hi, int32_t p0, int32_t K,
+                  OctetColumns& oc, Put put) {
+  std::vector<uint32_t> used(K, 0);  // residues mod 32 per final column
+  std::vector<uint8_t> res[8];
+  std::vector<int16_t> col[8];
+  for (int g = 0; g < 4; ++g) {
+    int32_t n[8];
+    const uint8_t* rp[8];
+    int16_t* cp[8];
+    std::vector<uint32_t> mine(K, 0);
+    for (int l = 0; l < 8; ++l) {
+      const int L = 8 * g + l;
+      n[l] = hi[L] - lo[L];
+      res[l].resize(n[l]);
+      col[l].resize(n[l]);
+      for (int32_t i = 0; i < n[l]; ++i) res[l][i] = (uint8_t)(ents[lo[L] + i].o & 7);
+      rp[l] = res[l].data();
+      cp[l] = col[l].data();
+    }
+    oc.run(n, rp, K, cp);
+    for (int l = 0; l < 8; ++l)
+      for (int32_t i = 0; i < n[l]; ++i) mine[col[l][i]] |= 1u << (ents[lo[8 * g + l] + i].o & 31);
+    // each of this octet's columns to the final column it clashes least with
+    std::vector<int32_t> to(K, -1);
+    std::vector<bool> taken(K, false);
+    for (int32_t c = 0; c < K; ++c) {
+      int32_t best = -1, bs = 64;
+      for (int32_t f = 0; f < K; ++f) {
+        if (taken[f]) continue;
+        const int sc = __builtin_popcount(used[f] & mine[c]);
+        if (sc < bs) best = f, bs = sc;
+      }
+      to[c] = best;
+      taken[best] = true;
+    }
+    for (int32_t c = 0; c < K; ++c) {
+      const int32_t f = to[c];
+      uint32_t used8 = 0;
+      int32_t named[8];
+      int16_t at[8];
+      for (int l = 0; l < 8; ++l) {
+        at[l] = oc.lane_at[l * K + c];
+        if (at[l] >= 0) named[l] = ents[lo[8 * g + l] + at[l]].o, used8 |= 1u << (named[l] & 7), used[f] |= 1u << (named[l] & 31);
+      }
+      for (int l = 0; l < 8; ++l) {
+        const int L = 8 * g + l;
+        if (at[l] >= 0) {
+          put(f, L, named[l], &ents[lo[L] + at[l]]);
+          continue;
+        }
+        int32_t best = p0 + L, bs = 8;
+        auto score = [&](int32_t o) {
+          for (int k = 0; k < 8; ++k)
+            if (at[k] >= 0 && named[k] == o) return 0;  // read there anyway
+          return 2 * (int)(used8 >> (o & 7) & 1u) + (int)(used[f] >> (o & 31) & 1u);
+        };
+        if ((bs = score(best)) > 0)
+          for (int32_t i = lo[L]; i < hi[L] && bs > 0; ++i) {
+            const int sc = score(ents[i].o);
+            if (sc < bs) best = ents[i].o, bs = sc;
+          }
+        if (n[l] == 0)  // no vertex here: anything another lane reads
+          for (int k = 0; k < 8 && bs > 0; ++k)
+            if (at[k] >= 0) best = named[k], bs = 0;
+        named[l] = best;
+        used8 |= 1u << (best & 7);
+        used[f] |= 1u << (best & 31);
+        put(f, L, best, (const Entry*)nullptr);
+      }
+    }
   }
 }
 
@@ -201,7 +335,23 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
       key[i] = {-((bnd ? 2 * kMarchMaxDegree : 0) + ptr[v + 1] - ptr[v]), i};
     }
     std::sort(key.begin(), key.end());
-    for (int32_t p = 0; p < d.own; ++p) rec[order[cut[q] + key[p].second]] = p;
+    std::vector<int32_t> vert(d.own), cnt(((size_t)d.own + 8) / 8 * 8, 0), seen;
+    for (int32_t p = 0; p < d.own; ++p) vert[p] = order[cut[q] + key[p].second], rec[vert[p]] = p;
+    for (int32_t p = 0; p < d.own; ++p)
+      for (int32_t j = ptr[vert[p]]; j < ptr[vert[p] + 1]; ++j)
+        if (part_of[nb[j]] == q) ++cnt[(p >> 3) * 8 + (rec[nb[j]] & 7)];
+    even_residues(
+        0, d.own, d.nb, cnt,
+        [&](int32_t p) -> const std::vector<int32_t>& {
+          seen.clear();
+          for (int32_t j = ptr[vert[p]]; j < ptr[vert[p] + 1]; ++j)
+            if (part_of[nb[j]] == q) seen.push_back(rec[nb[j]]);
+          return seen;
+        },
+        [&](int32_t i, int32_t j) {
+          std::swap(vert[i], vert[j]);
+          rec[vert[i]] = i, rec[vert[j]] = j;
+        });
     // (rec: position so far; its part's first record is added below)
   });
   // halo lists (by vertex, then sorted by record once the runs have a place)
@@ -235,7 +385,7 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
     MarchPart& d = L.part[q];
     Piece& t = piece[q];
     for (int32_t& v : t.halo) v = rec[v];
-    std::sort(t.halo.begin(), t.halo.end());
+    std::sort(t.halo.begin(), t.halo.end());  // the owners' order, but for the swaps inside octets
     std::vector<int32_t> vert(d.own);
     for (int64_t r = cut[q]; r < cut[q + 1]; ++r) vert[rec[order[r]] - d.lo] = order[r];
     std::vector<std::pair<int32_t, int32_t>> hpos(d.nh);  // record, position
@@ -244,6 +394,33 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
       return (int32_t)(std::lower_bound(hpos.begin(), hpos.end(), std::make_pair(r, (int32_t)-1)) - hpos.begin());
     };
     auto pos_of = [&](int32_t o) { return part_of[o] == q ? rec[o] - d.lo : hpos[halo_index(rec[o])].second; };
+    if (d.nh > 0) {  // residues of the halo, the own positions standing
+      std::vector<int32_t> cnt(((size_t)d.own + 8) / 8 * 8, 0), hp(d.nh + 1, 0), readers, index(d.nh), seen;
+      for (int32_t i = 0; i < d.nh; ++i) index[i] = i;  // halo position -> entry of hpos
+      std::vector<std::pair<int32_t, int32_t>> rd;
+      for (int32_t p = 0; p < d.own; ++p)
+        for (int32_t j = ptr[vert[p]]; j < ptr[vert[p] + 1]; ++j) {
+          const int32_t o = nb[j];
+          if (part_of[o] != q) rd.push_back({halo_index(rec[o]), p});
+          ++cnt[(p >> 3) * 8 + (pos_of(o) & 7)];
+        }
+      std::sort(rd.begin(), rd.end());
+      for (auto& x : rd) ++hp[x.first + 1], readers.push_back(x.second);
+      for (int32_t i = 0; i < d.nh; ++i) hp[i + 1] += hp[i];
+      even_residues(
+          d.hbase & ~7, d.hbase + d.nh, d.hbase, cnt,
+          [&](int32_t p) -> const std::vector<int32_t>& {
+            seen.clear();
+            if (p >= d.hbase) seen.assign(readers.begin() + hp[index[p - d.hbase]], readers.begin() + hp[index[p - d.hbase] + 1]);
+            return seen;
+          },
+          [&](int32_t i, int32_t j) {
+            const int32_t a = index[i - d.hbase], b = index[j - d.hbase];
+            std::swap(index[i - d.hbase], index[j - d.hbase]);
+            hpos[a].second = j, hpos[b].second = i;
+          });
+      for (int32_t i = 0; i < d.nh; ++i) t.halo[i] = hpos[index[i]].first;
+    }
     const int32_t W = L.warps;
     std::vector<int32_t> kcol(d.nsl), c0(d.nsl);
     for (int32_t j = 0; j < d.nsl; ++j)
@@ -263,6 +440,7 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
     t.ent.assign((size_t)cols * 32, 0);
     t.wmap.assign((size_t)cols * 64, -1);
     std::vector<Entry> ents;
+    OctetColumns oc;
     for (int32_t j = 0; j < d.nsl; ++j) {
       int32_t lo[32], hi[32];
       ents.clear();
@@ -276,7 +454,7 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
           }
         hi[l] = (int32_t)ents.size();
       }
-      spread_slice(ents, lo, hi, 32 * j, 2 * kcol[j], [&](int32_t c, int l, int32_t o, const Entry* x) {
+      spread_slice(ents, lo, hi, 32 * j, 2 * kcol[j], oc, [&](int32_t c, int l, int32_t o, const Entry* x) {
         const size_t at = (size_t)32 * (c0[j] + c / 2) + l;
         const uint32_t v = (uint32_t)o | (x && x->src ? kSlotSrc : 0u);
         t.ent[at] |= v << (16 * (c & 1));
