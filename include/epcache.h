@@ -317,13 +317,15 @@ int ep_finish(ep_schedule *s, int32_t D, float *x_lay, float tau, void *stream);
  * SpMV in schedule layout (bipartite schedules, Section 5.2): y_lay = A x_lay
  * with x_lay over column records and y_lay over row records (n floats each,
  * ep_spmv_x_in / ep_spmv_y_out permute), w_lay from ep_weights_in.  One
- * warp per schedule block: the block's x entries are staged in shared memory
- * (the software cache), its row-ranked entries are split into equal chunks,
- * one per lane, whatever the row lengths, and rows that cross chunk ends are
- * joined by a segmented scan over the warp.  Rows used by one block are
- * stored, rows shared by blocks accumulated with atomics after zeroing.
- * Buffers 16-byte aligned (EP_EINVAL otherwise); EP_EINVAL when one warp's
- * staged x and row totals of the largest block do not fit in shared memory.
+ * warp per schedule block at a time: its row-ranked entries are split into equal
+ * chunks, one per lane, whatever the row lengths, and rows that cross chunk
+ * ends are joined by a segmented scan over the warp.  x records are ordered by
+ * how many blocks use the column; on large matrices the most used ones are kept
+ * in shared memory (the software cache), the others are read at the entry.
+ * Rows used by one block are stored, rows shared by blocks accumulated with
+ * atomics after zeroing.  Buffers 16-byte aligned (EP_EINVAL otherwise);
+ * EP_EINVAL when one warp's row totals of the largest block do not fit in
+ * shared memory.
  */
 int ep_spmv_x_in(ep_schedule *s, const float *x, float *x_lay, void *stream);
 int ep_spmv_y_out(ep_schedule *s, const float *y_lay, float *y, void *stream);
@@ -413,7 +415,8 @@ int ep_timing_read(ep_schedule *s, int32_t kernel_class, double *total_ms, int64
 
 /* No counterpart in the paper (launch tuning): threads that compute per CUDA
  * block in the forward flux and SpMV kernels (32..1024, multiple of 32;
- * default 192), and in the adjoint flux kernels (default 352: the adjoint
+ * default 192; the SpMV kernel uses at most 256, and as many as it needs where
+ * it keeps columns in shared memory), and in the adjoint flux kernels (default 352: the adjoint
  * stages twice the state per kernel block and does about twice the arithmetic
  * per task, so fewer CUDA blocks fit an SM and each wants more warps).
  * EP_EINVAL for a count out of range.  Does not change results beyond FP32
@@ -485,7 +488,8 @@ int ep_check_errors(ep_schedule *s, int32_t *code, void *stream);
  * Where the forward flux and SpMV kernels read a block's data from (the
  * study of Section 5, Fig. 11 and Table 3: texture cache vs software cache).
  * EP_CACHE_SMEM (default): staged into shared memory (the flux kernels
- * chosen by ep_set_pipeline; SpMV stages x).  EP_CACHE_L1: nothing staged;
+ * chosen by ep_set_pipeline; SpMV keeps the most used columns of large
+ * matrices).  EP_CACHE_L1: nothing staged;
  * every read goes through the read-only data cache (ld.global.nc, which
  * replaces the texture binding of the paper's GPUs).  Flux: one CUDA block
  * per schedule block, one thread per vertex position (up to 4 per thread).

@@ -138,8 +138,7 @@ struct ep_schedule {
   int tpb_adj = 352;  // consumer threads of the adjoint kernels
   bool bacc_dirty = true;
   // device copy of the schedule
-  DBuf d_desc, d_flist, d_ylist, d_ent, d_wmap, d_rec, d_xrec, d_yrec, d_bptr, d_eu,
-      d_ev;
+  DBuf d_desc, d_ylist, d_ent, d_row0, d_wmap, d_rec, d_xrec, d_yrec, d_yrow, d_bptr, d_eu, d_ev;
   DBuf d_sidx, d_soff, d_sid, d_gslot, d_frec, d_fsid;  // flux layout
   // workspace
   DBuf ws_x, ws_out, ws_w, ws_bacc, ws_lam, ws_gw, ws_hist, ws_flags, ws_cnt;
@@ -214,9 +213,20 @@ int ensure_device(ep_schedule* s) {
   const ep::HostSchedule& h = s->h;
   if (bipartite(s)) {
     CU(upload(s->d_desc, h.sdesc));
-    CU(upload(s->d_flist, h.xlist));
     CU(upload(s->d_ylist, h.ylist));
-    CU(upload(s->d_ent, h.sent));
+    {
+      DBuf sent, xlist;
+      CU(upload(sent, h.sent));
+      CU(upload(xlist, h.xlist));
+      CU(s->d_ent.ensure(h.sent.size() * sizeof(uint32_t)));
+      CU(s->d_row0.ensure(32 * (size_t)h.k * sizeof(uint16_t)));
+      CU(ep::dev::spmv_entries(s->d_desc.as<ep::SpmvDesc>(), h.k, sent.as<uint32_t>(), xlist.as<int32_t>(),
+                               s->d_ent.as<uint32_t>(), s->d_row0.as<uint16_t>(), nullptr));
+      CU(cudaStreamSynchronize(nullptr));
+    }
+    std::vector<int32_t> yrow(h.n);
+    for (int64_t i = 0; i < h.n; ++i) yrow[h.yrec_of[i]] = (int32_t)i;
+    CU(upload(s->d_yrow, yrow));
     CU(upload(s->d_wmap, h.wmap));
     CU(upload(s->d_xrec, h.xrec_of));
     CU(upload(s->d_yrec, h.yrec_of));
@@ -629,35 +639,29 @@ int check_flux(ep_schedule* s, int32_t D) {
   return EP_OK;
 }
 
-// SpMV kernel on schedule-layout buffers
-int spmv_lay(ep_schedule* s, const float* x_lay, const float* w_lay, float* y_lay, cudaStream_t st) {
+// SpMV kernel: x records, weights in schedule layout, y records; or (direct)
+// weights in task order and y in the caller's row order.
+int spmv_lay(ep_schedule* s, const float* x_lay, const float* w, float* y, bool direct, cudaStream_t st) {
   const ep::HostSchedule& h = s->h;
   ep::dev::SpmvArgs a;
   a.desc = s->d_desc.as<ep::SpmvDesc>();
   a.k = h.k;
-  a.xlist = s->d_flist.as<int32_t>();
   a.ylist = s->d_ylist.as<int32_t>();
   a.ent = s->d_ent.as<uint32_t>();
-  a.w = w_lay;
+  a.row0 = s->d_row0.as<uint16_t>();
+  a.w = w;
+  a.wmap = direct ? wmap_of(s) : nullptr;
   a.x = x_lay;
-  a.y = y_lay;
+  a.y = y;
+  a.yrow = direct ? s->d_yrow.as<int32_t>() : nullptr;
+  a.n = h.n;
   a.ny_int = h.ny_int;
   a.ny_zero = h.n - h.ny_int;
-  a.max_nx = h.max_nx;
   a.max_ny = h.max_ny;
-  a.max_nxy = h.max_nxy;
   a.u = h.spmv_u;
   a.tpb = s->tpb;
   a.readonly = s->cache == EP_CACHE_L1;
   a.timer = s->t();
-  int dev = 0, optin = 0;
-  CU(cudaGetDevice(&dev));
-  CU(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  const ep::dev::SpmvPlan P = ep::dev::spmv_plan(a, optin);
-  if (P.wpb == 0)
-    return fail(EP_EINVAL,
-                "a schedule block needs %zu bytes of shared memory (limit %d): use a smaller C",
-                P.smem, optin - 1024);
   CU(ep::dev::spmv(a, st));
   return EP_OK;
 }
@@ -686,10 +690,15 @@ int run_spmv(ep_schedule* s, const float* x, const float* w, float* y, cudaStrea
              bool from_host = false) {
   const ep::HostSchedule& h = s->h;
   CU(s->ws_x.ensure((size_t)h.n * sizeof(float)));
-  CU(s->ws_out.ensure((size_t)h.n * sizeof(float)));
   CU(ep::dev::layout_in(s->d_xrec.as<int32_t>(), h.n, h.n, 1, x, s->ws_x.as<float>(), st, s->t()));
+  // device buffers: weights read through the slot map and rows written in the
+  // caller's order by the kernel itself (2^18 rows, partitioned: the gather of
+  // 4M weights beforehand took 18 us, the copy of y 4, the kernel 24)
+  const bool apart = y + h.n <= w || w + h.m <= y;  // weights are read while rows are written
+  if (!from_host && apart) return spmv_lay(s, s->ws_x.as<float>(), w, y, true, st);
+  CU(s->ws_out.ensure((size_t)h.n * sizeof(float)));
   if (int rc = weights_to_ws(s, w, from_host, st)) return rc;
-  if (int rc = spmv_lay(s, s->ws_x.as<float>(), s->ws_w.as<float>(), s->ws_out.as<float>(), st))
+  if (int rc = spmv_lay(s, s->ws_x.as<float>(), s->ws_w.as<float>(), s->ws_out.as<float>(), false, st))
     return rc;
   CU(ep::dev::layout_out(s->d_yrec.as<int32_t>(), h.n, h.n, 1, s->ws_out.as<float>(), y, st, s->t()));
   return EP_OK;
@@ -1599,7 +1608,7 @@ int ep_spmv(ep_schedule* s, const float* x_lay, const float* w_lay, float* y_lay
   if (!x_lay || !w_lay || !y_lay) return fail(EP_EINVAL, "null argument");
   if (misaligned(x_lay) || misaligned(w_lay) || misaligned(y_lay))
     return fail(EP_EINVAL, "schedule-layout buffers must be 16-byte aligned");
-  return spmv_lay(s, x_lay, w_lay, y_lay, as_stream(stream));
+  return spmv_lay(s, x_lay, w_lay, y_lay, false, as_stream(stream));
 }
 
 int ep_set_pipeline(ep_schedule* s, int32_t stages) {

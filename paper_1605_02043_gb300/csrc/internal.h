@@ -50,9 +50,12 @@ constexpr int32_t kSidMask = 0x7fffffff;
 // SpMV entry fields: (row position << 16) | x position
 constexpr int kRowShift = 16;
 constexpr uint32_t kColMask = 0xffffu;
+constexpr uint32_t kEntRow = 1u;  // device entries: 4 * x record, plus 1 on the first entry of a row
 
 // SpMV kernels (bipartite): x records are read only, y records accumulate.
-// x positions: [0, n_xo) the run x_lo.., then n_xf ids from xlist[fx0..].
+// x positions: [0, n_xo) the run x_lo.., then n_xf ids from xlist[fx0..]; the x
+// records are ordered by how many blocks use them, so the run is empty (n_xo =
+// 0) and every position is listed.
 // y positions: [0, n_yi) the single-block rows yi_lo.., [n_yi, n_yi + n_yob)
 // the run yb_lo.. of shared rows first touched here, then n_yf ids from
 // ylist[fy0..]; within each class rows are ordered by descending list length.
@@ -70,6 +73,9 @@ struct SpmvDesc {
 };
 static_assert(sizeof(SpmvDesc) == 64, "SpmvDesc layout");
 // slot (from i0) of the entry ranked t in row order, u entries per lane
+#ifdef __CUDACC__
+__host__ __device__
+#endif
 inline int32_t spmv_slot(int32_t t, int32_t u) {
   const int32_t lane = t / u, j = t % u;
   return ((j >> 2) * 32 + lane) * 4 + (j & 3);

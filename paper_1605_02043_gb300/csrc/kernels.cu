@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include <climits>
+#include <cstddef>
 #include <cstdint>
 #include <mutex>
 #include <unordered_set>
@@ -19,6 +20,7 @@
 #include "block_distinct.cuh"
 #include "flux_common.cuh"
 #include "kernels.h"
+#include "tma_sync.cuh"
 
 namespace ep {
 namespace dev {
@@ -186,117 +188,74 @@ __global__ void __launch_bounds__(1024) flux_adj_kernel(const FluxArgs a, float*
 
 // --------------------------------------------------------------------- SpMV
 
-// SpMV over the edge partition (Section 5.2), one warp per schedule block.
-// The block's entries are ranked by row position and cut into 32 equal
-// chunks, one per lane, so every lane does the same work whatever the row
-// lengths: a lane walks its chunk in order, summing runs of equal rows in a
-// register.  A run that neither starts nor ends the chunk is a whole row and
-// is stored at once; the first and last runs of the chunks are joined across
-// lanes by a segmented scan over the warp.  Row totals go to a shared array
-// and leave it in row order (plain stores for rows of this block alone,
-// atomics for shared rows).  With the software cache, x of the block's
-// columns is staged in shared memory first; the read-only-cache variant
-// reads x through the read-only data cache at every entry.
+// SpMV over the edge partition (Section 5.2), one warp per schedule block at
+// a time.  The block's entries are ranked by row position and cut into 32
+// equal chunks, one per lane, so every lane does the same work whatever the
+// row lengths: a lane walks its chunk in order, summing runs of equal rows in a
+// register.  A run that neither starts nor ends the chunk is a whole row and is
+// stored at once; the first and last runs of the chunks are joined across lanes
+// by a segmented scan over the warp.  Row totals go to a shared array and leave
+// it in row order (plain stores for rows of this block alone, atomics for
+// shared rows).
 //
-// Per-warp shared region: y totals at [0, ceil4(ny)), staged x after them.
+// The software cache (HOT): x records are ordered by how many blocks use the
+// column, and one persistent CUDA block per SM keeps the kSpmvHot most used ones
+// beside the row totals.  On power-law matrices most entries name one of those;
+// the others are read at the entry, through the L1 that is left: all of shared
+// memory for columns (about 45,000) leaves none, and R-MAT scale 20 in CSR order
+// takes 51.5 us instead of 44.0 (1,024 columns: 49.7; 8,192: 47.9), scale 18
+// partitioned 53 instead of 31.5.  Staging each block's own distinct columns, as
+// before, read an id and a 32-byte sector per column and block, with next to no
+// reuse inside a block of 512 tasks: 73.7 us at scale 20, of which staging was
+// 39.  Bound now by latency (the join and the write-out of one block follow its
+// entries; 24 warps per SM, 80 registers), at 2.2 times the time its 143 MB
+// take at 6.8 TB/s.
 constexpr int kSpmvBatch = 4;  // 16-byte chunks of entries (and weights) in flight per lane
-constexpr int kSpmvMaxThreads = 256;
+constexpr int kSpmvMaxThreads = 768;
+constexpr int64_t kSpmvHotBlocks = 24;
+constexpr int64_t kSpmvHot = 24576;
 
-__device__ __forceinline__ int spmv_up4(int v) { return (v + 3) & ~3; }
+__host__ __device__ constexpr int spmv_up4(int v) { return (v + 3) & ~3; }
 
-template <bool STAGE>
-__device__ __forceinline__ float spmv_x(const SpmvDesc& d, const int32_t* __restrict__ xlist,
-                                        const float* __restrict__ x, const float* xs, uint32_t col) {
-  if (STAGE) return xs[col];
-  const int c = (int)col;
-  return __ldg(x + (c < d.n_xo ? d.x_lo + c : __ldg(xlist + d.fx0 + (c - d.n_xo))));
+// x at byte offset `off` of the records: from the kept prefix or from memory.
+// The two loads go to registers of their own (one register for both makes the
+// second wait for the first), each lane making the one it needs; set to 0
+// first, or a register that some lanes leave alone stays live around the loop.
+template <bool HOT>
+__device__ __forceinline__ float spmv_x(const float* __restrict__ x, uint32_t hot_at, uint32_t hot4, uint32_t off) {
+  const float* p = reinterpret_cast<const float*>(reinterpret_cast<const char*>(x) + off);
+  if (!HOT) return __ldg(p);
+  float kept, cold;
+  asm volatile("{\n\t.reg .pred p;\n\tmov.f32 %0, 0f00000000;\n\tsetp.lt.u32 p, %1, %2;\n\t@p ld.shared.f32 %0, [%3];\n\t}"
+      : "=&f"(kept)
+      : "r"(off), "r"(hot4), "r"(hot_at + off));
+  asm volatile("{\n\t.reg .pred p;\n\tmov.f32 %0, 0f00000000;\n\tsetp.ge.u32 p, %1, %2;\n\t@p ld.global.nc.f32 %0, [%3];\n\t}"
+      : "=&f"(cold)
+      : "r"(off), "r"(hot4), "l"(p));
+  return off < hot4 ? kept : cold;
 }
 
-// x of the block's columns into xs: four (id, value) load chains in flight
-// per lane
-__device__ __forceinline__ void spmv_stage_x(const SpmvDesc& d, const SpmvArgs& a, float* xs, int lane) {
-  const int nx = d.n_xo + d.n_xf;
-  for (int i0 = lane; i0 < nx; i0 += 4 * 32) {
-    int32_t r[4];
+__device__ __forceinline__ uint32_t word(const uint4& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
+
+// chunks c of this lane, c0 <= c < c0 + kSpmvBatch: entries and weights (or the
+// tasks whose weights they are), read once and not kept in the caches
+template <bool MAP>
+__device__ __forceinline__ void spmv_load(const SpmvArgs& a, int64_t i0, int lane, int c0, uint4* ev, uint4* wv) {
+  const uint4* ep = reinterpret_cast<const uint4*>(a.ent + i0) + lane;
+  const uint4* wp = (MAP ? reinterpret_cast<const uint4*>(a.wmap + i0) : reinterpret_cast<const uint4*>(a.w + i0)) + lane;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int i = i0 + 32 * u;
-      r[u] = i >= nx ? -1 : (i < d.n_xo ? d.x_lo + i : __ldg(a.xlist + d.fx0 + (i - d.n_xo)));
+  for (int c = 0; c < kSpmvBatch; ++c)
+    if (4 * (c0 + c) < a.u) {
+      ev[c] = __ldcs(ep + 32 * (c0 + c));
+      wv[c] = __ldcs(wp + 32 * (c0 + c));
     }
-    float v[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) v[u] = r[u] >= 0 ? __ldg(a.x + r[u]) : 0.f;
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-      if (r[u] >= 0) xs[i0 + 32 * u] = v[u];
-  }
-}
-
-struct SpmvRun {
-  int cur = -1, hrow = -1;  // row of the open run; row of the chunk's first run once closed
-  float acc = 0.f, hsum = 0.f;
-  bool whole = true;  // no run closed yet: the chunk is one run so far
-};
-
-__device__ __forceinline__ void spmv_take(SpmvRun& r, float* ys, uint32_t e, float v) {
-  const int row = (int)(e >> kRowShift);
-  if (row != r.cur) {
-    if (r.cur >= 0) {
-      if (r.whole) {
-        r.hrow = r.cur;
-        r.hsum = r.acc;
-        r.whole = false;
-      } else {
-        ys[r.cur] = r.acc;  // a run inside the chunk: the whole row
-      }
-    }
-    r.cur = row;
-    r.acc = v;
-  } else {
-    r.acc += v;
-  }
-}
-
-// Four entries (one 16-byte chunk) of this lane; j: their rank in the chunk
-template <bool STAGE>
-__device__ __forceinline__ void spmv_chunk(SpmvRun& run, float* ys, const float* xs, const SpmvDesc& d,
-                                           const SpmvArgs& a, uint4 ev, float4 wv, int j, int nj) {
-  const uint32_t e[4] = {ev.x, ev.y, ev.z, ev.w};
-  const float w[4] = {wv.x, wv.y, wv.z, wv.w};
-#pragma unroll
-  for (int q = 0; q < 4; ++q)
-    if (j + q < nj) spmv_take(run, ys, e[q], w[q] * spmv_x<STAGE>(d, a.xlist, a.x, xs, e[q] & kColMask));
-}
-
-// Joins the chunks' end runs: lane l's first run continues lane l-1's last
-// run when both are the same row, and a lane whose chunk is one run passes
-// the sum on (segmented inclusive scan of the last-run sums over the lanes).
-// Afterwards every row of the block has its total in ys, stored once.
-__device__ __forceinline__ void spmv_join(const SpmvRun& run, float* ys, int lane) {
-  const unsigned full = 0xffffffffu;
-  const int rt = run.cur, rh = run.whole ? run.cur : run.hrow;
-  const int rt_prev = __shfl_up_sync(full, rt, 1);
-  const bool cont = lane > 0 && rh >= 0 && rh == rt_prev;
-  float S = run.acc;
-  int F = !(run.whole && cont);  // a segment starts here
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const float Sp = __shfl_up_sync(full, S, o);
-    const int Fp = __shfl_up_sync(full, F, o);
-    if (lane >= o && !F) {
-      S += Sp;
-      F = Fp;
-    }
-  }
-  const float S_prev = __shfl_up_sync(full, S, 1);
-  const int cont_next = __shfl_down_sync(full, (int)cont, 1);
-  if (!run.whole) ys[rh] = run.hsum + (cont ? S_prev : 0.f);
-  if (rt >= 0 && !(lane < 31 && cont_next)) ys[rt] = S;
 }
 
 // Row totals out: four rows in flight per lane
-__device__ __forceinline__ void spmv_write_out(const SpmvDesc& d, const SpmvArgs& a, const float* ys,
-                                               int lane) {
+struct SpmvRows {
+  int yi_lo, n_yi, yb_lo, n_yob, fy0, n_yf;
+};
+__device__ __forceinline__ void spmv_write_out(const SpmvRows& d, const SpmvArgs& a, const float* ys, int lane) {
   const int ny = d.n_yi + d.n_yob + d.n_yf, own = d.n_yi + d.n_yob;
   for (int p0 = lane; p0 < ny; p0 += 4 * 32) {
     int32_t r[4];
@@ -307,6 +266,11 @@ __device__ __forceinline__ void spmv_write_out(const SpmvDesc& d, const SpmvArgs
                      : (p < d.n_yi ? d.yi_lo + p
                                    : (p < own ? d.yb_lo + (p - d.n_yi)
                                               : __ldg(a.ylist + d.fy0 + (p - own))));
+    }
+    if (a.yrow) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (r[u] >= 0) r[u] = __ldg(a.yrow + r[u]);
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
@@ -320,49 +284,149 @@ __device__ __forceinline__ void spmv_write_out(const SpmvDesc& d, const SpmvArgs
   }
 }
 
-// One warp per schedule block (one pass, no pipeline): the lane's entries and
-// weights are loaded straight into registers while x is staged.
-template <bool STAGE>
-__global__ void __launch_bounds__(kSpmvMaxThreads) spmv_kernel(const SpmvArgs a, int wpb, int cap) {
+template <bool HOT, bool MAP>
+__global__ void __launch_bounds__(HOT ? kSpmvMaxThreads : 256, HOT ? 1 : 3) spmv_kernel(const SpmvArgs a, int cap, int hot) {
   extern __shared__ float4 smem4[];
-  const int wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t b = (int64_t)blockIdx.x * wpb + wi;
-  if (b >= a.k) return;  // warp-uniform; the warps of a CUDA block never synchronise
-  const SpmvDesc d = a.desc[b];
-  float* ys = reinterpret_cast<float*>(smem4) + (size_t)wi * cap;
-  float* xs = ys + spmv_up4(d.n_yi + d.n_yob + d.n_yf);
-  const int nj = min(max(d.ne - lane * d.u, 0), d.u);  // this lane's real entries
-  // chunk c of this lane: slots i0 + (32 c + lane) * 4 .. + 3
-  const uint4* ep = reinterpret_cast<const uint4*>(a.ent + d.i0) + lane;
-  const float4* wp = reinterpret_cast<const float4*>(a.w + d.i0) + lane;
-  uint4 ev[kSpmvBatch];
-  float4 wv[kSpmvBatch];
-#pragma unroll
-  for (int c = 0; c < kSpmvBatch; ++c)
-    if (4 * c < nj) {
-      ev[c] = __ldg(ep + 32 * c);
-      wv[c] = __ldg(wp + 32 * c);
+  __shared__ __align__(8) uint64_t bar;
+  const int wi = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  float* xs = reinterpret_cast<float*>(smem4);
+  float* ys = xs + (HOT ? hot : 0) + (size_t)wi * cap;
+  if (HOT) {
+    if (threadIdx.x == 0) {
+      mbar_init(&bar, 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      mbar_arrive_tx(&bar, 4u * hot);
+      bulk_load(xs, a.x, 4u * hot, &bar);
     }
-  if (STAGE) {
-    spmv_stage_x(d, a, xs, lane);
+    __syncthreads();
+  }
+  const uint32_t hot_at = HOT ? saddr(xs) : 0;
+  uint32_t hot4 = 4u * hot;
+  const int64_t stride = (int64_t)gridDim.x * nw;
+  int64_t b = (int64_t)blockIdx.x * nw + wi;
+  if (b >= a.k) return;  // warp-uniform; the warps do not synchronise from here on
+  uint4 ev[kSpmvBatch], wv[kSpmvBatch];
+  spmv_load<MAP>(a, 32 * (int64_t)a.u * b, lane, 0, ev, wv);
+  if (HOT) {  // the entries are in flight; a copy that does not land costs speed only
+    if (!mbar_wait(&bar, 0)) hot4 = 0;
+  }
+  // the descriptor as one word per lane (lane f holds word f), read a block
+  // ahead like the row positions of the lanes' first entries
+  const unsigned full = 0xffffffffu;
+  auto word_of = [&](int64_t blk) { return __ldg(reinterpret_cast<const int*>(a.desc + blk) + (lane & 15)); };
+  int next_word = word_of(b), next_row = __ldg(a.row0 + 32 * b + lane);
+  for (; b < a.k; b += stride) {
+    const int dw = next_word, row = next_row;
+    if (b + stride < a.k) {
+      next_word = word_of(b + stride);
+      next_row = __ldg(a.row0 + 32 * (b + stride) + lane);
+    }
+    const int ne = __shfl_sync(full, dw, offsetof(SpmvDesc, ne) / 4);
+    SpmvRows d;
+    d.fy0 = __shfl_sync(full, dw, offsetof(SpmvDesc, fy0) / 4);
+    d.n_yf = __shfl_sync(full, dw, offsetof(SpmvDesc, n_yf) / 4);
+    if (32 * lane < d.n_yf) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.ylist + d.fy0 + 32 * lane));
+    const int64_t i0 = 32 * (int64_t)a.u * b;
+    const int nj = min(max(ne - lane * a.u, 0), a.u);  // this lane's real entries
+    const bool cont = lane > 0 && nj > 0 && !(ev[0].x & kEntRow);  // which the lane before began
+    ev[0].x &= ~kEntRow;
+    // the next block's lines into the L2: the loads below then miss only the L1
+    if (b + stride < a.k && a.u == 4 * kSpmvBatch) {
+      const char* next = lane < 16 ? reinterpret_cast<const char*>(a.ent + i0 + 32 * (int64_t)a.u * stride)
+                                   : (MAP ? reinterpret_cast<const char*>(a.wmap + i0 + 32 * (int64_t)a.u * stride)
+                                          : reinterpret_cast<const char*>(a.w + i0 + 32 * (int64_t)a.u * stride));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(next + 128 * (lane & 15)));
+    }
+    // A run that ends inside the chunk goes to its row's total as it stands
+    // (the first one may still lack what the lanes before summed).
+    float acc = 0.f;
+    float* at = ys + row;
+    auto batch = [&](int c0, bool whole) {
+#pragma unroll
+      for (int h = 0; h < kSpmvBatch; h += 2) {  // eight entries' loads in flight, then their sums
+        float v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const uint32_t e = word(ev[h + (i >> 2)], i & 3), w = word(wv[h + (i >> 2)], i & 3);
+          if (whole || 4 * (c0 + h) + i < nj) {
+            const float wt = MAP ? __ldg(a.w + w) : __uint_as_float(w);
+            v[i] = wt * spmv_x<HOT>(a.x, hot_at, hot4, e & ~kEntRow);
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (whole || 4 * (c0 + h) + i < nj) {
+            if (word(ev[h + (i >> 2)], i & 3) & kEntRow) {
+              *at++ = acc;
+              acc = 0.f;
+            }
+            acc += v[i];
+          }
+      }
+    };
+    for (int c0 = 0; 4 * c0 < a.u; c0 += kSpmvBatch) {
+      if (c0 > 0) spmv_load<MAP>(a, i0, lane, c0, ev, wv);
+      if (ne - 31 * a.u >= 4 * (c0 + kSpmvBatch))  // every lane's batch is full
+        batch(c0, true);
+      else
+        batch(c0, false);
+    }
+    const bool whole = at == ys + row;  // the chunk is one run
+    // the next block's entries, in flight during the join and the write-out
+    if (b + stride < a.k) spmv_load<MAP>(a, i0 + 32 * (int64_t)a.u * stride, lane, 0, ev, wv);
+    // Joins the chunks' end runs: a lane's first run continues the lane
+    // before's last run (cont), and a lane whose chunk is one run passes the
+    // sum on (segmented inclusive scan of the last-run sums over the lanes).
+    // Afterwards every row of the block has its total in ys, stored once.
+    float S = acc;
+    int F = !(whole && cont);  // a segment starts here
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const float Sp = __shfl_up_sync(full, S, o);
+      const int Fp = __shfl_up_sync(full, F, o);
+      if (lane >= o && !F) {
+        S += Sp;
+        F = Fp;
+      }
+    }
+    const float S_prev = __shfl_up_sync(full, S, 1);
+    const int cont_next = __shfl_down_sync(full, (int)cont, 1);
+    if (!whole && cont) ys[row] += S_prev;
+    if (nj > 0 && !(lane < 31 && cont_next)) *at = S;
+    __syncwarp();
+    d.yi_lo = __shfl_sync(full, dw, offsetof(SpmvDesc, yi_lo) / 4);
+    d.n_yi = __shfl_sync(full, dw, offsetof(SpmvDesc, n_yi) / 4);
+    d.yb_lo = __shfl_sync(full, dw, offsetof(SpmvDesc, yb_lo) / 4);
+    d.n_yob = __shfl_sync(full, dw, offsetof(SpmvDesc, n_yob) / 4);
+    spmv_write_out(d, a, ys, lane);
     __syncwarp();
   }
-  SpmvRun run;
-  for (int c0 = 0; 4 * c0 < nj; c0 += kSpmvBatch) {
-    if (c0 > 0) {
-#pragma unroll
-      for (int c = 0; c < kSpmvBatch; ++c)
-        if (4 * (c0 + c) < nj) {
-          ev[c] = __ldg(ep + 32 * (c0 + c));
-          wv[c] = __ldg(wp + 32 * (c0 + c));
-        }
+}
+
+// Device entries of a schedule: one warp per block
+__global__ void spmv_entries_kernel(const SpmvDesc* __restrict__ desc, int64_t k, const uint32_t* __restrict__ sent,
+                                    const int32_t* __restrict__ xlist, uint32_t* __restrict__ ent,
+                                    uint16_t* __restrict__ row0) {
+  const int lane = threadIdx.x & 31;
+  const int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  if (b >= k) return;
+  const SpmvDesc d = desc[b];
+  const uint32_t* src = sent + d.i0;
+  uint32_t* dst = ent + d.i0;
+  for (int t = lane; t < 32 * d.u; t += 32) {
+    const int j = spmv_slot(t, d.u);
+    uint32_t v = 0;
+    if (t < d.ne) {
+      const uint32_t e = src[j], row = e >> kRowShift;
+      const int col = (int)(e & kColMask);
+      v = 4u * (uint32_t)(col < d.n_xo ? d.x_lo + col : xlist[d.fx0 + col - d.n_xo]);
+      if (t == 0 || src[spmv_slot(t - 1, d.u)] >> kRowShift != row) v |= kEntRow;
+      if (t % d.u == 0) row0[32 * b + t / d.u] = (uint16_t)row;
+    } else if (t % d.u == 0) {
+      row0[32 * b + t / d.u] = 0;
     }
-#pragma unroll
-    for (int c = 0; c < kSpmvBatch; ++c) spmv_chunk<STAGE>(run, ys, xs, d, a, ev[c], wv[c], 4 * (c0 + c), nj);
+    dst[j] = v;
   }
-  spmv_join(run, ys, lane);
-  __syncwarp();
-  spmv_write_out(d, a, ys, lane);
 }
 
 // ------------------------------------------------------------- shard halo
@@ -711,37 +775,62 @@ size_t flux_block_smem(const FluxArgs& a, int D, bool adjoint) {
   return (size_t)tma_layout(a, D, adjoint).stage_bytes;
 }
 
-SpmvPlan spmv_plan(const SpmvArgs& a, int smem_optin) {
+SpmvPlan spmv_plan(const SpmvArgs& a, int smem_optin, int sms) {
   SpmvPlan P = {};
-  int wpb = std::max(1, std::min(kSpmvMaxThreads / 32, a.tpb / 32));
-  P.cap = a.readonly ? (a.max_ny + 3) & ~3 : a.max_nxy;
-  const size_t per_warp = (size_t)P.cap * sizeof(float);
+  P.cap = spmv_up4(a.max_ny);
+  const size_t per_warp = (size_t)P.cap * sizeof(float), limit = (size_t)smem_optin - 1024;
+  if (per_warp > limit) return P;
+  // Columns are kept where an SM has at least kSpmvHotBlocks blocks of 512
+  // entries to share them.  Kept against not, us: scale 17 (25 blocks an SM)
+  // partitioned 15.5 / 16.1, CSR 13.9 / 13.6; scale 16 (12) 11.3 / 11.3 and
+  // 10.1 / 9.5; scale 15 (6) 9.6 / 9.2 and 10.3 / 9.1; scale 18 31.5 / 39.
+  // The SM's blocks are dealt to up to 24 warps in rounds of equal size.
+  const int64_t per_sm = (a.k + sms - 1) / sms;
+  if (!a.readonly && per_sm * a.u >= 16 * kSpmvHotBlocks) {
+    const int most = (int)std::min<int64_t>(kSpmvMaxThreads / 32, std::max<int64_t>(1, (int64_t)(limit / 2 / per_warp)));
+    const int64_t rounds = (per_sm + most - 1) / most;
+    P.wpb = (int)((per_sm + rounds - 1) / rounds);
+    P.grid = std::min<int64_t>(sms, (a.k + P.wpb - 1) / P.wpb);
+    P.hot = (int)std::min<int64_t>(std::min<int64_t>(a.n + 3, kSpmvHot) / 4 * 4, (int64_t)((limit - P.wpb * per_warp) / 16 * 4));
+    if (P.hot > a.n) P.hot = (int)(a.n / 4 * 4);  // whole 16-byte pieces of x
+    P.smem = P.wpb * per_warp + (size_t)P.hot * sizeof(float);
+    return P;
+  }
+  int wpb = std::max(1, std::min(8, a.tpb / 32));
   while (wpb > 1 && per_warp * wpb > (size_t)48 * 1024) --wpb;  // room for several CUDA blocks per SM
+  P.wpb = wpb;
+  P.grid = (a.k + wpb - 1) / wpb;
   P.smem = per_warp * wpb;
-  P.wpb = P.smem + 1024 <= (size_t)smem_optin ? wpb : 0;
   return P;
 }
 
 cudaError_t spmv(const SpmvArgs& a, cudaStream_t st) {
-  int dev = 0, optin = 0;
+  int dev = 0, optin = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  const SpmvPlan P = spmv_plan(a, optin);
+  const SpmvPlan P = spmv_plan(a, optin, sms);
   if (P.wpb == 0) return cudaErrorInvalidValue;
-  e = a.readonly ? allow_smem(spmv_kernel<false>, P.smem) : allow_smem(spmv_kernel<true>, P.smem);
-  if (e != cudaSuccess) return e;
-  if (a.ny_zero > 0) {
+  using Kernel = void (*)(const SpmvArgs, int, int);
+  const Kernel kern = P.hot ? (a.wmap ? (Kernel)spmv_kernel<true, true> : (Kernel)spmv_kernel<true, false>)
+                            : (a.wmap ? (Kernel)spmv_kernel<false, true> : (Kernel)spmv_kernel<false, false>);
+  if ((e = allow_smem(kern, P.smem)) != cudaSuccess) return e;
+  // rows that several blocks add to (all rows, where records are not in order)
+  if (a.yrow)
+    e = cudaMemsetAsync(a.y, 0, (size_t)a.n * sizeof(float), st);
+  else if (a.ny_zero > 0)
     e = cudaMemsetAsync(a.y + a.ny_int, 0, (size_t)a.ny_zero * sizeof(float), st);
-    if (e != cudaSuccess) return e;
-  }
+  if (e != cudaSuccess) return e;
   if (a.k <= 0) return cudaSuccess;
   Scope sc(a.timer, T_SPMV, st);
-  const unsigned grid = (unsigned)((a.k + P.wpb - 1) / P.wpb);
-  if (a.readonly)
-    spmv_kernel<false><<<grid, 32 * P.wpb, P.smem, st>>>(a, P.wpb, P.cap);
-  else
-    spmv_kernel<true><<<grid, 32 * P.wpb, P.smem, st>>>(a, P.wpb, P.cap);
+  kern<<<(unsigned)P.grid, 32 * P.wpb, P.smem, st>>>(a, P.cap, P.hot);
+  return cudaGetLastError();
+}
+
+cudaError_t spmv_entries(const SpmvDesc* desc, int64_t k, const uint32_t* sent, const int32_t* xlist, uint32_t* ent,
+                         uint16_t* row0, cudaStream_t st) {
+  spmv_entries_kernel<<<(unsigned)((k + 7) / 8), 256, 0, st>>>(desc, k, sent, xlist, ent, row0);
   return cudaGetLastError();
 }
 

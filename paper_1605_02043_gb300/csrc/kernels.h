@@ -45,17 +45,19 @@ struct FluxArgs {
 struct SpmvArgs {
   const SpmvDesc* desc;
   int64_t k;
-  const int32_t* xlist;
   const int32_t* ylist;
-  const uint32_t* ent;   // entries, (row position << 16) | x position
-  const float* w;        // weight layout (one weight per entry, same index)
-  const float* x;        // x records
-  float* y;              // y records; [ny_int, ny_int + ny_zero) zeroed first
-  int64_t ny_int, ny_zero;
-  int32_t max_nx, max_ny, max_nxy;
-  int32_t u;              // entries per lane (every block's runs: 32 u slots)
-  int tpb;                // threads per CUDA block (one warp per schedule block)
-  bool readonly = false;  // x read through the read-only cache, not staged
+  const uint32_t* ent;     // device entries (kEntRow | x record)
+  const uint16_t* row0;    // row position of every lane's first entry, 32 per block
+  const float* w;          // weight layout (one weight per entry, same index), or
+  const int32_t* wmap;     // task weights read through this map (slot -> task)
+  const float* x;          // x records, the most used first
+  float* y;                // y records; the shared ones are zeroed first
+  const int32_t* yrow;     // y record -> row: results straight to the caller's rows, or nullptr
+  int64_t n, ny_int, ny_zero;
+  int32_t max_ny;
+  int32_t u;               // entries per lane (every block's runs: 32 u slots)
+  int tpb;                 // threads per CUDA block where no columns are kept
+  bool readonly = false;   // no columns kept: x read through the read-only cache
   Timer* timer;
 };
 
@@ -151,14 +153,18 @@ cudaError_t flux_adjoint_step(const FluxArgs& a, int D, float* lam, float* gw, c
 cudaError_t spmv(const SpmvArgs& a, cudaStream_t st);
 // shared memory the one-block kernels stage for the schedule's largest block
 size_t flux_block_smem(const FluxArgs& a, int D, bool adjoint);
-// SpMV launch shape: warps (schedule blocks) per CUDA block and the shared
-// memory of one CUDA block; 0 warps when one warp's share does not fit
+// SpMV launch shape; 0 warps when one warp's row totals do not fit
 struct SpmvPlan {
-  int wpb;      // warps per CUDA block (0: does not fit)
-  int cap;      // floats of the per-warp x / y region
-  size_t smem;  // dynamic shared memory per CUDA block
+  int wpb;       // warps per CUDA block (0: does not fit)
+  int cap;       // floats of a warp's row totals
+  int hot;       // x records kept in shared memory
+  int64_t grid;
+  size_t smem;   // dynamic shared memory per CUDA block
 };
-SpmvPlan spmv_plan(const SpmvArgs& a, int smem_optin);
+SpmvPlan spmv_plan(const SpmvArgs& a, int smem_optin, int sms);
+// device entries of a schedule from its host entries and x lists
+cudaError_t spmv_entries(const SpmvDesc* desc, int64_t k, const uint32_t* sent, const int32_t* xlist, uint32_t* ent,
+                         uint16_t* row0, cudaStream_t st);
 // SpMV layout in (one record per vertex): x_lay[rec_of[v]] <- x[v]
 cudaError_t layout_in(const int32_t* rec_of, int64_t n, int64_t n_rec, int D, const float* x,
                       float* x_lay, cudaStream_t st, Timer* t);

@@ -43,18 +43,18 @@ struct Entry {
 // the 1M-point mesh (4 is the least), and the gathers were what a step waited
 // for (11 us of 14).
 
-// Residues: swaps inside octets of [lo, hi) (aligned to 8) that even out, for
-// every reading octet, how many of its slots fall on each residue (sum of
-// squares).  readers(p): positions whose slots name position p; cnt: [octet][8].
-// swapped(a, b) carries the swap out.
-template <typename Readers, typename Swapped>
-void even_residues(int32_t lo, int32_t hi, int32_t keep, std::vector<int32_t>& cnt, Readers readers, Swapped swapped) {
-  auto shift = [&](int32_t p, int from, int to) {  // cost change when p's residue moves
+// Residues: swaps inside the octets of [lo, hi) (lo aligned to 8; positions
+// below `keep` and those from it on do not mix) that even out, for every reading
+// octet, how many of its slots fall on each residue (sum of squares).  who[p -
+// lo]: the vertex at position p (negative: none); its slots' octets are oct[ptr[v]
+// .. ptr[v + 1]); cnt: [octet][8].
+void even_residues(int32_t lo, int32_t hi, int32_t keep, const std::vector<int32_t>& ptr, const std::vector<int32_t>& oct,
+                   std::vector<int32_t>& cnt, std::vector<int32_t>& who) {
+  auto shift = [&](int32_t v, int from, int to) {  // cost change (halved) when v's residue moves
     int32_t c = 0;
-    for (int32_t q : readers(p)) {
-      int32_t* n = &cnt[(q >> 3) * 8];
-      c += 1 - 2 * n[from]--;
-      c += 1 + 2 * n[to]++;
+    for (int32_t i = ptr[v]; i < ptr[v + 1]; ++i) {
+      int32_t* n = &cnt[8 * (size_t)oct[i]];
+      c += 1 + n[to]++ - n[from]--;
     }
     return c;
   };
@@ -62,13 +62,13 @@ void even_residues(int32_t lo, int32_t hi, int32_t keep, std::vector<int32_t>& c
     for (int32_t o = lo; o < hi; o += 8)
       for (int32_t i = o; i < std::min(hi, o + 8); ++i)
         for (int32_t j = i + 1; j < std::min(hi, o + 8); ++j) {
-          if ((i < keep) != (j < keep)) continue;  // a boundary position stays one
-          const int32_t c = shift(i, i & 7, j & 7) + shift(j, j & 7, i & 7);
-          if (c < 0) {
-            swapped(i, j);
+          int32_t &a = who[i - lo], &b = who[j - lo];
+          if ((i < keep) != (j < keep) || a < 0 || b < 0) continue;
+          if (shift(a, i & 7, j & 7) + shift(b, j & 7, i & 7) < 0) {
+            std::swap(a, b);
           } else {
-            shift(i, j & 7, i & 7);
-            shift(j, i & 7, j & 7);
+            shift(a, j & 7, i & 7);
+            shift(b, i & 7, j & 7);
           }
         }
 }
@@ -80,6 +80,10 @@ void even_residues(int32_t lo, int32_t hi, int32_t keep, std::vector<int32_t>& c
 // receives the column of entry i.
 struct OctetColumns {
   std::vector<int16_t> lane_at, res_at;  // [8][K]: entry of a lane / lane of a residue in a column
+  std::vector<uint32_t> used, mine;      // spread_slice's scratch
+  std::vector<uint8_t> res[8], taken;
+  std::vector<int16_t> col[8];
+  std::vector<int32_t> to;
   void run(const int32_t* n, const uint8_t* const* res, int32_t K, int16_t* const* col) {
     lane_at.assign(8 * (size_t)K, -1);
     res_at.assign(8 * (size_t)K, -1);
@@ -139,14 +143,15 @@ struct OctetColumns {
 template <typename Put>
 void spread_slice(const std::vector<Entry>& ents, const int32_t* lo, const int32_t* hi, int32_t p0, int32_t K,
                   OctetColumns& oc, Put put) {
-  std::vector<uint32_t> used(K, 0);  // residues mod 32 per final column
-  std::vector<uint8_t> res[8];
-  std::vector<int16_t> col[8];
+  std::vector<uint32_t>&used = oc.used, &mine = oc.mine;
+  used.assign(K, 0);  // residues mod 32 per final column
+  std::vector<uint8_t>* res = oc.res;
+  std::vector<int16_t>* col = oc.col;
   for (int g = 0; g < 4; ++g) {
     int32_t n[8];
     const uint8_t* rp[8];
     int16_t* cp[8];
-    std::vector<uint32_t> mine(K, 0);
+    mine.assign(K, 0);
     for (int l = 0; l < 8; ++l) {
       const int L = 8 * g + l;
       n[l] = hi[L] - lo[L];
@@ -160,8 +165,10 @@ void spread_slice(const std::vector<Entry>& ents, const int32_t* lo, const int32
     for (int l = 0; l < 8; ++l)
       for (int32_t i = 0; i < n[l]; ++i) mine[col[l][i]] |= 1u << (ents[lo[8 * g + l] + i].o & 31);
     // each of this octet's columns to the final column it clashes least with
-    std::vector<int32_t> to(K, -1);
-    std::vector<bool> taken(K, false);
+    std::vector<int32_t>& to = oc.to;
+    std::vector<uint8_t>& taken = oc.taken;
+    to.assign(K, -1);
+    taken.assign(K, 0);
     for (int32_t c = 0; c < K; ++c) {
       int32_t best = -1, bs = 64;
       for (int32_t f = 0; f < K; ++f) {
@@ -170,7 +177,7 @@ void spread_slice(const std::vector<Entry>& ents, const int32_t* lo, const int32
         if (sc < bs) best = f, bs = sc;
       }
       to[c] = best;
-      taken[best] = true;
+      taken[best] = 1;
     }
     for (int32_t c = 0; c < K; ++c) {
       const int32_t f = to[c];
@@ -260,7 +267,7 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
   if (s.flags & 1u) return false;
   if (threads <= 0) threads = (int)std::max(1u, std::thread::hardware_concurrency());
   const int64_t nd = s.nd, m = s.m, n = s.touched;
-  threads = (int)std::max<int64_t>(1, std::min<int64_t>(threads, m / 8192));  // a thread costs about 50 us
+  threads = (int)std::max<int64_t>(1, std::min<int64_t>(threads, m / 1024));  // a thread costs about 50 us
   std::vector<int32_t> ru(m), rv(m);  // endpoint ranks in schedule order
   constexpr int64_t kChunk = 1 << 14;
   parallel_for((m + kChunk - 1) / kChunk, threads, [&](int, int64_t c) {
@@ -335,23 +342,21 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
       key[i] = {-((bnd ? 2 * kMarchMaxDegree : 0) + ptr[v + 1] - ptr[v]), i};
     }
     std::sort(key.begin(), key.end());
-    std::vector<int32_t> vert(d.own), cnt(((size_t)d.own + 8) / 8 * 8, 0), seen;
-    for (int32_t p = 0; p < d.own; ++p) vert[p] = order[cut[q] + key[p].second], rec[vert[p]] = p;
-    for (int32_t p = 0; p < d.own; ++p)
-      for (int32_t j = ptr[vert[p]]; j < ptr[vert[p] + 1]; ++j)
-        if (part_of[nb[j]] == q) ++cnt[(p >> 3) * 8 + (rec[nb[j]] & 7)];
-    even_residues(
-        0, d.own, d.nb, cnt,
-        [&](int32_t p) -> const std::vector<int32_t>& {
-          seen.clear();
-          for (int32_t j = ptr[vert[p]]; j < ptr[vert[p] + 1]; ++j)
-            if (part_of[nb[j]] == q) seen.push_back(rec[nb[j]]);
-          return seen;
-        },
-        [&](int32_t i, int32_t j) {
-          std::swap(vert[i], vert[j]);
-          rec[vert[i]] = i, rec[vert[j]] = j;
-        });
+    for (int32_t p = 0; p < d.own; ++p) rec[order[cut[q] + key[p].second]] = p;
+    std::vector<int32_t> cnt(((size_t)d.own + 7) / 8 * 8, 0), who(d.own), rp(d.own + 1, 0), ro;
+    for (int32_t i = 0; i < d.own; ++i) {
+      const int32_t v = order[cut[q] + i];
+      who[rec[v]] = i;
+      for (int32_t j = ptr[v]; j < ptr[v + 1]; ++j)
+        if (part_of[nb[j]] == q) {
+          const int32_t o = rec[nb[j]] >> 3;
+          ro.push_back(o);
+          ++cnt[8 * o + (rec[v] & 7)];
+        }
+      rp[i + 1] = (int32_t)ro.size();
+    }
+    even_residues(0, d.own, d.nb, rp, ro, cnt, who);
+    for (int32_t p = 0; p < d.own; ++p) rec[order[cut[q] + who[p]]] = p;
     // (rec: position so far; its part's first record is added below)
   });
   // halo lists (by vertex, then sorted by record once the runs have a place)
@@ -388,38 +393,40 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
     std::sort(t.halo.begin(), t.halo.end());  // the owners' order, but for the swaps inside octets
     std::vector<int32_t> vert(d.own);
     for (int64_t r = cut[q]; r < cut[q + 1]; ++r) vert[rec[order[r]] - d.lo] = order[r];
-    std::vector<std::pair<int32_t, int32_t>> hpos(d.nh);  // record, position
-    for (int32_t i = 0; i < d.nh; ++i) hpos[i] = {t.halo[i], d.hbase + i};
-    auto halo_index = [&](int32_t r) {
-      return (int32_t)(std::lower_bound(hpos.begin(), hpos.end(), std::make_pair(r, (int32_t)-1)) - hpos.begin());
-    };
-    auto pos_of = [&](int32_t o) { return part_of[o] == q ? rec[o] - d.lo : hpos[halo_index(rec[o])].second; };
-    if (d.nh > 0) {  // residues of the halo, the own positions standing
-      std::vector<int32_t> cnt(((size_t)d.own + 8) / 8 * 8, 0), hp(d.nh + 1, 0), readers, index(d.nh), seen;
-      for (int32_t i = 0; i < d.nh; ++i) index[i] = i;  // halo position -> entry of hpos
-      std::vector<std::pair<int32_t, int32_t>> rd;
+    // positions of the other endpoints, slot by slot; then the halo's residues,
+    // the own positions standing
+    std::vector<int32_t> ip(d.own + 1, 0), pos;
+    pos.reserve(8 * (size_t)d.own);
+    for (int32_t p = 0; p < d.own; ++p) {
+      for (int32_t j = ptr[vert[p]]; j < ptr[vert[p] + 1]; ++j)
+        pos.push_back(part_of[nb[j]] == q ? rec[nb[j]] - d.lo
+                                          : d.hbase + (int32_t)(std::lower_bound(t.halo.begin(), t.halo.end(), rec[nb[j]]) -
+                                                                t.halo.begin()));
+      ip[p + 1] = (int32_t)pos.size();
+    }
+    if (d.nh > 0) {
+      std::vector<int32_t> cnt(((size_t)d.own + 7) / 8 * 8, 0), rp(d.nh + 1, 0), ro, at, moved(d.nh);
+      for (int32_t x : pos)
+        if (x >= d.hbase) ++rp[x - d.hbase + 1];
+      for (int32_t i = 0; i < d.nh; ++i) rp[i + 1] += rp[i];
+      ro.resize(rp[d.nh]);
+      at.assign(rp.begin(), rp.end() - 1);
       for (int32_t p = 0; p < d.own; ++p)
-        for (int32_t j = ptr[vert[p]]; j < ptr[vert[p] + 1]; ++j) {
-          const int32_t o = nb[j];
-          if (part_of[o] != q) rd.push_back({halo_index(rec[o]), p});
-          ++cnt[(p >> 3) * 8 + (pos_of(o) & 7)];
+        for (int32_t i = ip[p]; i < ip[p + 1]; ++i) {
+          ++cnt[8 * (p >> 3) + (pos[i] & 7)];
+          if (pos[i] >= d.hbase) ro[at[pos[i] - d.hbase]++] = p >> 3;
         }
-      std::sort(rd.begin(), rd.end());
-      for (auto& x : rd) ++hp[x.first + 1], readers.push_back(x.second);
-      for (int32_t i = 0; i < d.nh; ++i) hp[i + 1] += hp[i];
-      even_residues(
-          d.hbase & ~7, d.hbase + d.nh, d.hbase, cnt,
-          [&](int32_t p) -> const std::vector<int32_t>& {
-            seen.clear();
-            if (p >= d.hbase) seen.assign(readers.begin() + hp[index[p - d.hbase]], readers.begin() + hp[index[p - d.hbase] + 1]);
-            return seen;
-          },
-          [&](int32_t i, int32_t j) {
-            const int32_t a = index[i - d.hbase], b = index[j - d.hbase];
-            std::swap(index[i - d.hbase], index[j - d.hbase]);
-            hpos[a].second = j, hpos[b].second = i;
-          });
-      for (int32_t i = 0; i < d.nh; ++i) t.halo[i] = hpos[index[i]].first;
+      const int32_t lo8 = d.hbase & ~7;
+      std::vector<int32_t> who(d.hbase + d.nh - lo8, -1), rec_at(t.halo);
+      for (int32_t i = 0; i < d.nh; ++i) who[d.hbase - lo8 + i] = i;
+      even_residues(lo8, d.hbase + d.nh, 0, rp, ro, cnt, who);
+      for (int32_t i = 0; i < d.nh; ++i) {
+        const int32_t h = who[d.hbase - lo8 + i];
+        t.halo[i] = rec_at[h];
+        moved[h] = d.hbase + i;
+      }
+      for (int32_t& x : pos)
+        if (x >= d.hbase) x = moved[x - d.hbase];
     }
     const int32_t W = L.warps;
     std::vector<int32_t> kcol(d.nsl), c0(d.nsl);
@@ -448,10 +455,8 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
         lo[l] = (int32_t)ents.size();
         const int32_t p = 32 * j + l;
         if (p < d.own)
-          for (int32_t i = ptr[vert[p]]; i < ptr[vert[p] + 1]; ++i) {
-            const int32_t o = nb[i], e = s.edge_perm[inc[i] < 0 ? ~inc[i] : inc[i]];
-            ents.push_back(Entry{pos_of(o), e, inc[i] >= 0});
-          }
+          for (int32_t i = ptr[vert[p]], k = ip[p]; i < ptr[vert[p] + 1]; ++i, ++k)
+            ents.push_back(Entry{pos[k], s.edge_perm[inc[i] < 0 ? ~inc[i] : inc[i]], inc[i] >= 0});
         hi[l] = (int32_t)ents.size();
       }
       spread_slice(ents, lo, hi, 32 * j, 2 * kcol[j], oc, [&](int32_t c, int l, int32_t o, const Entry* x) {

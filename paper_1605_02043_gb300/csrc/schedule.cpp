@@ -444,19 +444,18 @@ std::string spmv_layout(HostSchedule& s) {
   s.yrec_of.assign(n, -1);
   s.sdesc.assign(s.k, SpmvDesc{});
   std::vector<int32_t> deg(s.nd, 0), cls;
-  // x records: cpack order restricted to columns
-  int32_t nx = 0;
-  for (int64_t b = 0; b < s.k; ++b) {
-    SpmvDesc& d = s.sdesc[b];
-    d.x_lo = nx;
-    for (int64_t i = s.vert_ptr[b]; i < s.vert_ptr[b + 1]; ++i) {
-      const int32_t v = s.vert_list[i];
-      if (v < n && owner[v] == b) s.xrec_of[v] = nx++;
-    }
-    d.n_xo = nx - d.x_lo;
+  // x records: the columns that most blocks use first (the kernel keeps a
+  // prefix of them in shared memory), columns of equal use in cpack order
+  {
+    int32_t most = 0;
+    for (int32_t v = 0; v < n; ++v) most = std::max(most, p[v]);
+    std::vector<int32_t> at(most + 2, 0), by_rank(s.nd, -1);
+    for (int32_t v = 0; v < n; ++v) ++at[most - p[v] + 1];
+    for (int32_t q = 0; q <= most; ++q) at[q + 1] += at[q];
+    for (int32_t v = 0; v < n; ++v) by_rank[s.relabel[v]] = v;
+    for (int32_t v : by_rank)
+      if (v >= 0) s.xrec_of[v] = at[most - p[v]]++;
   }
-  for (int32_t j = 0; j < n; ++j)
-    if (s.xrec_of[j] < 0) s.xrec_of[j] = nx++;
   // y records: single-block rows first, then shared rows; longest lists first
   int32_t ny = 0;
   for (int64_t b = 0; b < s.k; ++b) {
@@ -501,12 +500,8 @@ std::string spmv_layout(HostSchedule& s) {
     for (int64_t i = s.vert_ptr[b]; i < s.vert_ptr[b + 1]; ++i) {
       const int32_t v = s.vert_list[i];
       if (v >= n) continue;
-      if (owner[v] == b)
-        pos[v] = s.xrec_of[v] - d.x_lo;
-      else {
-        pos[v] = d.n_xo + nxf++;
-        s.xlist.push_back(s.xrec_of[v]);
-      }
+      pos[v] = nxf++;
+      s.xlist.push_back(s.xrec_of[v]);
     }
     d.n_xf = nxf;
     block_degrees(s, b, deg);
