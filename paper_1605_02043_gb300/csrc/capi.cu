@@ -294,22 +294,45 @@ int ensure_task_slots(ep_schedule* s) {
   return EP_OK;
 }
 
-// State from the caller's order into schedule layout: every vertex's values
-// are read once, in vertex order, and written to each of its records (a
-// gather by record would read each record's components from scattered
-// 4-byte locations).  Records of no vertex are left as they are: no kernel
-// reads them.
-int layout_in_state(ep_schedule* s, int32_t D, const float* x, float* x_lay, cudaStream_t st) {
-  if (int rc = ensure_host_maps(s)) return rc;
-  CU(ep::dev::layout_in_csr(s->d_hptr.as<int32_t>(), s->d_hrec.as<int32_t>(), s->h.nd, s->h.n_rec, D, x, x_lay,
-                            st, s->t()));
-  return EP_OK;
+// A state from the caller's order into one record per vertex (march and SpMV
+// layouts), with the weights if `wmap` is given.
+ep::dev::LayoutIn layout_rec(const int32_t* rec_of, int64_t n, int64_t n_rec, const float* x, float* x_lay) {
+  ep::dev::LayoutIn in;
+  in.map = rec_of;
+  in.n = n;
+  in.n_rec = n_rec;
+  in.x = x;
+  in.x_lay = x_lay;
+  return in;
 }
 
 // weight layout: flux schedules one weight per slot (two per task), SpMV
 // schedules one per task, both padded per block (wmap: slot -> task)
 const int32_t* wmap_of(ep_schedule* s) { return s->d_wmap.as<int32_t>(); }
 int64_t wlen_of(const ep_schedule* s) { return s->h.w_pad; }
+
+// State from the caller's order into schedule layout: every vertex's values
+// are read once, in vertex order, and written to each of its records (a
+// gather by record would read each record's components from scattered
+// 4-byte locations).  Records of no vertex are left as they are: no kernel
+// reads them.  With w, the weights go into `w_lay` in the same launch; from_host:
+// w is read in task order (it lives in host memory and crosses the host link
+// once, coalesced).
+int layout_in_state(ep_schedule* s, int32_t D, const float* x, float* x_lay, const float* w, float* w_lay,
+                    bool from_host, cudaStream_t st) {
+  if (int rc = ensure_host_maps(s)) return rc;
+  ep::dev::LayoutIn in = layout_rec(s->d_hptr.as<int32_t>(), s->h.nd, s->h.n_rec, x, x_lay);
+  in.recs = s->d_hrec.as<int32_t>();
+  if (w) {
+    in.scatter = from_host;
+    in.wmap = from_host ? s->d_tslot.as<int32_t>() : wmap_of(s);
+    in.nw = from_host ? s->h.m : wlen_of(s);
+    in.w = w;
+    in.w_lay = w_lay;
+  }
+  CU(ep::dev::inputs(in, D, st, s->t()));
+  return EP_OK;
+}
 
 // accumulator sets: forward steps and adjoint steps rotate their own three
 // buffers with their own phase word
@@ -666,14 +689,12 @@ int spmv_lay(ep_schedule* s, const float* x_lay, const float* w, float* y, bool 
   return EP_OK;
 }
 
-// Workspace w in schedule layout from the caller's w.  from_host: w is read
-// in task order (it lives in host memory and crosses the host link once,
-// coalesced); the padding slots, never written then, are cleared with the
+// Workspace w ready to be written: allocated, and for weights read in task
+// order (from_host) the padding slots, never written then, cleared with the
 // buffer.
-int weights_to_ws(ep_schedule* s, const float* w, bool from_host, cudaStream_t st) {
+int ensure_ws_w(ep_schedule* s, bool from_host, cudaStream_t st) {
   CU(s->ws_w.ensure((size_t)wlen_of(s) * sizeof(float)));
   if (!from_host) {
-    CU(ep::dev::gather(wmap_of(s), wlen_of(s), w, s->ws_w.as<float>(), st, s->t()));
     s->zeroed_w = nullptr;
     return EP_OK;
   }
@@ -682,7 +703,6 @@ int weights_to_ws(ep_schedule* s, const float* w, bool from_host, cudaStream_t s
     CU(cudaMemsetAsync(s->ws_w.p, 0, s->ws_w.bytes, st));
     s->zeroed_w = s->ws_w.p;
   }
-  CU(ep::dev::weights_scatter(s->d_tslot.as<int32_t>(), s->h.m, w, s->ws_w.as<float>(), st, s->t()));
   return EP_OK;
 }
 
@@ -690,17 +710,23 @@ int run_spmv(ep_schedule* s, const float* x, const float* w, float* y, cudaStrea
              bool from_host = false) {
   const ep::HostSchedule& h = s->h;
   CU(s->ws_x.ensure((size_t)h.n * sizeof(float)));
-  CU(ep::dev::layout_in(s->d_xrec.as<int32_t>(), h.n, h.n, 1, x, s->ws_x.as<float>(), st, s->t()));
-  // device buffers: weights read through the slot map and rows written in the
-  // caller's order by the kernel itself (2^18 rows, partitioned: the gather of
-  // 4M weights beforehand took 18 us, the copy of y 4, the kernel 24)
+  CU(ep::dev::inputs(layout_rec(s->d_xrec.as<int32_t>(), h.n, h.n, x, s->ws_x.as<float>()), 1, st, s->t()));
+  // weights read through the slot map and rows written in the caller's order
+  // by the kernel itself (2^18 rows, partitioned: the gather of 4M weights
+  // beforehand took 18 us, the copy of y 4, the kernel 24)
+  if (from_host) {  // x, w and y cross the host link once, in order
+    CU(s->ws_hw.ensure((size_t)h.m * sizeof(float)));
+    CU(s->ws_out.ensure((size_t)h.n * sizeof(float)));
+    CU(cudaMemcpyAsync(s->ws_hw.p, w, (size_t)h.m * sizeof(float), cudaMemcpyDefault, st));
+    if (int rc = spmv_lay(s, s->ws_x.as<float>(), s->ws_hw.as<float>(), s->ws_out.as<float>(), true, st)) return rc;
+    CU(cudaMemcpyAsync(y, s->ws_out.p, (size_t)h.n * sizeof(float), cudaMemcpyDefault, st));
+    return EP_OK;
+  }
   const bool apart = y + h.n <= w || w + h.m <= y;  // weights are read while rows are written
-  if (!from_host && apart) return spmv_lay(s, s->ws_x.as<float>(), w, y, true, st);
+  if (apart) return spmv_lay(s, s->ws_x.as<float>(), w, y, true, st);
   CU(s->ws_out.ensure((size_t)h.n * sizeof(float)));
-  if (int rc = weights_to_ws(s, w, from_host, st)) return rc;
-  if (int rc = spmv_lay(s, s->ws_x.as<float>(), s->ws_w.as<float>(), s->ws_out.as<float>(), false, st))
-    return rc;
-  CU(ep::dev::layout_out(s->d_yrec.as<int32_t>(), h.n, h.n, 1, s->ws_out.as<float>(), y, st, s->t()));
+  if (int rc = spmv_lay(s, s->ws_x.as<float>(), w, s->ws_out.as<float>(), true, st)) return rc;
+  CU(cudaMemcpyAsync(y, s->ws_out.p, (size_t)h.n * sizeof(float), cudaMemcpyDeviceToDevice, st));
   return EP_OK;
 }
 
@@ -1090,7 +1116,7 @@ int ep_layout_in(ep_schedule* s, int32_t D, const float* x, float* x_lay, void* 
   if (misaligned(x_lay)) return fail(EP_EINVAL, "schedule-layout buffers must be 16-byte aligned");
   if (int rc = ensure_device(s)) return rc;
   fresh_state(s);
-  return layout_in_state(s, D, x, x_lay, as_stream(stream));
+  return layout_in_state(s, D, x, x_lay, nullptr, nullptr, false, as_stream(stream));
 }
 
 int ep_layout_out(ep_schedule* s, int32_t D, const float* x_lay, float* x, void* stream) {
@@ -1099,8 +1125,8 @@ int ep_layout_out(ep_schedule* s, int32_t D, const float* x_lay, float* x, void*
   if (!x || !x_lay) return fail(EP_EINVAL, "null argument");
   if (misaligned(x_lay)) return fail(EP_EINVAL, "schedule-layout buffers must be 16-byte aligned");
   if (int rc = ensure_device(s)) return rc;
-  CU(ep::dev::layout_out(s->d_rec.as<int32_t>(), s->h.nd, s->h.n_rec, D, x_lay, x,
-                         as_stream(stream), s->t()));
+  CU(ep::dev::layout_out(s->d_rec.as<int32_t>(), s->h.nd, s->h.n_rec, D, x_lay, x, nullptr,
+                         nullptr, as_stream(stream), s->t()));
   return EP_OK;
 }
 
@@ -1249,15 +1275,18 @@ int run_march(ep_schedule* s, const ep::dev::MarchPlan& P, int32_t D, int32_t st
     CU(cudaMemcpyAsync(s->ws_hw.p, w, (size_t)s->h.m * sizeof(float), cudaMemcpyDefault, st));
     w = s->ws_hw.as<float>();
   }
-  CU(ep::dev::layout_in(rec, s->h.nd, L.n_rec, D, x, mx, st, s->t()));
-  CU(ep::dev::gather(s->d_mwmap.as<int32_t>(), 64 * L.n_col, w, mw, st, s->t()));
+  ep::dev::LayoutIn in = layout_rec(rec, s->h.nd, L.n_rec, x, mx);
+  in.wmap = s->d_mwmap.as<int32_t>();
+  in.nw = 64 * L.n_col;
+  in.w = w;
+  in.w_lay = mw;
+  CU(ep::dev::inputs(in, D, st, s->t()));
   if (mout && s->h.touched < s->h.nd) CU(cudaMemsetAsync(mout, 0, (size_t)L.n_rec * D * sizeof(float), st));
   ep::dev::MarchArgs a = march_args(s, mw, steps, 1, tau);
   a.x_in = a.x_out = mx;
   a.out = mout;
   if (int rc = march_launch(s, P, a, D, false, st)) return rc;
-  CU(ep::dev::layout_out(rec, s->h.nd, L.n_rec, D, mx, x, st, s->t()));
-  if (out) CU(ep::dev::layout_out(rec, s->h.nd, L.n_rec, D, mout, out, st, s->t()));
+  CU(ep::dev::layout_out(rec, s->h.nd, L.n_rec, D, mx, x, mout, out, st, s->t()));
   return EP_OK;
 }
 
@@ -1294,8 +1323,8 @@ int run_flux(ep_schedule* s, int32_t D, int32_t steps, float tau, float* x, cons
     CU(cudaMemsetAsync(s->ws_x.p, 0, s->ws_x.bytes, st));
     s->zeroed_x = s->ws_x.p;
   }
-  if (int rc = layout_in_state(s, D, x, s->ws_x.as<float>(), st)) return rc;
-  if (int rc = weights_to_ws(s, w, from_host, st)) return rc;
+  if (int rc = ensure_ws_w(s, from_host, st)) return rc;
+  if (int rc = layout_in_state(s, D, x, s->ws_x.as<float>(), w, s->ws_w.as<float>(), from_host, st)) return rc;
   if (out) CU(cudaMemsetAsync(s->ws_out.p, 0, lay, st));
   // the shared copies stay pending between steps; the last step finishes them
   for (int32_t t = 0; t < steps; ++t) {
@@ -1305,8 +1334,8 @@ int run_flux(ep_schedule* s, int32_t D, int32_t steps, float tau, float* x, cons
                                tau, last, st))
       return rc;
   }
-  CU(ep::dev::layout_out(s->d_rec.as<int32_t>(), h.nd, h.n_rec, D, s->ws_x.as<float>(), x, st, s->t()));
-  if (out) CU(ep::dev::layout_out(s->d_rec.as<int32_t>(), h.nd, h.n_rec, D, s->ws_out.as<float>(), out, st, s->t()));
+  CU(ep::dev::layout_out(s->d_rec.as<int32_t>(), h.nd, h.n_rec, D, s->ws_x.as<float>(), x,
+                         out ? s->ws_out.as<float>() : nullptr, out, st, s->t()));
   return EP_OK;
 }
 
@@ -1388,9 +1417,13 @@ int run_adjoint_march(ep_schedule* s, const ep::dev::MarchPlan& P, const float* 
   CU(s->ws_mw.ensure(wl * sizeof(float)));
   CU(s->ws_gw.ensure(wl * sizeof(float)));
   const int32_t* rec = s->d_mrec.as<int32_t>();
-  CU(ep::dev::layout_in(rec, s->h.nd, L.n_rec, D, x0, s->ws_mx.as<float>(), st, s->t()));
-  CU(ep::dev::layout_in(rec, s->h.nd, L.n_rec, D, lam, s->ws_lam.as<float>(), st, s->t()));
-  CU(ep::dev::gather(s->d_mwmap.as<int32_t>(), (int64_t)wl, w, s->ws_mw.as<float>(), st, s->t()));
+  ep::dev::LayoutIn in = layout_rec(rec, s->h.nd, L.n_rec, x0, s->ws_mx.as<float>());
+  in.wmap = s->d_mwmap.as<int32_t>();
+  in.nw = (int64_t)wl;
+  in.w = w;
+  in.w_lay = s->ws_mw.as<float>();
+  CU(ep::dev::inputs(in, D, st, s->t()));
+  CU(ep::dev::inputs(layout_rec(rec, s->h.nd, L.n_rec, lam, s->ws_lam.as<float>()), D, st, s->t()));
   CU(cudaMemsetAsync(s->ws_gw.p, 0, wl * sizeof(float), st));
   ep::dev::MarchArgs a = march_args(s, s->ws_mw.as<float>(), steps, steps, tau);
   a.x_in = s->ws_mx.as<float>();
@@ -1403,7 +1436,7 @@ int run_adjoint_march(ep_schedule* s, const ep::dev::MarchPlan& P, const float* 
     if (int rc = carry_untouched(s, D, a.lam_in, a.lam_out, st)) return rc;
   }
   if (int rc = march_launch(s, P, a, D, true, st)) return rc;
-  CU(ep::dev::layout_out(rec, s->h.nd, L.n_rec, D, a.lam_out, lam, st, s->t()));
+  CU(ep::dev::layout_out(rec, s->h.nd, L.n_rec, D, a.lam_out, lam, nullptr, nullptr, st, s->t()));
   CU(ep::dev::gather_add(s->d_mgslot.as<int32_t>(), s->h.m, s->ws_gw.as<float>(), grad_w, st, s->t()));
   return EP_OK;
 }
@@ -1433,21 +1466,21 @@ int ep_run_adjoint(ep_schedule* s, const float* x0, const float* w, float* lam, 
     if (int rc = march_plan_of(s, D, true, P)) return rc;
   if (P.parts) return run_adjoint_march(s, P, x0, w, lam, grad_w, D, steps, tau, st);
   float* hist = s->ws_hist.as<float>();
-  if (int rc = layout_in_state(s, D, x0, hist, st)) return rc;
-  CU(ep::dev::gather(wmap_of(s), wlen_of(s), w, s->ws_w.as<float>(), st, s->t()));
+  s->zeroed_w = nullptr;
+  if (int rc = layout_in_state(s, D, x0, hist, w, s->ws_w.as<float>(), false, st)) return rc;
   CU(cudaMemsetAsync(s->ws_gw.p, 0, (size_t)wlen_of(s) * sizeof(float), st));
   // the recomputed states are read whole by the adjoint: finish every one
   for (int32_t t = 0; t + 1 < steps; ++t)
     if (int rc = flux_step_any(s, D, s->ws_w.as<float>(), hist + lay * t, hist + lay * (t + 1), nullptr,
                                tau, true, st))
       return rc;
-  if (int rc = layout_in_state(s, D, lam, s->ws_lam.as<float>(), st)) return rc;
+  if (int rc = layout_in_state(s, D, lam, s->ws_lam.as<float>(), nullptr, nullptr, false, st)) return rc;
   // the cotangent's shared copies stay pending between adjoint steps
   for (int32_t t = steps - 1; t >= 0; --t)
     if (int rc = flux_adj_any(s, D, s->ws_w.as<float>(), hist + lay * t, s->ws_lam.as<float>(),
                               s->ws_gw.as<float>(), tau, t == 0, st))
       return rc;
-  CU(ep::dev::layout_out(s->d_rec.as<int32_t>(), h.nd, h.n_rec, D, s->ws_lam.as<float>(), lam, st, s->t()));
+  CU(ep::dev::layout_out(s->d_rec.as<int32_t>(), h.nd, h.n_rec, D, s->ws_lam.as<float>(), lam, nullptr, nullptr, st, s->t()));
   CU(ep::dev::gather_add(s->d_gslot.as<int32_t>(), h.m, s->ws_gw.as<float>(), grad_w, st, s->t()));
   return EP_OK;
 }
@@ -1491,7 +1524,7 @@ int ep_grad_state_in(ep_schedule* s, int32_t D, const float* x, float* x_lay, vo
   cudaStream_t st = as_stream(stream);
   if (int rc = grad_checks(s, D, x_lay, x_lay, x_lay, x_lay, false, P, st)) return rc;
   if (!x) return fail(EP_EINVAL, "null argument");
-  CU(ep::dev::layout_in(s->d_mrec.as<int32_t>(), s->h.nd, s->ml.n_rec, D, x, x_lay, st, s->t()));
+  CU(ep::dev::inputs(layout_rec(s->d_mrec.as<int32_t>(), s->h.nd, s->ml.n_rec, x, x_lay), D, st, s->t()));
   return EP_OK;
 }
 
@@ -1500,7 +1533,7 @@ int ep_grad_state_out(ep_schedule* s, int32_t D, const float* x_lay, float* x, v
   cudaStream_t st = as_stream(stream);
   if (int rc = grad_checks(s, D, x_lay, x_lay, x_lay, x_lay, false, P, st)) return rc;
   if (!x) return fail(EP_EINVAL, "null argument");
-  CU(ep::dev::layout_out(s->d_mrec.as<int32_t>(), s->h.nd, s->ml.n_rec, D, x_lay, x, st, s->t()));
+  CU(ep::dev::layout_out(s->d_mrec.as<int32_t>(), s->h.nd, s->ml.n_rec, D, x_lay, x, nullptr, nullptr, st, s->t()));
   return EP_OK;
 }
 
@@ -1590,7 +1623,7 @@ int ep_spmv_x_in(ep_schedule* s, const float* x, float* x_lay, void* stream) {
   g_error.clear();
   if (int rc = check_spmv(s)) return rc;
   if (!x || !x_lay) return fail(EP_EINVAL, "null argument");
-  CU(ep::dev::layout_in(s->d_xrec.as<int32_t>(), s->h.n, s->h.n, 1, x, x_lay, as_stream(stream), s->t()));
+  CU(ep::dev::inputs(layout_rec(s->d_xrec.as<int32_t>(), s->h.n, s->h.n, x, x_lay), 1, as_stream(stream), s->t()));
   return EP_OK;
 }
 
@@ -1598,7 +1631,7 @@ int ep_spmv_y_out(ep_schedule* s, const float* y_lay, float* y, void* stream) {
   g_error.clear();
   if (int rc = check_spmv(s)) return rc;
   if (!y || !y_lay) return fail(EP_EINVAL, "null argument");
-  CU(ep::dev::layout_out(s->d_yrec.as<int32_t>(), s->h.n, s->h.n, 1, y_lay, y, as_stream(stream), s->t()));
+  CU(ep::dev::layout_out(s->d_yrec.as<int32_t>(), s->h.n, s->h.n, 1, y_lay, y, nullptr, nullptr, as_stream(stream), s->t()));
   return EP_OK;
 }
 

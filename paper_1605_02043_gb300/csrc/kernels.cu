@@ -460,67 +460,121 @@ __global__ void halo_kernel(const FluxArgs a, const int32_t* __restrict__ hmap, 
 
 // ------------------------------------------------------------------- layout
 
-// caller layout [D][n] (by data vertex) <-> planar records (by record id)
-template <int D>
-__global__ void layout_in_kernel(const int32_t* __restrict__ rec_of, int64_t n, int64_t n_rec,
-                                 const float* __restrict__ x, float* __restrict__ x_lay) {
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
-       v += (int64_t)gridDim.x * blockDim.x) {
-    float t[D];
+// Every element of these conversions costs two dependent loads (a map entry,
+// then a record or value somewhere else), so a thread takes several elements,
+// a block's width apart, and has all of their loads in flight together.
+constexpr int kLayoutThreads = 256;
+__host__ __device__ constexpr int layout_batch(int D) { return D <= 4 ? 4 : 2; }  // vertices per thread
+constexpr int kWeightBatch = 8;                               // weights per thread
+
+// caller layout [D][n] (by data vertex) -> planar records: x read in vertex
+// order (coalesced; in host memory the GPU reads it over the host link); CSR:
+// every record of vertex v is written (its record and the copies of a shared
+// vertex, recs[ptr[v] .. ptr[v + 1])), else the one record map[v]
+template <int D, bool CSR>
+__device__ __forceinline__ void state_in(int64_t tile, const int32_t* __restrict__ map, const int32_t* __restrict__ recs,
+                                         int64_t n, int64_t n_rec, const float* __restrict__ x,
+                                         float* __restrict__ x_lay) {
+  constexpr int B = layout_batch(D);
+  const int64_t v0 = tile * (B * kLayoutThreads) + threadIdx.x;
+  float t[B][D];
+  int32_t lo[B], hi[B];
 #pragma unroll
-    for (int c = 0; c < D; ++c) t[c] = __ldg(x + (size_t)c * n + v);
-    rec_store<D>(x_lay, n_rec, __ldg(rec_of + v), t);
-  }
-}
-
-// flux layout in: x read in vertex order (coalesced; in host memory the GPU
-// reads it over the host link), every record of vertex v written (its record
-// and the copies of a shared vertex): recs[ptr[v] .. ptr[v + 1])
-template <int D>
-__global__ void layout_in_csr_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ recs,
-                                     int64_t n, int64_t n_rec, const float* __restrict__ x,
-                                     float* __restrict__ x_lay) {
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
-       v += (int64_t)gridDim.x * blockDim.x) {
-    float t[D];
+  for (int u = 0; u < B; ++u) {
+    const int64_t v = v0 + u * kLayoutThreads;
+    lo[u] = v < n ? __ldg(map + v) : 0;
+    hi[u] = v < n ? (CSR ? __ldg(map + v + 1) : lo[u] + 1) : 0;
 #pragma unroll
-    for (int c = 0; c < D; ++c) t[c] = x[(size_t)c * n + v];
-    for (int32_t i = __ldg(ptr + v), e = __ldg(ptr + v + 1); i < e; ++i) rec_store<D>(x_lay, n_rec, __ldg(recs + i), t);
+    for (int c = 0; c < D; ++c) t[u][c] = v < n ? x[(size_t)c * n + v] : 0.f;
   }
-}
-
-// w read in task order, written to the task's slots (two, -1 for none)
-__global__ void weights_scatter_kernel(const int2* __restrict__ slots, int64_t m, const float* __restrict__ w,
-                                       float* __restrict__ w_lay) {
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < m;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const float v = w[t];
-    const int2 sl = __ldg(slots + t);
-    if (sl.x >= 0) w_lay[sl.x] = v;
-    if (sl.y >= 0) w_lay[sl.y] = v;
-  }
-}
-
-template <int D>
-__global__ void layout_out_kernel(const int32_t* __restrict__ rec_of, int64_t n, int64_t n_rec,
-                                  const float* __restrict__ x_lay, float* __restrict__ x) {
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
-       v += (int64_t)gridDim.x * blockDim.x) {
-    float t[D];
-    rec_load<D, true>(x_lay, n_rec, __ldg(rec_of + v), t);
 #pragma unroll
-    for (int c = 0; c < D; ++c) x[(size_t)c * n + v] = t[c];
+  for (int u = 0; u < B; ++u)
+    for (int32_t i = lo[u]; i < hi[u]; ++i) rec_store<D>(x_lay, n_rec, CSR ? __ldg(recs + i) : i, t[u]);
+}
+
+// weights: gathered into slots (perm: slot -> task, -1 unused), or read in task
+// order and written to the task's two slots (-1 for none; w in host memory)
+__device__ __forceinline__ void weights_gather(int64_t tile, const int32_t* __restrict__ perm, int64_t m,
+                                               const float* __restrict__ w, float* __restrict__ w_lay) {
+  const int64_t i0 = tile * (kWeightBatch * kLayoutThreads) + threadIdx.x;
+  int32_t t[kWeightBatch];
+  float v[kWeightBatch];
+#pragma unroll
+  for (int u = 0; u < kWeightBatch; ++u) t[u] = i0 + u * kLayoutThreads < m ? __ldg(perm + i0 + u * kLayoutThreads) : -1;
+#pragma unroll
+  for (int u = 0; u < kWeightBatch; ++u) v[u] = t[u] >= 0 ? __ldg(w + t[u]) : 0.f;
+#pragma unroll
+  for (int u = 0; u < kWeightBatch; ++u)
+    if (i0 + u * kLayoutThreads < m) w_lay[i0 + u * kLayoutThreads] = v[u];
+}
+__device__ __forceinline__ void weights_scatter(int64_t tile, const int2* __restrict__ slots, int64_t m,
+                                                const float* __restrict__ w, float* __restrict__ w_lay) {
+  const int64_t i0 = tile * (kWeightBatch * kLayoutThreads) + threadIdx.x;
+  int2 sl[kWeightBatch];
+  float v[kWeightBatch];
+#pragma unroll
+  for (int u = 0; u < kWeightBatch; ++u) {
+    const int64_t t = i0 + u * kLayoutThreads;
+    v[u] = t < m ? w[t] : 0.f;
+    sl[u] = t < m ? __ldg(slots + t) : make_int2(-1, -1);
+  }
+#pragma unroll
+  for (int u = 0; u < kWeightBatch; ++u) {
+    if (sl[u].x >= 0) w_lay[sl[u].x] = v[u];
+    if (sl[u].y >= 0) w_lay[sl[u].y] = v[u];
   }
 }
 
-__global__ void gather_kernel(const int32_t* __restrict__ perm, int64_t m, const float* __restrict__ w,
-                              float* __restrict__ w_lay) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
-       i += (int64_t)gridDim.x * blockDim.x)
-  {
-    const int32_t t = perm[i];
-    w_lay[i] = t >= 0 ? __ldg(w + t) : 0.f;
-  }
+// A state and (W: 1 gathered, 2 scattered) the weights in one launch: the first
+// `state_tiles` blocks do the state, the others the weights.
+struct InputArgs {
+  const int32_t *map, *recs, *wmap;
+  const float *x, *w;
+  float *x_lay, *w_lay;
+  int64_t n, n_rec, nw, state_tiles;
+};
+template <int D, bool CSR, int W>
+__global__ void __launch_bounds__(kLayoutThreads) inputs_kernel(const InputArgs a) {
+  if (W == 0 || blockIdx.x < a.state_tiles)
+    state_in<D, CSR>(blockIdx.x, a.map, a.recs, a.n, a.n_rec, a.x, a.x_lay);
+  else if (W == 1)
+    weights_gather(blockIdx.x - a.state_tiles, a.wmap, a.nw, a.w, a.w_lay);
+  else
+    weights_scatter(blockIdx.x - a.state_tiles, reinterpret_cast<const int2*>(a.wmap), a.nw, a.w, a.w_lay);
+}
+__global__ void __launch_bounds__(kLayoutThreads) gather_kernel(const int32_t* __restrict__ perm, int64_t m,
+                                                               const float* __restrict__ w, float* __restrict__ w_lay) {
+  weights_gather(blockIdx.x, perm, m, w, w_lay);
+}
+
+// planar records -> caller layout, one state or two (TWO) over the same map
+template <int D, bool TWO>
+__global__ void __launch_bounds__(kLayoutThreads) layout_out_kernel(const int32_t* __restrict__ rec_of, int64_t n,
+                                                                   int64_t n_rec, const float* __restrict__ x_lay,
+                                                                   float* __restrict__ x,
+                                                                   const float* __restrict__ y_lay,
+                                                                   float* __restrict__ y) {
+  constexpr int B = layout_batch(D);
+  const int64_t v0 = blockIdx.x * (int64_t)(B * kLayoutThreads) + threadIdx.x;
+  int32_t r[B];
+  float t[B][D], q[B][D];
+#pragma unroll
+  for (int u = 0; u < B; ++u) r[u] = v0 + u * kLayoutThreads < n ? __ldg(rec_of + v0 + u * kLayoutThreads) : -1;
+#pragma unroll
+  for (int u = 0; u < B; ++u)
+    if (r[u] >= 0) {
+      rec_load<D, true>(x_lay, n_rec, r[u], t[u]);
+      if (TWO) rec_load<D, true>(y_lay, n_rec, r[u], q[u]);
+    }
+#pragma unroll
+  for (int u = 0; u < B; ++u)
+    if (r[u] >= 0) {
+#pragma unroll
+      for (int c = 0; c < D; ++c) {
+        x[(size_t)c * n + v0 + u * kLayoutThreads] = t[u][c];
+        if (TWO) y[(size_t)c * n + v0 + u * kLayoutThreads] = q[u][c];
+      }
+    }
 }
 
 __global__ void scatter_add_kernel(const int32_t* __restrict__ perm, int64_t m,
@@ -834,16 +888,6 @@ cudaError_t spmv_entries(const SpmvDesc* desc, int64_t k, const uint32_t* sent, 
   return cudaGetLastError();
 }
 
-cudaError_t layout_in(const int32_t* rec_of, int64_t n, int64_t n_rec, int D, const float* x,
-                      float* x_lay, cudaStream_t st, Timer* t) {
-  Scope sc(t, T_LAYOUT, st);
-  const int g = grid_for(n, 256);
-#define EP_LIN(DD) layout_in_kernel<DD><<<g, 256, 0, st>>>(rec_of, n, n_rec, x, x_lay)
-  EP_DISPATCH_D(D, EP_LIN)
-#undef EP_LIN
-  return cudaGetLastError();
-}
-
 cudaError_t halo_move(const FluxArgs& a, int D, const int32_t* hmap, int64_t nh, float* buf, bool pack,
                       cudaStream_t st) {
   if (nh <= 0) return cudaSuccess;
@@ -854,37 +898,55 @@ cudaError_t halo_move(const FluxArgs& a, int D, const int32_t* hmap, int64_t nh,
   return cudaGetLastError();
 }
 
-cudaError_t layout_in_csr(const int32_t* ptr, const int32_t* recs, int64_t n, int64_t n_rec, int D,
-                          const float* x, float* x_lay, cudaStream_t st, Timer* t) {
+namespace {
+template <int D>
+void inputs_launch(const InputArgs& a, bool csr, int w, unsigned grid, cudaStream_t st) {
+  using Kernel = void (*)(const InputArgs);
+  const Kernel k = csr ? (w == 0 ? (Kernel)inputs_kernel<D, true, 0> : w == 1 ? (Kernel)inputs_kernel<D, true, 1>
+                                                                              : (Kernel)inputs_kernel<D, true, 2>)
+                       : (w == 0 ? (Kernel)inputs_kernel<D, false, 0> : (Kernel)inputs_kernel<D, false, 1>);
+  k<<<grid, kLayoutThreads, 0, st>>>(a);
+}
+int64_t tiles(int64_t n, int per_thread) {
+  return std::max<int64_t>(1, (n + (int64_t)per_thread * kLayoutThreads - 1) / ((int64_t)per_thread * kLayoutThreads));
+}
+}  // namespace
+
+cudaError_t inputs(const LayoutIn& in, int D, cudaStream_t st, Timer* t) {
   Scope sc(t, T_LAYOUT, st);
-  const int g = grid_for(n, 256);
-#define EP_LIN(DD) layout_in_csr_kernel<DD><<<g, 256, 0, st>>>(ptr, recs, n, n_rec, x, x_lay)
+  InputArgs a;
+  a.map = in.map, a.recs = in.recs, a.x = in.x, a.x_lay = in.x_lay, a.n = in.n, a.n_rec = in.n_rec;
+  a.wmap = in.wmap, a.w = in.w, a.w_lay = in.w_lay, a.nw = in.nw;
+  a.state_tiles = tiles(in.n, layout_batch(D));
+  const int w = in.w_lay == nullptr ? 0 : in.scatter ? 2 : 1;
+  if (w == 2 && !in.recs) return cudaErrorInvalidValue;
+  const unsigned g = (unsigned)(a.state_tiles + (w ? tiles(in.nw, kWeightBatch) : 0));
+#define EP_LIN(DD) inputs_launch<DD>(a, in.recs != nullptr, w, g, st)
   EP_DISPATCH_D(D, EP_LIN)
 #undef EP_LIN
   return cudaGetLastError();
 }
 
-cudaError_t weights_scatter(const int32_t* slots, int64_t m, const float* w, float* w_lay, cudaStream_t st,
-                            Timer* t) {
+cudaError_t layout_out(const int32_t* rec_of, int64_t n, int64_t n_rec, int D, const float* x_lay, float* x,
+                       const float* y_lay, float* y, cudaStream_t st, Timer* t) {
   Scope sc(t, T_LAYOUT, st);
-  weights_scatter_kernel<<<grid_for(m, 256), 256, 0, st>>>(reinterpret_cast<const int2*>(slots), m, w, w_lay);
-  return cudaGetLastError();
-}
-
-cudaError_t layout_out(const int32_t* rec_of, int64_t n, int64_t n_rec, int D, const float* x_lay,
-                       float* x, cudaStream_t st, Timer* t) {
-  Scope sc(t, T_LAYOUT, st);
-  const int g = grid_for(n, 256);
-#define EP_LOUT(DD) layout_out_kernel<DD><<<g, 256, 0, st>>>(rec_of, n, n_rec, x_lay, x)
-  EP_DISPATCH_D(D, EP_LOUT)
+  const unsigned g = (unsigned)tiles(n, layout_batch(D));
+  if (y) {
+#define EP_LOUT(DD) layout_out_kernel<DD, true><<<g, kLayoutThreads, 0, st>>>(rec_of, n, n_rec, x_lay, x, y_lay, y)
+    EP_DISPATCH_D(D, EP_LOUT)
 #undef EP_LOUT
+  } else {
+#define EP_LOUT(DD) layout_out_kernel<DD, false><<<g, kLayoutThreads, 0, st>>>(rec_of, n, n_rec, x_lay, x, nullptr, nullptr)
+    EP_DISPATCH_D(D, EP_LOUT)
+#undef EP_LOUT
+  }
   return cudaGetLastError();
 }
 
 cudaError_t gather(const int32_t* perm, int64_t m, const float* w, float* w_lay, cudaStream_t st,
                    Timer* t) {
   Scope sc(t, T_LAYOUT, st);
-  gather_kernel<<<grid_for(m, 256), 256, 0, st>>>(perm, m, w, w_lay);
+  gather_kernel<<<(unsigned)tiles(m, kWeightBatch), kLayoutThreads, 0, st>>>(perm, m, w, w_lay);
   return cudaGetLastError();
 }
 

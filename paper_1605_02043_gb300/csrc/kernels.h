@@ -165,24 +165,32 @@ SpmvPlan spmv_plan(const SpmvArgs& a, int smem_optin, int sms);
 // device entries of a schedule from its host entries and x lists
 cudaError_t spmv_entries(const SpmvDesc* desc, int64_t k, const uint32_t* sent, const int32_t* xlist, uint32_t* ent,
                          uint16_t* row0, cudaStream_t st);
-// SpMV layout in (one record per vertex): x_lay[rec_of[v]] <- x[v]
-cudaError_t layout_in(const int32_t* rec_of, int64_t n, int64_t n_rec, int D, const float* x,
-                      float* x_lay, cudaStream_t st, Timer* t);
-cudaError_t layout_out(const int32_t* rec_of, int64_t n, int64_t n_rec, int D, const float* x_lay,
-                       float* x, cudaStream_t st, Timer* t);
+// planar records -> caller layout, one state (y null) or two over the same map
+cudaError_t layout_out(const int32_t* rec_of, int64_t n, int64_t n_rec, int D, const float* x_lay, float* x,
+                       const float* y_lay, float* y, cudaStream_t st, Timer* t);
 // halo sums of a shard schedule (forward kind): pack the last edge kernel's
 // sums of halo vertices i (shared id hmap[i], -1: not here) into buf[i][D], or
 // unpack buf into them
 cudaError_t halo_move(const FluxArgs& a, int D, const int32_t* hmap, int64_t nh, float* buf, bool pack,
                       cudaStream_t st);
-// vertex- and task-ordered input forms: x plane by plane in vertex order into
-// every record of each vertex (CSR ptr/recs; the flux layout in), and w in
-// task order into the task's two slots (slots[2 t], slots[2 t + 1], -1 for
-// none; for weights in host memory)
-cudaError_t layout_in_csr(const int32_t* ptr, const int32_t* recs, int64_t n, int64_t n_rec, int D,
-                          const float* x, float* x_lay, cudaStream_t st, Timer* t);
-cudaError_t weights_scatter(const int32_t* slots, int64_t m, const float* w, float* w_lay, cudaStream_t st,
-                            Timer* t);
+// Inputs into a layout, a state and (w_lay not null) the weights in one launch.
+// State, in vertex order: into the record map[v], or with recs into every record
+// recs[map[v] .. map[v + 1]).  Weights: w_lay[i] = w[wmap[i]] for i < nw (0
+// where negative), or with scatter (and recs) w read in task order and written
+// to the slots wmap[2 t] and wmap[2 t + 1] (-1 for none; w in host memory).
+struct LayoutIn {
+  const int32_t* map = nullptr;
+  const int32_t* recs = nullptr;
+  int64_t n = 0, n_rec = 0;
+  const float* x = nullptr;
+  float* x_lay = nullptr;
+  const int32_t* wmap = nullptr;
+  int64_t nw = 0;
+  const float* w = nullptr;
+  float* w_lay = nullptr;
+  bool scatter = false;
+};
+cudaError_t inputs(const LayoutIn& in, int D, cudaStream_t st, Timer* t);
 cudaError_t gather(const int32_t* perm, int64_t m, const float* w, float* w_lay, cudaStream_t st,
                    Timer* t);
 cudaError_t scatter_add(const int32_t* perm, int64_t m, const float* w_lay, float* w, cudaStream_t st,
