@@ -361,6 +361,12 @@ int ep_adjoint_finish(ep_schedule *s, int32_t D, float *lam, float tau, void *st
  *                                (may be the same buffer when steps > 1); ckpt
  *                                receives the states before steps 0, every,
  *                                2 every, ... (ceil(steps / every) states)
+ *   ep_grad_run                  the first three and ep_grad_state_out together:
+ *                                xT (float[D][n]) from x0 and w, filling w_lay
+ *                                and ckpt; work: one state, two if steps = 1
+ *   ep_grad_sweep                dx0 and dw (overwritten) from g = dL/dx_T; work:
+ *                                a weight buffer and min(steps, every) states,
+ *                                at least two
  *   ep_grad_backward             lam_out <- dL/dx_0 from lam_in = dL/dx_T (may
  *                                be the same buffer when steps > 1), gw_lay <-
  *                                dL/dw, from ep_grad_forward's ckpt; hist:
@@ -374,6 +380,11 @@ int ep_grad_weights_in(ep_schedule *s, int32_t D, const float *w, float *w_lay, 
 int ep_grad_weights_out(ep_schedule *s, int32_t D, const float *gw_lay, float *grad_w, void *stream);
 int ep_grad_forward(ep_schedule *s, int32_t D, const float *x_lay, float *xT_lay, const float *w_lay,
                     float *ckpt, int32_t steps, int32_t every, float tau, void *stream);
+int ep_grad_run(ep_schedule *s, int32_t D, const float *x0, const float *w, float *xT, float *work,
+                float *w_lay, float *ckpt, int32_t steps, int32_t every, float tau, void *stream);
+int ep_grad_sweep(ep_schedule *s, int32_t D, const float *ckpt, const float *w_lay, const float *g,
+                  float *dx0, float *dw, float *work, int32_t steps, int32_t every, float tau,
+                  void *stream);
 int ep_grad_backward(ep_schedule *s, int32_t D, const float *ckpt, float *hist, const float *w_lay,
                      const float *lam_in, float *lam_out, float *gw_lay, int32_t steps,
                      int32_t every, float tau, void *stream);

@@ -41,6 +41,8 @@ def _stream(stream):
     import torch
 
     if stream is None:
+        if torch.cuda.is_initialized():  # the raw handle: a Stream object costs 3 us
+            return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
         stream = torch.cuda.current_stream()
     return ctypes.c_void_p(stream.cuda_stream)
 
@@ -316,6 +318,16 @@ class Schedule:
         """A run in one launch that keeps its checkpoints (ep_grad_forward)."""
         check(lib().ep_grad_forward(self._h, D, _vp(x_lay), _vp(xT_lay), _vp(w_lay), _vp(ckpt), steps, every,
                                     tau, _stream(stream)))
+
+    def grad_run(self, x0, w, xT, work, w_lay, ckpt, steps: int, every: int, tau: float = 1e-3, stream=None):
+        """Inputs in, grad_forward and xT out in one call (ep_grad_run)."""
+        check(lib().ep_grad_run(self._h, int(x0.shape[0]), _vp(x0), _vp(w), _vp(xT), _vp(work), _vp(w_lay),
+                                _vp(ckpt), steps, every, tau, _stream(stream)))
+
+    def grad_sweep(self, ckpt, w_lay, g, dx0, dw, work, steps: int, every: int, tau: float = 1e-3, stream=None):
+        """g in, grad_backward, dx0 and dw out in one call (ep_grad_sweep)."""
+        check(lib().ep_grad_sweep(self._h, int(g.shape[0]), _vp(ckpt), _vp(w_lay), _vp(g), _vp(dx0), _vp(dw),
+                                  _vp(work), steps, every, tau, _stream(stream)))
 
     def grad_backward(self, D: int, ckpt, hist, w_lay, lam_in, lam_out, gw_lay, steps: int, every: int,
                       tau: float = 1e-3, stream=None):

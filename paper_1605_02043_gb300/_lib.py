@@ -53,6 +53,8 @@ SIGNATURES = {
     "ep_grad_state_out": (ctypes.c_int, [P, I32, P, P, P]),
     "ep_grad_weights_in": (ctypes.c_int, [P, I32, P, P, P]),
     "ep_grad_weights_out": (ctypes.c_int, [P, I32, P, P, P]),
+    "ep_grad_run": (ctypes.c_int, [P, I32, P, P, P, P, P, P, I32, I32, F32, P]),
+    "ep_grad_sweep": (ctypes.c_int, [P, I32, P, P, P, P, P, P, I32, I32, F32, P]),
     "ep_grad_forward": (ctypes.c_int, [P, I32, P, P, P, P, I32, I32, F32, P]),
     "ep_grad_backward": (ctypes.c_int, [P, I32, P, P, P, P, P, P, I32, I32, F32, P]),
     "ep_spmv_x_in": (ctypes.c_int, [P, P, P, P]),

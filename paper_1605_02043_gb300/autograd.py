@@ -29,15 +29,13 @@ class FluxSteps(torch.autograd.Function):
         ns, nw = sched.grad_sizes(D) if steps > 0 and every > 0 else (0, 0)
         ctx.on_chip = ns > 0
         if ctx.on_chip:
-            xl, wl = torch.empty(ns, **f32), torch.empty(nw, **f32)
-            xo = xl if steps > 1 else torch.empty_like(xl)
-            ckpt = torch.empty(-(-steps // every), ns, **f32)
-            sched.grad_state_in(x0, xl)
-            sched.grad_weights_in(D, w, wl)
-            sched.grad_forward(D, xl, xo, wl, ckpt, steps, every, tau)
+            # one call and three allocations: the host side of a short run is what takes time
+            saved = torch.empty(nw + -(-steps // every) * ns, **f32)  # weights, checkpoints
+            work = torch.empty(ns if steps > 1 else 2 * ns, **f32)
             xT = torch.empty_like(x0)
-            sched.grad_state_out(xo, xT)
-            ctx.save_for_backward(wl, ckpt)
+            sched.grad_run(x0, w, xT, work, saved, saved[nw:], steps, every, tau)
+            ctx.nw = nw
+            ctx.save_for_backward(saved)
             return xT
         xl = torch.empty(sched.layout_floats(D), **f32)
         wl = torch.empty(sched.weights_floats(), **f32)
@@ -62,19 +60,11 @@ class FluxSteps(torch.autograd.Function):
         wl, *ckpts = ctx.saved_tensors
         g = g.contiguous()
         if ctx.on_chip:
-            ckpt = ckpts[0]
-            ns = ckpt.shape[1]
-            # images between two checkpoints: every - 1 at most, and no more than the run has
-            hist = torch.empty(max(min(every, steps) - 2, 0), ns, device=g.device, dtype=torch.float32)
-            lam = torch.empty(ns, device=g.device, dtype=torch.float32)
-            lo = lam if steps > 1 else torch.empty_like(lam)
-            gwl = torch.empty_like(wl)
-            sched.grad_state_in(g, lam)
-            sched.grad_backward(D, ckpt, hist if hist.numel() else None, wl, lam, lo, gwl, steps, every, tau)
+            ns, nw = (wl.numel() - ctx.nw) // -(-steps // every), ctx.nw
+            work = torch.empty(nw + max(min(every, steps), 2) * ns, device=g.device, dtype=torch.float32)
             dx0 = torch.empty_like(g)
-            sched.grad_state_out(lo, dx0)
             dw = torch.empty(sched.m, device=g.device, dtype=torch.float32)
-            sched.grad_weights_out(D, gwl, dw)
+            sched.grad_sweep(wl[nw:], wl, g, dx0, dw, work, steps, every, tau)
             return dx0, dw, None, None, None, None
         lam = torch.empty_like(ckpts[0])
         sched.layout_in(g, lam)

@@ -198,12 +198,14 @@ constexpr int32_t kMarchParts = 152;  // one part per SM of the GPU the library 
 
 // Makes sure a CUDA device exists and the schedule is uploaded to the current one.
 int ensure_device(ep_schedule* s) {
-  int count = 0;
-  if (cudaGetDeviceCount(&count) != cudaSuccess || count == 0) {
-    cudaGetLastError();
-    return fail(EP_ENODEV, "no CUDA device");
-  }
   int dev = 0;
+  if (s->device < 0) {
+    int count = 0;
+    if (cudaGetDeviceCount(&count) != cudaSuccess || count == 0) {
+      cudaGetLastError();
+      return fail(EP_ENODEV, "no CUDA device");
+    }
+  }
   CU(cudaGetDevice(&dev));
   if (s->device >= 0) {
     if (dev != s->device)
@@ -1424,7 +1426,6 @@ int run_adjoint_march(ep_schedule* s, const ep::dev::MarchPlan& P, const float* 
   in.w_lay = s->ws_mw.as<float>();
   CU(ep::dev::inputs(in, D, st, s->t()));
   CU(ep::dev::inputs(layout_rec(rec, s->h.nd, L.n_rec, lam, s->ws_lam.as<float>()), D, st, s->t()));
-  CU(cudaMemsetAsync(s->ws_gw.p, 0, wl * sizeof(float), st));
   ep::dev::MarchArgs a = march_args(s, s->ws_mw.as<float>(), steps, steps, tau);
   a.x_in = s->ws_mx.as<float>();
   a.ckpt = s->ws_hist.as<float>();
@@ -1587,7 +1588,6 @@ int ep_grad_backward(ep_schedule* s, int32_t D, const float* ckpt, float* hist, 
   if (!hist && std::min(steps, every) > 2) return fail(EP_EINVAL, "null history buffer");
   if (steps == 1 && lam_in == lam_out) return fail(EP_EINVAL, "one step cannot be made in place");
   if (int rc = carry_untouched(s, D, lam_in, lam_out, st)) return rc;
-  CU(cudaMemsetAsync(gw_lay, 0, (size_t)s->ml.n_col * 64 * sizeof(float), st));
   ep::dev::MarchArgs a = march_args(s, w_lay, steps, every, tau);
   a.ckpt = const_cast<float*>(ckpt);  // only read: x_in is null
   a.hist = hist;
@@ -1595,6 +1595,44 @@ int ep_grad_backward(ep_schedule* s, int32_t D, const float* ckpt, float* hist, 
   a.lam_out = lam_out;
   a.gw = gw_lay;
   return march_launch(s, P, a, D, true, st);
+}
+
+int ep_grad_run(ep_schedule* s, int32_t D, const float* x0, const float* w, float* xT, float* work, float* w_lay,
+                float* ckpt, int32_t steps, int32_t every, float tau, void* stream) {
+  ep::dev::MarchPlan P;
+  cudaStream_t st = as_stream(stream);
+  if (int rc = grad_checks(s, D, work, w_lay, work, ckpt, false, P, st)) return rc;
+  if (!x0 || !w || !xT) return fail(EP_EINVAL, "null argument");
+  const int32_t* rec = s->d_mrec.as<int32_t>();
+  ep::dev::LayoutIn in = layout_rec(rec, s->h.nd, s->ml.n_rec, x0, work);
+  in.wmap = s->d_mwmap.as<int32_t>();
+  in.nw = 64 * s->ml.n_col;
+  in.w = w;
+  in.w_lay = w_lay;
+  CU(ep::dev::inputs(in, D, st, s->t()));
+  float* out = steps > 1 ? work : work + s->ml.n_rec * D;
+  if (int rc = ep_grad_forward(s, D, work, out, w_lay, ckpt, steps, every, tau, stream)) return rc;
+  CU(ep::dev::layout_out(rec, s->h.nd, s->ml.n_rec, D, out, xT, nullptr, nullptr, st, s->t()));
+  return EP_OK;
+}
+
+int ep_grad_sweep(ep_schedule* s, int32_t D, const float* ckpt, const float* w_lay, const float* g, float* dx0,
+                  float* dw, float* work, int32_t steps, int32_t every, float tau, void* stream) {
+  ep::dev::MarchPlan P;
+  cudaStream_t st = as_stream(stream);
+  if (int rc = grad_checks(s, D, ckpt, w_lay, work, work, true, P, st)) return rc;
+  if (!g || !dx0 || !dw) return fail(EP_EINVAL, "null argument");
+  const int32_t* rec = s->d_mrec.as<int32_t>();
+  const int64_t state = s->ml.n_rec * D;
+  float* gw = work;
+  float* lam = gw + s->ml.n_col * 64;
+  float* out = steps > 1 ? lam : lam + state;
+  float* hist = out + state;
+  CU(ep::dev::inputs(layout_rec(rec, s->h.nd, s->ml.n_rec, g, lam), D, st, s->t()));
+  if (int rc = ep_grad_backward(s, D, ckpt, hist, w_lay, lam, out, gw, steps, every, tau, stream)) return rc;
+  CU(ep::dev::layout_out(rec, s->h.nd, s->ml.n_rec, D, out, dx0, nullptr, nullptr, st, s->t()));
+  CU(ep::dev::gather(s->d_mgslot.as<int32_t>(), s->h.m, gw, dw, st, s->t()));
+  return EP_OK;
 }
 
 int ep_timing(ep_schedule* s, int32_t enable) {

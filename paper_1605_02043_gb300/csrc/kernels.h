@@ -112,7 +112,7 @@ struct MarchArgs {
   float* out;          // flux of the last step, or nullptr
   float* ckpt;         // images of the states before steps 0, every, 2 every, ...; or nullptr
   const float* lam_in; // gradient: cotangent in and out, images between two
-  float* lam_out;      // checkpoints (every - 1), weight gradient slots (added to)
+  float* lam_out;      // checkpoints (every - 1), weight gradient slots (tasks' first endpoints)
   float* hist;
   float* gw;
   float* ex;           // 2 x n_rec exchange records (ex_chunks(D) chunks)

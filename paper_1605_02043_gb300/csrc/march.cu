@@ -461,11 +461,11 @@ __global__ void __launch_bounds__(march_threads(D, false), 1) march_fwd_kernel(c
 
 // One reverse step of this warp's slices at the state S.x, cotangent S.lam
 // (flux_common.cuh adj_slice): new cotangents published and held like the
-// forward's values (the last one to memory), weight gradients added to their
-// task's slot at its first endpoint.
+// forward's values (the last one to memory), weight gradients added to (by the
+// first reverse step: stored in) their task's slot at its first endpoint.
 template <int D, bool RES>
 __device__ __forceinline__ void adjoint_slices(const MarchArgs& a, const MarchPart& d, const MarchSmem& S, uint32_t hold,
-                                               float* ex, uint32_t tag, bool last) {
+                                               float* ex, uint32_t tag, bool first, bool last) {
   constexpr int NC = ex_chunks(D);
   const int lane = threadIdx.x & 31, nw = blockDim.x >> 5, npos = a.npos;
   uint32_t at = hold;
@@ -491,7 +491,12 @@ __device__ __forceinline__ void adjoint_slices(const MarchArgs& a, const MarchPa
     const float inv = rcp_approx(q), s = dg * inv, two = 2.f * s * inv;
 #pragma unroll
     for (int c = 0; c < D; ++c) acc[c] -= w * (dl[c] * inv - two * dx[c]);
-    if (e & kSlotSrc) atomicAdd(g, a.tau * s);  // fire-and-forget reduction
+    if (e & kSlotSrc) {  // one lane's slot throughout: no reader before the next launch
+      if (first)
+        *g = a.tau * s;
+      else
+        atomicAdd(g, a.tau * s);  // fire-and-forget reduction
+    }
   };
   auto take = [&](uint32_t e, float2 w, int i) {
     one(e & 0xffffu, w.x, gw + 64 * (int64_t)i);
@@ -566,6 +571,7 @@ __global__ void __launch_bounds__(march_threads(D, true), 1) march_grad_kernel(c
   }
   const uint32_t hold = tmem + ((uint32_t)(warp & 3) << 21) + (uint32_t)(warp >> 2) * a.hold_cols;
   uint32_t sent = 0;  // exchanges so far, states and cotangents
+  bool first = true;  // the first reverse step sets the weight gradients, the others add
   auto ex_of = [&](uint32_t s) { return a.ex + (size_t)((s + 1) & 1) * a.n_rec * (4 * NC); };
   for (; seg >= 0 && fail == 0; --seg) {
     const int T = min(a.every, a.steps - seg * a.every);
@@ -594,7 +600,8 @@ __global__ void __launch_bounds__(march_threads(D, true), 1) march_grad_kernel(c
       const bool last = t == 0 && seg == 0;
       float* ex = ex_of(sent);
       const uint32_t tag = base + sent + 1u;
-      adjoint_slices<D, RES>(a, d, S, hold, ex, tag, last);
+      adjoint_slices<D, RES>(a, d, S, hold, ex, tag, first, last);
+      first = false;
       if (last) break;
       ++sent;
       // the state before this one, or the checkpoint before this segment's
