@@ -1,6 +1,8 @@
 // march.cpp -- host side of the resident run kernels' layout (march.h).
 #include "march.h"
 
+#include "banks.h"
+
 #include <algorithm>
 #include <atomic>
 #include <thread>
@@ -26,195 +28,6 @@ void parallel_for(int64_t n, int threads, F f) {
   for (int t = 1; t < threads; ++t) pool.emplace_back(work, t);
   work(0);
   for (auto& th : pool) th.join();
-}
-
-struct Entry {
-  int32_t o;  // position of the other endpoint
-  int32_t e;  // task
-  bool src;
-};
-
-// Shared-memory banks.  A column of a slice is one load per plane: a 16-byte
-// load is served 8 lanes at a time, each record covering the 4 banks of its
-// position mod 8; a 4-byte load 32 lanes at a time, position mod 32.  Two
-// things are free: the order of the 8 vertices of an octet of positions (the
-// residues its neighbours see), and which column a slot goes to.  Both are
-// chosen here; greedy columns alone left 8.3 wavefronts per 16-byte column on
-// the 1M-point mesh (4 is the least), and the gathers were what a step waited
-// for (11 us of 14).
-
-// Residues: swaps inside the octets of [lo, hi) (lo aligned to 8; positions
-// below `keep` and those from it on do not mix) that even out, for every reading
-// octet, how many of its slots fall on each residue (sum of squares).  who[p -
-// lo]: the vertex at position p (negative: none); its slots' octets are oct[ptr[v]
-// .. ptr[v + 1]); cnt: [octet][8].
-void even_residues(int32_t lo, int32_t hi, int32_t keep, const std::vector<int32_t>& ptr, const std::vector<int32_t>& oct,
-                   std::vector<int32_t>& cnt, std::vector<int32_t>& who) {
-  auto shift = [&](int32_t v, int from, int to) {  // cost change (halved) when v's residue moves
-    int32_t c = 0;
-    for (int32_t i = ptr[v]; i < ptr[v + 1]; ++i) {
-      int32_t* n = &cnt[8 * (size_t)oct[i]];
-      c += 1 + n[to]++ - n[from]--;
-    }
-    return c;
-  };
-  for (int pass = 0; pass < 2; ++pass)
-    for (int32_t o = lo; o < hi; o += 8)
-      for (int32_t i = o; i < std::min(hi, o + 8); ++i)
-        for (int32_t j = i + 1; j < std::min(hi, o + 8); ++j) {
-          int32_t &a = who[i - lo], &b = who[j - lo];
-          if ((i < keep) != (j < keep) || a < 0 || b < 0) continue;
-          if (shift(a, i & 7, j & 7) + shift(b, j & 7, i & 7) < 0) {
-            std::swap(a, b);
-          } else {
-            shift(a, j & 7, i & 7);
-            shift(b, i & 7, j & 7);
-          }
-        }
-}
-
-// Columns of one octet: lane l's entries (n[l] <= K of them, residues in
-// res[l]) get different columns, and entries of one residue different columns
-// too as far as there are no more than K of them: an edge colouring of the
-// bipartite lane-residue graph, by alternating paths (Koenig).  col[l][i]
-// receives the column of entry i.
-struct OctetColumns {
-  std::vector<int16_t> lane_at, res_at;  // [8][K]: entry of a lane / lane of a residue in a column
-  std::vector<uint32_t> used, mine;      // spread_slice's scratch
-  std::vector<uint8_t> res[8], taken;
-  std::vector<int16_t> col[8];
-  std::vector<int32_t> to;
-  void run(const int32_t* n, const uint8_t* const* res, int32_t K, int16_t* const* col) {
-    lane_at.assign(8 * (size_t)K, -1);
-    res_at.assign(8 * (size_t)K, -1);
-    for (int l = 0; l < 8; ++l)
-      for (int32_t i = 0; i < n[l]; ++i) {
-        const int r = res[l][i];
-        int32_t a = -1, b = -1, both = -1;
-        for (int32_t c = 0; c < K && both < 0; ++c) {
-          const bool fl = lane_at[l * K + c] < 0, fr = res_at[r * K + c] < 0;
-          if (fl && fr) both = c;
-          if (fl && a < 0) a = c;
-          if (fr && b < 0) b = c;
-        }
-        if (both < 0 && b >= 0) {  // a is free at the lane, b at the residue: swap a and b along the path from r
-          int rr = r;
-          const int32_t x = a, y = b;
-          int path_l[8], n_path = 0;  // residue -x- lane -y- residue -x- ...
-          while (n_path < 8) {
-            const int ll = res_at[rr * K + x];
-            if (ll < 0) break;
-            path_l[n_path++] = ll;
-            const int16_t e2 = lane_at[ll * K + y];
-            if (e2 < 0) break;
-            rr = res[ll][e2];
-            if (res_at[rr * K + y] != ll) break;  // an overflowing entry ends the path
-          }
-          auto mark = [&](int k, bool on) {
-            const int ll = path_l[k];
-            for (int32_t c : {x, y}) {
-              const int16_t e2 = lane_at[ll * K + c];
-              if (e2 < 0) continue;
-              int16_t& at = res_at[res[ll][e2] * K + c];
-              if (on ? at < 0 : at == ll) at = on ? (int16_t)ll : (int16_t)-1;
-            }
-          };
-          for (int k = 0; k < n_path; ++k) mark(k, false);
-          for (int k = 0; k < n_path; ++k) std::swap(lane_at[path_l[k] * K + x], lane_at[path_l[k] * K + y]);
-          for (int k = 0; k < n_path; ++k) mark(k, true);
-          both = a;
-        }
-        const int32_t c = both >= 0 ? both : a;
-        lane_at[l * K + c] = (int16_t)i;
-        if (res_at[r * K + c] < 0) res_at[r * K + c] = (int16_t)l;
-      }
-    for (int l = 0; l < 8; ++l)
-      for (int32_t c = 0; c < K; ++c)
-        if (lane_at[l * K + c] >= 0) col[l][lane_at[l * K + c]] = (int16_t)c;
-  }
-};
-
-// The slots of one slice: lane l's entries ents[lo[l] .. hi[l]) over K columns,
-// octet by octet; an octet's columns are then ordered so that the four octets'
-// positions mod 32 differ where they can.  An unused slot names the lane's own
-// position or one of its neighbours, whichever falls on a bank that is free or
-// read there anyway (its weight is 0 and its term zero whenever the lane's
-// used slots are finite); put(column, lane, position, entry or null).
-template <typename Put>
-void spread_slice(const std::vector<Entry>& ents, const int32_t* lo, const int32_t* hi, int32_t p0, int32_t K,
-                  OctetColumns& oc, Put put) {
-  std::vector<uint32_t>&used = oc.used, &mine = oc.mine;
-  used.assign(K, 0);  // residues mod 32 per final column
-  std::vector<uint8_t>* res = oc.res;
-  std::vector<int16_t>* col = oc.col;
-  for (int g = 0; g < 4; ++g) {
-    int32_t n[8];
-    const uint8_t* rp[8];
-    int16_t* cp[8];
-    mine.assign(K, 0);
-    for (int l = 0; l < 8; ++l) {
-      const int L = 8 * g + l;
-      n[l] = hi[L] - lo[L];
-      res[l].resize(n[l]);
-      col[l].resize(n[l]);
-      for (int32_t i = 0; i < n[l]; ++i) res[l][i] = (uint8_t)(ents[lo[L] + i].o & 7);
-      rp[l] = res[l].data();
-      cp[l] = col[l].data();
-    }
-    oc.run(n, rp, K, cp);
-    for (int l = 0; l < 8; ++l)
-      for (int32_t i = 0; i < n[l]; ++i) mine[col[l][i]] |= 1u << (ents[lo[8 * g + l] + i].o & 31);
-    // each of this octet's columns to the final column it clashes least with
-    std::vector<int32_t>& to = oc.to;
-    std::vector<uint8_t>& taken = oc.taken;
-    to.assign(K, -1);
-    taken.assign(K, 0);
-    for (int32_t c = 0; c < K; ++c) {
-      int32_t best = -1, bs = 64;
-      for (int32_t f = 0; f < K; ++f) {
-        if (taken[f]) continue;
-        const int sc = __builtin_popcount(used[f] & mine[c]);
-        if (sc < bs) best = f, bs = sc;
-      }
-      to[c] = best;
-      taken[best] = 1;
-    }
-    for (int32_t c = 0; c < K; ++c) {
-      const int32_t f = to[c];
-      uint32_t used8 = 0;
-      int32_t named[8];
-      int16_t at[8];
-      for (int l = 0; l < 8; ++l) {
-        at[l] = oc.lane_at[l * K + c];
-        if (at[l] >= 0) named[l] = ents[lo[8 * g + l] + at[l]].o, used8 |= 1u << (named[l] & 7), used[f] |= 1u << (named[l] & 31);
-      }
-      for (int l = 0; l < 8; ++l) {
-        const int L = 8 * g + l;
-        if (at[l] >= 0) {
-          put(f, L, named[l], &ents[lo[L] + at[l]]);
-          continue;
-        }
-        int32_t best = p0 + L, bs = 8;
-        auto score = [&](int32_t o) {
-          for (int k = 0; k < 8; ++k)
-            if (at[k] >= 0 && named[k] == o) return 0;  // read there anyway
-          return 2 * (int)(used8 >> (o & 7) & 1u) + (int)(used[f] >> (o & 31) & 1u);
-        };
-        if ((bs = score(best)) > 0)
-          for (int32_t i = lo[L]; i < hi[L] && bs > 0; ++i) {
-            const int sc = score(ents[i].o);
-            if (sc < bs) best = ents[i].o, bs = sc;
-          }
-        if (n[l] == 0)  // no vertex here: anything another lane reads
-          for (int k = 0; k < 8 && bs > 0; ++k)
-            if (at[k] >= 0) best = named[k], bs = 0;
-        named[l] = best;
-        used8 |= 1u << (best & 7);
-        used[f] |= 1u << (best & 31);
-        put(f, L, best, (const Entry*)nullptr);
-      }
-    }
-  }
 }
 
 // The first block that touches a vertex is not always the part most of its
@@ -446,7 +259,7 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
     d.ncol = cols;
     t.ent.assign((size_t)cols * 32, 0);
     t.wmap.assign((size_t)cols * 64, -1);
-    std::vector<Entry> ents;
+    std::vector<SlotEntry> ents;
     OctetColumns oc;
     for (int32_t j = 0; j < d.nsl; ++j) {
       int32_t lo[32], hi[32];
@@ -456,10 +269,21 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
         const int32_t p = 32 * j + l;
         if (p < d.own)
           for (int32_t i = ptr[vert[p]], k = ip[p]; i < ptr[vert[p] + 1]; ++i, ++k)
-            ents.push_back(Entry{pos[k], s.edge_perm[inc[i] < 0 ? ~inc[i] : inc[i]], inc[i] >= 0});
+            ents.push_back(SlotEntry{pos[k], s.edge_perm[inc[i] < 0 ? ~inc[i] : inc[i]], inc[i] >= 0});
         hi[l] = (int32_t)ents.size();
       }
-      spread_slice(ents, lo, hi, 32 * j, 2 * kcol[j], oc, [&](int32_t c, int l, int32_t o, const Entry* x) {
+      // An unused slot names the lane's own position or one of its neighbours:
+      // its weight is 0, and its term zero whenever the lane's used slots are
+      // finite.  A lane of no vertex names what another lane reads.
+      auto pad = [&](int l, int32_t read_there, auto score) {
+        int32_t best = 32 * j + l;
+        if (lo[l] == hi[l] && read_there >= 0) return read_there;
+        int bs = score(best);
+        for (int32_t i = lo[l]; i < hi[l] && bs > 0; ++i)
+          if (const int sc = score(ents[i].o); sc < bs) best = ents[i].o, bs = sc;
+        return best;
+      };
+      spread_slice(ents, lo, hi, 2 * kcol[j], oc, pad, [&](int32_t c, int l, int32_t o, const SlotEntry* x) {
         const size_t at = (size_t)32 * (c0[j] + c / 2) + l;
         const uint32_t v = (uint32_t)o | (x && x->src ? kSlotSrc : 0u);
         t.ent[at] |= v << (16 * (c & 1));

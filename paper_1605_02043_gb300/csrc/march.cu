@@ -229,15 +229,6 @@ struct HaloBatch {
   }
 };
 
-// The denominator 1 + |d|^2 is at least 1, so the approximate reciprocal (1
-// ulp, no scaling steps for denominators near the ends of the range) is as
-// accurate here as __fdividef; past 2^126 both give 0.
-__device__ __forceinline__ float rcp_approx(float v) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
-  return r;
-}
-
 // A warp's slices as one stream of pair columns: begin(slice) starts a slice,
 // take(entries, weights, column) handles one pair column of it, end(slice)
 // finishes it.  Entries and weights are read ahead across the slices' ends into

@@ -19,6 +19,7 @@
 #include <climits>
 #include <thread>
 
+#include "banks.h"
 #include "internal.h"
 
 namespace ep {
@@ -116,22 +117,11 @@ void class_order(const HostSchedule& s, int64_t b, const std::vector<int32_t>& d
   std::stable_sort(out.begin(), out.end(), [&](int32_t a, int32_t c) { return deg[a] > deg[c]; });
 }
 
-struct SlotEntry {
-  int32_t o;  // the other position
-  int32_t e;  // task
-  bool src;   // source side of the task (owns its weight-gradient element)
-};
-
-// Places the entries of slice j (positions 32 j + l, l < 32) in its columns.
-// Column by column, each lane takes one of its remaining entries so that the
-// 32 lanes read their other positions from different shared-memory banks as
-// far as the lists allow: different (o mod 8) within each group of 8 lanes
-// (a 16-byte load is served 8 lanes at a time, 4 banks each) and different
-// (o mod 32) over the slice (4-byte loads).  A lane with fewer entries than
-// columns leaves slots unused; an unused slot has weight 0, so its term is
-// exactly zero whatever position it names, and it takes a free bank too.
+// Places the entries of slice j (positions 32 j + l, l < 32) in its columns
+// (banks.h).  An unused slot has weight 0, so its term is exactly zero whatever
+// position it names: the one of the first 32 that falls on a free bank.
 void place_slice(HostSchedule& s, const FluxDesc& d, int32_t j, const std::vector<int32_t>& ent_ptr,
-                 std::vector<SlotEntry>& ents) {
+                 const std::vector<SlotEntry>& ents, OctetColumns& oc) {
   const int32_t c0 = s.soff[d.q0 + j], K = s.soff[d.q0 + j + 1] - c0;
   int32_t lo[32], hi[32];
   for (int l = 0; l < 32; ++l) {
@@ -139,50 +129,21 @@ void place_slice(HostSchedule& s, const FluxDesc& d, int32_t j, const std::vecto
     lo[l] = p < d.nv ? ent_ptr[p] : 0;
     hi[l] = p < d.nv ? ent_ptr[p + 1] : 0;
   }
-  const int32_t npad = std::min(d.nv, 32);  // unused slots name one of the first 32 positions
-  for (int32_t c = 0; c < K; ++c) {
-    uint32_t used32 = 0;
-    uint32_t used8[4] = {0, 0, 0, 0};
-    auto score = [&](int l, int32_t o) {
-      return 2 * (int)((used8[l >> 3] >> (o & 7)) & 1u) + (int)((used32 >> (o & 31)) & 1u);
-    };
-    // lanes that must place an entry in every remaining column go first
-    uint32_t forced_mask = 0;
-    for (int l = 0; l < 32; ++l)
-      if (hi[l] - lo[l] == K - c) forced_mask |= 1u << l;
-    for (int pass = 0; pass < 2; ++pass)
-      for (int l = 0; l < 32; ++l) {
-        const int32_t rem = hi[l] - lo[l];
-        const bool forced = (forced_mask >> l) & 1u;
-        if ((pass == 0) != forced) continue;
-        int32_t best = -1, bs = 4;
-        for (int32_t i = lo[l]; i < hi[l] && bs > 0; ++i) {
-          const int sc = score(l, ents[i].o);
-          if (sc < bs) best = i, bs = sc;
-        }
-        int32_t pad = 0, ps = 4;
-        if (!forced)
-          for (int32_t o = 0; o < npad && ps > 0; ++o) {
-            const int sc = score(l, o);
-            if (sc < ps) pad = o, ps = sc;
-          }
-        const int64_t slot = (int64_t)d.s0 + 32 * ((int64_t)c0 + c) + l;
-        int32_t o;
-        if (rem > 0 && (forced || bs <= ps)) {
-          std::swap(ents[lo[l]], ents[best]);
-          const SlotEntry& t = ents[lo[l]++];
-          o = t.o;
-          s.sidx[slot] = (uint16_t)((uint32_t)t.o | (t.src ? kSlotSrc : 0u));
-          s.wmap[slot] = t.e;
-          if (t.src) s.gslot[t.e] = (int32_t)slot;
-        } else {
-          o = pad;
-          s.sidx[slot] = (uint16_t)pad;  // weight slot stays -1: weight 0
-        }
-        used8[l >> 3] |= 1u << (o & 7);
-        used32 |= 1u << (o & 31);
-      }
-  }
+  const int32_t npad = std::min(d.nv, 32);
+  auto pad = [&](int, int32_t read_there, auto score) {
+    if (read_there >= 0 && read_there < npad) return read_there;
+    int32_t best = 0, bs = 4;
+    for (int32_t o = 0; o < npad && bs > 0; ++o)
+      if (const int sc = score(o); sc < bs) best = o, bs = sc;
+    return best;
+  };
+  spread_slice(ents, lo, hi, K, oc, pad, [&](int32_t c, int l, int32_t o, const SlotEntry* x) {
+    const int64_t slot = (int64_t)d.s0 + 32 * ((int64_t)c0 + c) + l;
+    s.sidx[slot] = (uint16_t)((uint32_t)o | (x && x->src ? kSlotSrc : 0u));
+    if (!x) return;  // weight slot stays -1: weight 0
+    s.wmap[slot] = x->e;
+    if (x->src) s.gslot[x->e] = (int32_t)slot;
+  });
 }
 
 // f(lo, hi) over contiguous ranges of [0, n), one host thread each
@@ -223,7 +184,7 @@ std::string flux_layout_blocks(HostSchedule& s, int threads) {
   // every block by itself: its positions (interior vertices, then shared
   // ones, each by descending degree) and its slices' columns
   parallel_blocks(s.k, threads, [&](int64_t lo, int64_t hi) {
-    std::vector<int32_t> deg(s.nd, 0), ord, cls;
+    std::vector<int32_t> deg(s.nd, 0), pos(s.nd), ord, cls, rp, ro, cnt, who;
     for (int64_t b = lo; b < hi; ++b) {
       FluxDesc& d = s.fdesc[b];
       d.ne = (int32_t)(s.block_ptr[b + 1] - s.block_ptr[b]);
@@ -233,7 +194,29 @@ std::string flux_layout_blocks(HostSchedule& s, int threads) {
       class_order(s, b, deg, [&](int32_t v) { return p[v] > 1; }, cls);
       ord.insert(ord.end(), cls.begin(), cls.end());
       d.nv = (int32_t)ord.size();
-      std::copy(ord.begin(), ord.end(), order.begin() + s.vert_ptr[b]);
+      // the order inside an octet of positions, by bank
+      for (int32_t q = 0; q < d.nv; ++q) pos[ord[q]] = q;
+      rp.assign(d.nv + 1, 0);
+      auto ends = [&](auto f) {  // f(position, the other endpoint's) for every slot of the block
+        for (int64_t i = s.block_ptr[b]; i < s.block_ptr[b + 1]; ++i) {
+          int32_t u, v;
+          task_ends(s, s.edge_perm[i], u, v);
+          f(pos[u], pos[v]);
+          if (v != u) f(pos[v], pos[u]);
+        }
+      };
+      ends([&](int32_t, int32_t o) { ++rp[o + 1]; });
+      for (int32_t q = 0; q < d.nv; ++q) rp[q + 1] += rp[q];
+      ro.resize(rp[d.nv]);
+      cnt.assign(((size_t)d.nv + 7) / 8 * 8, 0);
+      who.assign(rp.begin(), rp.end() - 1);  // fill positions first
+      ends([&](int32_t p_, int32_t o) {
+        ro[who[o]++] = p_ >> 3;
+        ++cnt[8 * (p_ >> 3) + (o & 7)];
+      });
+      for (int32_t q = 0; q < d.nv; ++q) who[q] = q;
+      even_residues(0, d.nv, d.ni, rp, ro, cnt, who);
+      for (int32_t q = 0; q < d.nv; ++q) order[s.vert_ptr[b] + q] = ord[who[q]];
       // slices of 32 positions; columns = largest degree in the slice
       d.nsl = (d.nv + 31) / 32;
       uint16_t* off = &cols[s.vert_ptr[b] + b];
@@ -281,9 +264,10 @@ std::string flux_layout_blocks(HostSchedule& s, int threads) {
   parallel_blocks(s.k, threads, [&](int64_t blo, int64_t bhi) {
     std::vector<int32_t> pos(s.nd), ent_ptr, col;
     std::vector<SlotEntry> ents;
+    OctetColumns oc;
     for (int64_t b = blo; b < bhi; ++b) {
       const FluxDesc& d = s.fdesc[b];
-      const int32_t* ord = &order[s.vert_ptr[b]];
+      const int32_t* ord = order.data() + s.vert_ptr[b];
       // shared ids of positions [ni, nv); the first copy of each shared vertex
       // (in its first block) carries kSidFirst and is the vertex's record
       for (int32_t q = 0; q < d.nv; ++q) {
@@ -313,7 +297,7 @@ std::string flux_layout_blocks(HostSchedule& s, int threads) {
         ents[col[pu]++] = SlotEntry{pv, e, true};
         if (v != u) ents[col[pv]++] = SlotEntry{pu, e, false};
       }
-      for (int32_t j = 0; j < d.nsl; ++j) place_slice(s, d, j, ent_ptr, ents);
+      for (int32_t j = 0; j < d.nsl; ++j) place_slice(s, d, j, ent_ptr, ents, oc);
     }
   });
   s.n_run = align4(next);
