@@ -481,7 +481,7 @@ int march_plan_of(ep_schedule* s, int32_t D, bool grad, ep::dev::MarchPlan& P) {
     Q = ep::dev::march_plan({L.parts, L.warps, L.max_pos, L.max_col, L.max_nsl}, D, grad, smem_max);
     if (!coop || sms < L.parts) Q.parts = 0;
     if (Q.parts) {
-      const void* k = ep::dev::march_kernel_ptr(D, grad, Q.resident);
+      const void* k = ep::dev::march_kernel_ptr(Q, D, grad);
       CU(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
       int per_sm = 0;
       CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, Q.threads, Q.smem));

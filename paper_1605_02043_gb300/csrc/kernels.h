@@ -134,11 +134,12 @@ struct MarchPlan {
   int parts;  // 0: does not fit
   int threads, warps, npos, off_lam, off_tab, off_ent, off_w, hold_cols, tmem_cols;
   bool resident;  // slots and weights stay in shared memory too
+  bool wide;      // the variant with more threads and fewer registers
   size_t smem;
 };
 // grad: the reverse sweep (state and cotangent on the chip), else the forward run
 MarchPlan march_plan(const MarchSizes& z, int D, bool grad, int smem_max);
-const void* march_kernel_ptr(int D, bool grad, bool resident);
+const void* march_kernel_ptr(const MarchPlan& P, int D, bool grad);
 cudaError_t march_run(const MarchArgs& a, const MarchPlan& P, int D, bool grad, cudaStream_t st);
 
 cudaError_t flux_step(const FluxArgs& a, int D, cudaStream_t st);

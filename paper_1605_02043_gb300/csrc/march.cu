@@ -42,10 +42,18 @@ namespace dev {
 namespace {
 
 constexpr int kErrTimeoutNeighbour = 4;
-// Threads of a block, by the registers a slot pair in flight takes (65,536 per
-// SM): below these limits the kernels spill next to nothing.  150,001 points,
-// D = 8, ten steps: 103 us with 1024 threads, 81 with 512.
-constexpr int march_threads(int D, bool grad) { return D <= (grad ? 2 : 5) ? 1024 : 512; }
+// Threads of a block, which set the registers a thread has for slot pairs in
+// flight (65,536 per SM).  Widths above 5 (the reverse sweep: above 2) spill
+// with 1024 threads: 150,001 points, D = 8, ten steps 103 us, 81 with 512.
+// Widths 3 to 5 (WIDE: 1024) need the warps only where a warp has many slices,
+// and otherwise fewer threads meet sooner at a step's two barriers: 2^20 points
+// (223 slices a part) 1228 us with 1024, 1285 with 512; 2^18 in input order (57
+// slices, a large halo) 143 and 130; 4096 points, 50 steps 105 and 101.
+constexpr int kWideSlices = 128;
+constexpr int march_threads(int D, bool grad, bool wide) {
+  return D <= 2 || (!grad && D <= 5 && wide) ? 1024 : 512;
+}
+constexpr bool march_wide(int D, bool grad, int slices) { return grad || D < 3 || D > 5 || slices > kWideSlices; }
 
 // Exchange chunk: three components and the step's tag, one 128-bit access.
 __device__ __forceinline__ void chunk_store(float* p, const float* v, uint32_t tag) {
@@ -388,8 +396,8 @@ __device__ __forceinline__ bool settle(const MarchArgs& a, const MarchPart& d, f
 
 // ------------------------------------------------------------------ forward
 
-template <int D, bool RES>
-__global__ void __launch_bounds__(march_threads(D, false), 1) march_fwd_kernel(const MarchArgs a) {
+template <int D, bool RES, bool WIDE>
+__global__ void __launch_bounds__(march_threads(D, false, WIDE), 1) march_fwd_kernel(const MarchArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t bar;
   __shared__ uint32_t tmem_at;
@@ -522,7 +530,7 @@ __device__ __forceinline__ void adjoint_slices(const MarchArgs& a, const MarchPa
 // with one segment `x_in` may give its state instead (owners' records, `ckpt`
 // then receives the image).
 template <int D, bool RES>
-__global__ void __launch_bounds__(march_threads(D, true), 1) march_grad_kernel(const MarchArgs a) {
+__global__ void __launch_bounds__(march_threads(D, true, true), 1) march_grad_kernel(const MarchArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t bar;
   __shared__ uint32_t tmem_at;
@@ -637,29 +645,35 @@ cudaError_t march_launch_t(K kernel, const MarchArgs& a, const MarchPlan& P, cud
 }
 
 using MarchKernel = void (*)(const MarchArgs);
-template <int D>
-MarchKernel march_kernel_t(bool grad, bool res) {
-  if (grad) return res ? march_grad_kernel<D, true> : march_grad_kernel<D, false>;
-  return res ? march_fwd_kernel<D, true> : march_fwd_kernel<D, false>;
+template <int D, bool WIDE>
+MarchKernel march_fwd_t(bool res) {
+  return res ? march_fwd_kernel<D, true, WIDE> : march_fwd_kernel<D, false, WIDE>;
 }
-MarchKernel march_kernel(int D, bool grad, bool res) {
+template <int D>
+MarchKernel march_kernel_t(bool grad, bool res, bool wide) {
+  if (grad) return res ? march_grad_kernel<D, true> : march_grad_kernel<D, false>;
+  if constexpr (D >= 3 && D <= 5)
+    if (!wide) return march_fwd_t<D, false>(res);
+  return march_fwd_t<D, true>(res);
+}
+MarchKernel march_kernel(int D, bool grad, bool res, bool wide) {
   switch (D) {
-    case 1: return march_kernel_t<1>(grad, res);
-    case 2: return march_kernel_t<2>(grad, res);
-    case 3: return march_kernel_t<3>(grad, res);
-    case 4: return march_kernel_t<4>(grad, res);
-    case 5: return march_kernel_t<5>(grad, res);
-    case 6: return march_kernel_t<6>(grad, res);
-    case 7: return march_kernel_t<7>(grad, res);
-    case 8: return march_kernel_t<8>(grad, res);
+    case 1: return march_kernel_t<1>(grad, res, wide);
+    case 2: return march_kernel_t<2>(grad, res, wide);
+    case 3: return march_kernel_t<3>(grad, res, wide);
+    case 4: return march_kernel_t<4>(grad, res, wide);
+    case 5: return march_kernel_t<5>(grad, res, wide);
+    case 6: return march_kernel_t<6>(grad, res, wide);
+    case 7: return march_kernel_t<7>(grad, res, wide);
+    case 8: return march_kernel_t<8>(grad, res, wide);
   }
   return nullptr;
 }
 
 }  // namespace
 
-const void* march_kernel_ptr(int D, bool grad, bool res) {
-  return reinterpret_cast<const void*>(march_kernel(D, grad, res));
+const void* march_kernel_ptr(const MarchPlan& P, int D, bool grad) {
+  return reinterpret_cast<const void*>(march_kernel(D, grad, P.resident, P.wide));
 }
 
 // Shared-memory layout of a part and the launch shape, from the largest part's
@@ -679,7 +693,8 @@ MarchPlan march_plan(const MarchSizes& z, int D, bool grad, int smem_max) {
   P.smem = (size_t)(base + (P.resident ? cols * 384 : 0));
   // a warp per stream of slices (march.h), in whole groups of four: one per
   // quadrant of the tensor memory
-  P.threads = std::min(32 * z.warps, march_threads(D, grad));
+  P.wide = march_wide(D, grad, z.max_nsl);
+  P.threads = std::min(32 * z.warps, march_threads(D, grad, P.wide));
   P.warps = z.warps;
   const int per_warp = (z.warps * 32 + P.threads - 1) / P.threads;  // streams of one warp
   const int iters = (z.max_nsl + z.warps - 1) / z.warps * per_warp;
@@ -702,7 +717,7 @@ cudaError_t march_run(const MarchArgs& a0, const MarchPlan& P, int D, bool grad,
   a.off_w = P.off_w;
   a.hold_cols = (uint32_t)P.hold_cols;
   a.tmem_cols = (uint32_t)P.tmem_cols;
-  const MarchKernel k = march_kernel(D, grad, P.resident);
+  const MarchKernel k = march_kernel(D, grad, P.resident, P.wide);
   return k ? march_launch_t(k, a, P, st) : cudaErrorInvalidValue;
 }
 
