@@ -32,27 +32,36 @@ struct SlotEntry {
 // .. ptr[v + 1]); cnt: [octet][8].
 inline void even_residues(int32_t lo, int32_t hi, int32_t keep, const std::vector<int32_t>& ptr, const std::vector<int32_t>& oct,
                    std::vector<int32_t>& cnt, std::vector<int32_t>& who) {
-  auto shift = [&](int32_t v, int from, int to) {  // cost change (halved) when v's residue moves
+  auto cost = [&](int32_t v, int from, int to) {  // half the change when v's residue moves
     int32_t c = 0;
     for (int32_t i = ptr[v]; i < ptr[v + 1]; ++i) {
-      int32_t* n = &cnt[8 * (size_t)oct[i]];
-      c += 1 + n[to]++ - n[from]--;
+      const int32_t* n = &cnt[8 * (size_t)oct[i]];
+      c += 1 + n[to] - n[from];
     }
     return c;
   };
-  for (int pass = 0; pass < 2; ++pass)
+  auto move = [&](int32_t v, int from, int to) {
+    for (int32_t i = ptr[v]; i < ptr[v + 1]; ++i) {
+      int32_t* n = &cnt[8 * (size_t)oct[i]];
+      --n[from], ++n[to];
+    }
+  };
+  bool moved = true;
+  for (int pass = 0; pass < 2 && moved; ++pass) {
+    moved = false;
     for (int32_t o = lo; o < hi; o += 8)
       for (int32_t i = o; i < std::min(hi, o + 8); ++i)
         for (int32_t j = i + 1; j < std::min(hi, o + 8); ++j) {
           int32_t &a = who[i - lo], &b = who[j - lo];
           if ((i < keep) != (j < keep) || a < 0 || b < 0) continue;
-          if (shift(a, i & 7, j & 7) + shift(b, j & 7, i & 7) < 0) {
-            std::swap(a, b);
-          } else {
-            shift(a, j & 7, i & 7);
-            shift(b, i & 7, j & 7);
-          }
+          // (an octet that reads both counts as worse than it is)
+          if (cost(a, i & 7, j & 7) + cost(b, j & 7, i & 7) >= 0) continue;
+          move(a, i & 7, j & 7);
+          move(b, j & 7, i & 7);
+          std::swap(a, b);
+          moved = true;
         }
+  }
 }
 
 // Columns of one octet: lane l's entries (n[l] <= K of them, residues in
@@ -195,9 +204,10 @@ void spread_slice(const std::vector<SlotEntry>& ents, const int32_t* lo, const i
           continue;
         }
         named[l] = pad(L, read, [&](int32_t o) {
-          for (int k = 0; k < 8; ++k)
+          const int sc = 2 * (int)(used8 >> (o & 7) & 1u) + (int)(used[f] >> (o & 31) & 1u);
+          for (int k = 0; k < 8 && sc > 0; ++k)
             if (at[k] >= 0 && named[k] == o) return 0;  // read there anyway
-          return 2 * (int)(used8 >> (o & 7) & 1u) + (int)(used[f] >> (o & 31) & 1u);
+          return sc;
         });
         used8 |= 1u << (named[l] & 7);
         used[f] |= 1u << (named[l] & 31);
