@@ -3,11 +3,40 @@
 #pragma once
 
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
+#include <new>
+#include <system_error>
+#include <thread>
 #include <utility>
 #include <vector>
 
 namespace ep {
+
+// f(i) for i < n on up to `threads` host threads (fewer where no more can be
+// started).  Memory running out in one of them is thrown here.
+template <typename F>
+void parallel_for(int64_t n, int threads, F f) {
+  threads = (int)std::max<int64_t>(1, std::min<int64_t>(threads, n));
+  std::atomic<int64_t> next{0};
+  std::atomic<bool> failed{false};
+  auto work = [&] {
+    try {
+      for (int64_t i; !failed && (i = next.fetch_add(1)) < n;) f(i);
+    } catch (const std::bad_alloc&) {
+      failed = true;
+    }
+  };
+  std::vector<std::thread> pool;
+  pool.reserve(threads);
+  try {
+    for (int t = 1; t < threads; ++t) pool.emplace_back(work);
+  } catch (const std::system_error&) {
+  }
+  work();
+  for (auto& th : pool) th.join();
+  if (failed) throw std::bad_alloc();
+}
 
 struct SlotEntry {
   int32_t o;  // position of the other endpoint
@@ -21,9 +50,9 @@ struct SlotEntry {
 // things are free: the order of the 8 vertices of an octet of positions (the
 // residues its neighbours see), and which column a slot goes to.  Both are
 // chosen here; greedy columns alone left 8.3 wavefronts per 16-byte column on
-// the 1M-point mesh (4 is the least), 5.3 now; the gathers were what a step of
-// a resident run waited for (11 us of 14), and two thirds of the step kernels'
-// shared-memory time.
+// the 1M-point mesh (4 is the least), 5.4 now; the gathers were what a step of
+// a resident run waited for (11 us of 14, 8.4 now), and a third of the step
+// kernels' shared-memory wavefronts were conflicts.
 
 // Residues: swaps inside the octets of [lo, hi) (lo aligned to 8; positions
 // below `keep` and those from it on do not mix) that even out, for every reading

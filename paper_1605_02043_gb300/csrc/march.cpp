@@ -17,19 +17,6 @@ constexpr int32_t kMarchMaxDegree = 192;
 // Vertices per part below which more parts only add neighbours to wait for.
 constexpr int64_t kMarchMinPart = 64;
 
-template <typename F>
-void parallel_for(int64_t n, int threads, F f) {
-  threads = (int)std::max<int64_t>(1, std::min<int64_t>(threads, n));
-  std::atomic<int64_t> next{0};
-  auto work = [&](int t) {
-    for (int64_t i; (i = next.fetch_add(1)) < n;) f(t, i);
-  };
-  std::vector<std::thread> pool;
-  for (int t = 1; t < threads; ++t) pool.emplace_back(work, t);
-  work(0);
-  for (auto& th : pool) th.join();
-}
-
 // The first block that touches a vertex is not always the part most of its
 // neighbours are in, and the parts' cuts fall anywhere: passes over the
 // vertices move each one to the part that most of its neighbours are in, as
@@ -83,7 +70,7 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
   threads = (int)std::max<int64_t>(1, std::min<int64_t>(threads, m / 1024));  // a thread costs about 50 us
   std::vector<int32_t> ru(m), rv(m);  // endpoint ranks in schedule order
   constexpr int64_t kChunk = 1 << 14;
-  parallel_for((m + kChunk - 1) / kChunk, threads, [&](int, int64_t c) {
+  parallel_for((m + kChunk - 1) / kChunk, threads, [&](int64_t c) {
     for (int64_t i = c * kChunk; i < std::min(m, (c + 1) * kChunk); ++i) {
       const int32_t e = s.edge_perm[i];
       ru[i] = s.relabel[s.src[e]];
@@ -144,7 +131,7 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
   }
   L.warps = std::max(4, std::min(32, (L.max_nsl + 3) / 4 * 4));
   // positions: boundary vertices first, then by descending degree
-  parallel_for(P, threads, [&](int, int64_t q) {
+  parallel_for(P, threads, [&](int64_t q) {
     MarchPart& d = L.part[q];
     std::vector<std::pair<int32_t, int32_t>> key(d.own);  // (class and degree, place)
     for (int32_t i = 0; i < d.own; ++i) {
@@ -179,7 +166,7 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
     std::vector<uint32_t> ent;
   };
   std::vector<Piece> piece(P);
-  parallel_for(P, threads, [&](int, int64_t q) {
+  parallel_for(P, threads, [&](int64_t q) {
     std::vector<int32_t>& halo = piece[q].halo;
     for (int64_t i = cut[q]; i < cut[q + 1]; ++i)
       for (int32_t j = ptr[order[i]]; j < ptr[order[i] + 1]; ++j)
@@ -199,7 +186,7 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
   // the slots
   L.gslot.assign(m, -1);
   std::atomic<bool> ok{true};
-  parallel_for(P, threads, [&](int, int64_t q) {
+  parallel_for(P, threads, [&](int64_t q) {
     MarchPart& d = L.part[q];
     Piece& t = piece[q];
     for (int32_t& v : t.halo) v = rec[v];
@@ -305,7 +292,7 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
   if (nc > INT32_MAX / 64) return false;
   L.n_col = nc;
   L.halo.resize(nh), L.tab.resize(nq), L.ent.resize(32 * nc, 0), L.wmap.resize(64 * nc, -1);
-  parallel_for(P, threads, [&](int, int64_t q) {
+  parallel_for(P, threads, [&](int64_t q) {
     const MarchPart& d = L.part[q];
     const Piece& t = piece[q];
     std::copy(t.halo.begin(), t.halo.end(), L.halo.begin() + d.h0);

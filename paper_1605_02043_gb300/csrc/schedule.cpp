@@ -12,8 +12,8 @@
 //                    followed by its own copies of the shared vertices
 //                    (accumulated by atomics, refreshed by the fold), the
 //                    incidence in sliced-ELL slots with one weight per slot,
-//                    and the copy lists of the shared vertices; SpMV: row
-//                    lists over x records staged by owner and foreign ids.
+//                    and the copy lists of the shared vertices; SpMV: row-
+//                    ranked entries over x records ordered by use.
 #include <algorithm>
 #include <atomic>
 #include <climits>
@@ -146,14 +146,11 @@ void place_slice(HostSchedule& s, const FluxDesc& d, int32_t j, const std::vecto
   });
 }
 
-// f(lo, hi) over contiguous ranges of [0, n), one host thread each
+// f(lo, hi) over contiguous ranges of [0, n), one per host thread
 template <typename F>
 void parallel_blocks(int64_t n, int threads, F f) {
   threads = (int)std::max<int64_t>(1, std::min<int64_t>(threads, n / 16));
-  std::vector<std::thread> pool;
-  for (int t = 1; t < threads; ++t) pool.emplace_back([&f, n, t, threads] { f(n * t / threads, n * (t + 1) / threads); });
-  f(0, n / threads);
-  for (auto& th : pool) th.join();
+  parallel_for(threads, threads, [&](int64_t t) { f(n * t / threads, n * (t + 1) / threads); });
 }
 
 std::string flux_layout_blocks(HostSchedule& s, int threads) {
