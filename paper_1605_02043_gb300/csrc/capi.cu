@@ -712,18 +712,24 @@ int run_spmv(ep_schedule* s, const float* x, const float* w, float* y, cudaStrea
              bool from_host = false) {
   const ep::HostSchedule& h = s->h;
   CU(s->ws_x.ensure((size_t)h.n * sizeof(float)));
-  CU(ep::dev::inputs(layout_rec(s->d_xrec.as<int32_t>(), h.n, h.n, x, s->ws_x.as<float>()), 1, st, s->t()));
+  ep::dev::LayoutIn in = layout_rec(s->d_xrec.as<int32_t>(), h.n, h.n, x, s->ws_x.as<float>());
+  if (from_host) {  // x, w and y cross the host link once, in order, by the layout kernels
+    CU(s->ws_out.ensure((size_t)h.n * sizeof(float)));
+    if (int rc = ensure_ws_w(s, true, st)) return rc;
+    in.scatter = true;
+    in.wmap = s->d_tslot.as<int32_t>();
+    in.nw = h.m;
+    in.w = w;
+    in.w_lay = s->ws_w.as<float>();
+    CU(ep::dev::inputs(in, 1, st, s->t()));
+    if (int rc = spmv_lay(s, s->ws_x.as<float>(), in.w_lay, s->ws_out.as<float>(), false, st)) return rc;
+    CU(ep::dev::layout_out(s->d_yrec.as<int32_t>(), h.n, h.n, 1, s->ws_out.as<float>(), y, nullptr, nullptr, st, s->t()));
+    return EP_OK;
+  }
+  CU(ep::dev::inputs(in, 1, st, s->t()));
   // weights read through the slot map and rows written in the caller's order
   // by the kernel itself (2^18 rows, partitioned: the gather of 4M weights
   // beforehand took 18 us, the copy of y 4, the kernel 24)
-  if (from_host) {  // x, w and y cross the host link once, in order
-    CU(s->ws_hw.ensure((size_t)h.m * sizeof(float)));
-    CU(s->ws_out.ensure((size_t)h.n * sizeof(float)));
-    CU(cudaMemcpyAsync(s->ws_hw.p, w, (size_t)h.m * sizeof(float), cudaMemcpyDefault, st));
-    if (int rc = spmv_lay(s, s->ws_x.as<float>(), s->ws_hw.as<float>(), s->ws_out.as<float>(), true, st)) return rc;
-    CU(cudaMemcpyAsync(y, s->ws_out.p, (size_t)h.n * sizeof(float), cudaMemcpyDefault, st));
-    return EP_OK;
-  }
   const bool apart = y + h.n <= w || w + h.m <= y;  // weights are read while rows are written
   if (apart) return spmv_lay(s, s->ws_x.as<float>(), w, y, true, st);
   CU(s->ws_out.ensure((size_t)h.n * sizeof(float)));

@@ -904,7 +904,8 @@ void inputs_launch(const InputArgs& a, bool csr, int w, unsigned grid, cudaStrea
   using Kernel = void (*)(const InputArgs);
   const Kernel k = csr ? (w == 0 ? (Kernel)inputs_kernel<D, true, 0> : w == 1 ? (Kernel)inputs_kernel<D, true, 1>
                                                                               : (Kernel)inputs_kernel<D, true, 2>)
-                       : (w == 0 ? (Kernel)inputs_kernel<D, false, 0> : (Kernel)inputs_kernel<D, false, 1>);
+                       : (w == 0 ? (Kernel)inputs_kernel<D, false, 0> : w == 1 ? (Kernel)inputs_kernel<D, false, 1>
+                                                                               : (Kernel)inputs_kernel<D, false, 2>);
   k<<<grid, kLayoutThreads, 0, st>>>(a);
 }
 int64_t tiles(int64_t n, int per_thread) {
@@ -919,7 +920,6 @@ cudaError_t inputs(const LayoutIn& in, int D, cudaStream_t st, Timer* t) {
   a.wmap = in.wmap, a.w = in.w, a.w_lay = in.w_lay, a.nw = in.nw;
   a.state_tiles = tiles(in.n, layout_batch(D));
   const int w = in.w_lay == nullptr ? 0 : in.scatter ? 2 : 1;
-  if (w == 2 && !in.recs) return cudaErrorInvalidValue;
   const unsigned g = (unsigned)(a.state_tiles + (w ? tiles(in.nw, kWeightBatch) : 0));
 #define EP_LIN(DD) inputs_launch<DD>(a, in.recs != nullptr, w, g, st)
   EP_DISPATCH_D(D, EP_LIN)

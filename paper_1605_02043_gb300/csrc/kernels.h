@@ -177,7 +177,7 @@ cudaError_t halo_move(const FluxArgs& a, int D, const int32_t* hmap, int64_t nh,
 // Inputs into a layout, a state and (w_lay not null) the weights in one launch.
 // State, in vertex order: into the record map[v], or with recs into every record
 // recs[map[v] .. map[v + 1]).  Weights: w_lay[i] = w[wmap[i]] for i < nw (0
-// where negative), or with scatter (and recs) w read in task order and written
+// where negative), or with scatter w read in task order and written
 // to the slots wmap[2 t] and wmap[2 t + 1] (-1 for none; w in host memory).
 struct LayoutIn {
   const int32_t* map = nullptr;
