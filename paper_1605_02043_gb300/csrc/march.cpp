@@ -67,6 +67,7 @@ bool build_march(const HostSchedule& s, int32_t max_parts, int threads, MarchLay
   if (s.flags & 1u) return false;
   if (threads <= 0) threads = (int)std::max(1u, std::thread::hardware_concurrency());
   const int64_t nd = s.nd, m = s.m, n = s.touched;
+  if (n > (int64_t)max_parts * kSlotPos) return false;  // more positions a part than an entry can name
   threads = (int)std::max<int64_t>(1, std::min<int64_t>(threads, m / 1024));  // a thread costs about 50 us
   std::vector<int32_t> ru(m), rv(m);  // endpoint ranks in schedule order
   constexpr int64_t kChunk = 1 << 14;
