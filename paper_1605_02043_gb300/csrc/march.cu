@@ -438,6 +438,9 @@ __global__ void __launch_bounds__(march_threads(D, false, WIDE), 1) march_fwd_ke
     }
     forward_slices<D, RES>(a, d, S, hold, ex, tag, last);
     if (last) break;
+    // the checkpoint's copy out of S.x is over before settle()'s barrier lets
+    // S.x change (usually it is by now: the slices take longer)
+    if (a.ckpt && threadIdx.x == 0) bulk_wait_read();
     const bool here = settle<D>(a, d, S.x, hold, ex, tag, [] {});
     if (!here) {
       fail = 1;

@@ -161,3 +161,45 @@ def test_wait_for_a_neighbour_expires_then_recovers():
     assert ei.value.code == -4
     S.debug_stall(-1)
     assert run_against_oracle(S, src, dst, n, 5, 4, 2, tau=1e-3) == 1
+
+
+@pytest.mark.parametrize("n,D,steps,every", [(131072, 8, 6, 1), (131072, 5, 6, 1), (90001, 8, 7, 2), (4099, 8, 9, 1)])
+def test_checkpoints_hold_one_state_each(n, D, steps, every):
+    """Every checkpoint of a forward run is the state before its step, own records and
+    halo: the copy out of shared memory must be over before the next state overwrites
+    it.  Input order: images several times a part's own records beside few slices, so
+    the copy has the least time."""
+    src, dst = W.knn_mesh(n, 4, 6)
+    S = E.Schedule.partition(src, dst, n, 512, default_order=True)
+    ns, nw = S.grad_sizes(D)
+    assert ns > 0
+    x0, w, tau = W.flux_state(n, D, 6), W.flux_weights(src.size, 6), 1e-2
+    f32 = dict(device="cuda", dtype=torch.float32)
+    x, wl = cuda(x0), torch.empty(nw, **f32)
+    xl, xT = torch.empty(ns, **f32), torch.empty(ns, **f32)
+    S.grad_state_in(x, xl)
+    S.grad_weights_in(D, cuda(w), wl)
+    nseg = -(-steps // every)
+    ref = [x0.astype(np.float64)]
+    for _ in range(nseg - 1):
+        ref.append(O.flux_steps(src, dst, ref[-1], w, every, tau)[0])
+    got = torch.empty_like(x)
+    for _ in range(5):
+        ckpt = torch.full((nseg, ns), float("nan"), **f32)
+        S.grad_forward(D, xl, xT, wl, ckpt, steps, every, tau)
+        for i in range(nseg):
+            S.grad_state_out(ckpt[i], got)
+            check_state(got, ref[i], x0, i * every, f"checkpoint {i}")
+    # the halo parts of the images are what the reverse sweep recomputes from
+    g = W.loss_weights(n, D, 2)
+    lam, gw, work = torch.empty(ns, **f32), torch.empty(nw, **f32), torch.empty(max(every, 2) * ns, **f32)
+    gl = torch.empty(ns, **f32)
+    S.grad_state_in(cuda(g), gl)
+    S.grad_backward(D, ckpt, work, wl, gl, lam, gw, steps, every, tau)
+    S.grad_state_out(lam, got)
+    dw = torch.empty(src.size, **f32)
+    S.grad_weights_out(D, gw, dw)
+    dx_ref, dw_ref = O.flux_adjoint(src, dst, x0, w, steps, tau, g)
+    check_state(got, dx_ref, g, steps, "dx0")
+    check_field(dw, dw_ref, "dw")
+    assert S.check_errors() == 0
