@@ -139,7 +139,10 @@ __device__ __forceinline__ void acc_zero(float* bacc, int64_t h) {
 
 // The denominator 1 + |d|^2 is at least 1, so the approximate reciprocal (1
 // ulp, no scaling steps for denominators near the ends of the range) is as
-// accurate here as __fdividef; past 2^126 both give 0.
+// accurate here as __fdividef; past 2^126 both give 0.  |d|^2 is summed from 0
+// and the 1 added at the end, one rounding at the size of the sum: summed onto
+// 1, every component's term is rounded there (|d_c| ~ 0.1, relative rms of the
+// denominator: D = 5 3.3e-8 against 7.3e-8, D = 8 3.2e-8 against 9.0e-8).
 __device__ __forceinline__ float rcp_approx(float v) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
@@ -152,13 +155,13 @@ __device__ __forceinline__ void fwd_entry(const float* xs, int64_t n, int64_t ba
                                           const float* xp, float* acc) {
   float xo[D];
   rec_load<D, NC>(xs, n, base + (e & kSlotPos), xo);
-  float q = 1.f;
+  float q = 0.f;
 #pragma unroll
   for (int c = 0; c < D; ++c) {
     xo[c] -= xp[c];
     q = fmaf(xo[c], xo[c], q);
   }
-  const float coef = wt * rcp_approx(q);
+  const float coef = wt * rcp_approx(1.f + q);
 #pragma unroll
   for (int c = 0; c < D; ++c) acc[c] = fmaf(coef, xo[c], acc[c]);
 }
@@ -213,7 +216,7 @@ __device__ __forceinline__ void adj_slice(const float* xs, const float* ls, int6
     float xo[D], lo[D];
     rec_load<D>(xs, n, o, xo);
     rec_load<D>(ls, n, o, lo);
-    float q = 1.f, dg = 0.f;
+    float q = 0.f, dg = 0.f;
 #pragma unroll
     for (int c = 0; c < D; ++c) {
       xo[c] -= xp[c];        // d
@@ -221,7 +224,7 @@ __device__ __forceinline__ void adj_slice(const float* xs, const float* ls, int6
       q = fmaf(xo[c], xo[c], q);
       dg = fmaf(xo[c], lo[c], dg);
     }
-    const float inv = rcp_approx(q);
+    const float inv = rcp_approx(1.f + q);
     const float two = 2.f * dg * inv * inv;
 #pragma unroll
     for (int c = 0; c < D; ++c) acc[c] -= we * (lo[c] * inv - two * xo[c]);
