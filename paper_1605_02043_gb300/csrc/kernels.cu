@@ -845,10 +845,10 @@ SpmvPlan spmv_plan(const SpmvArgs& a, int smem_optin, int sms) {
     const int64_t rounds = (per_sm + most - 1) / most;
     P.wpb = (int)((per_sm + rounds - 1) / rounds);
     P.grid = std::min<int64_t>(sms, (a.k + P.wpb - 1) / P.wpb);
-    P.hot = (int)std::min<int64_t>(std::min<int64_t>(a.n + 3, kSpmvHot) / 4 * 4, (int64_t)((limit - P.wpb * per_warp) / 16 * 4));
-    if (P.hot > a.n) P.hot = (int)(a.n / 4 * 4);  // whole 16-byte pieces of x
+    // whole 16-byte pieces of x: none of a vector of fewer than 4 elements
+    P.hot = (int)std::min<int64_t>(std::min<int64_t>(a.n, kSpmvHot) / 4 * 4, (int64_t)((limit - P.wpb * per_warp) / 16 * 4));
     P.smem = P.wpb * per_warp + (size_t)P.hot * sizeof(float);
-    return P;
+    if (P.hot > 0) return P;
   }
   int wpb = std::max(1, std::min(8, a.tpb / 32));
   while (wpb > 1 && per_warp * wpb > (size_t)48 * 1024) --wpb;  // room for several CUDA blocks per SM
