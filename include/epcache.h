@@ -211,7 +211,10 @@ int ep_cost(ep_schedule *s, int64_t *loads, int64_t *vertex_cut, void *stream);
  * vertex is in more than 192 tasks; other runs launch one edge kernel a step.
  * Both give the same results up to FP32 rounding order.
  * Uses schedule-owned device workspace (allocated on first use: make the
- * first call before any stream capture).  Every step kernel stages a whole
+ * first call before any stream capture).  The on-chip layout and its workspace
+ * are made by the first eager call of two or more steps (host work about as
+ * long as the schedule took, once); a captured run before that takes the step
+ * kernels.  Every step kernel stages a whole
  * schedule block in shared memory: EP_EINVAL (nothing launched) when the
  * largest block does not fit, i.e. C too large for the graph and D (for
  * D = 5 on mesh-like graphs, C up to a few thousand tasks fits).

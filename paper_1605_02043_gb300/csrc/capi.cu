@@ -168,10 +168,12 @@ struct ep_schedule {
   // steps inside a stream capture only enqueue work
   ep::dev::TmaPlan plans[EP_MAX_D + 1][2];
   int plan_key[EP_MAX_D + 1][2] = {};
-  // resident runs of several steps (march.h): the host layout until it is
-  // uploaded, its device copy, the run's workspace and the launch plans
+  // resident runs of several steps (march.h): the layout, built when a call
+  // first asks for such a run (its arrays go once they are uploaded), its device
+  // copy, the run's workspace and the launch plans
   ep::MarchLayout ml;
-  bool march = false, march_up = false;
+  int march_threads = 0;  // host threads it is built with (0: all)
+  bool march_built = false, march = false, march_up = false;
   bool march_dirty = true;  // the exchange records and the parts' counts need clearing
   int32_t march_D = 0;      // state width they were last used with
   DBuf d_mpart, d_mhalo, d_mtab, d_ment, d_mwmap, d_mrec, d_mgslot;
@@ -463,13 +465,29 @@ int ensure_ctl(ep_schedule* s, cudaStream_t st) {
   return EP_OK;
 }
 
+// The resident layout, built on first need (host work only): a program that
+// makes single steps never asks for it, and it takes about as long as the rest
+// of the schedule (2^18 nodes, 8 cores: 73 ms beside 89, in input order 155
+// beside 105).  False where the graph does not suit it; where host memory runs
+// out for it, too: the step kernels need nothing more.
+bool march_layout(ep_schedule* s) {
+  if (!s->march_built) {
+    try {
+      s->march = ep::build_march(s->h, kMarchParts, s->march_threads, s->ml);
+    } catch (const std::bad_alloc&) {
+      s->march = false;
+    }
+    if (!s->march) s->ml = ep::MarchLayout();
+    s->march_built = true;
+  }
+  return s->march;
+}
+
 // Launch plan of a resident run (grad: of its reverse sweep) at state width D;
 // P.parts stays 0 where it cannot be resident: the graph does not suit the
 // layout, a part does not fit an SM, or the GPU has fewer SMs than parts.
 int march_plan_of(ep_schedule* s, int32_t D, bool grad, ep::dev::MarchPlan& P) {
   P.parts = 0;
-  if (!s->march) return EP_OK;
-  const ep::MarchLayout& L = s->ml;
   ep::dev::MarchPlan& Q = s->mplans[D][grad];
   if (!s->mplan_set[D][grad]) {
     int dev = 0, optin = 0, sms = 0, coop = 0;
@@ -478,8 +496,14 @@ int march_plan_of(ep_schedule* s, int32_t D, bool grad, ep::dev::MarchPlan& P) {
     CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     CU(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
     const int smem_max = optin - 512;  // less the kernels' static shared memory
-    Q = ep::dev::march_plan({L.parts, L.warps, L.max_pos, L.max_col, L.max_nsl}, D, grad, smem_max);
-    if (!coop || sms < L.parts) Q.parts = 0;
+    Q.parts = 0;
+    // not built for a width at which the vertices alone, evenly cut, are too many
+    const int64_t own = (s->h.touched + kMarchParts - 1) / kMarchParts;
+    if (coop && own * D * 4 * (grad ? 2 : 1) <= smem_max && march_layout(s)) {
+      const ep::MarchLayout& L = s->ml;
+      Q = ep::dev::march_plan({L.parts, L.warps, L.max_pos, L.max_col, L.max_nsl}, D, grad, smem_max);
+      if (sms < L.parts) Q.parts = 0;
+    }
     if (Q.parts) {
       const void* k = ep::dev::march_kernel_ptr(Q, D, grad);
       CU(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
@@ -496,23 +520,35 @@ int march_plan_of(ep_schedule* s, int32_t D, bool grad, ep::dev::MarchPlan& P) {
 // Whether runs may be resident under the schedule's settings (another kernel
 // organisation, the read-only cache and a shard's halo keep the step kernels).
 bool march_wanted(const ep_schedule* s) {
-  return s->march && s->stages != 0 && s->cache == EP_CACHE_SMEM && s->h.halo.empty();
+  return !bipartite(s) && s->stages != 0 && s->cache == EP_CACHE_SMEM && s->h.halo.empty();
+}
+
+// Uploads v and lets the host copy go (a second try after a failure finds it empty).
+template <typename T>
+cudaError_t hand_over(DBuf& d, std::vector<T>& v) {
+  const cudaError_t e = upload(d, v);
+  if (e == cudaSuccess) std::vector<T>().swap(v);
+  return e;
+}
+
+size_t march_ex_bytes(const ep_schedule* s, int32_t D) {
+  return 2 * (size_t)s->ml.n_rec * ep::dev::ex_chunks(D) * 16;
 }
 
 // Device copy of the layout, and the exchange records.
 int ensure_march(ep_schedule* s, int32_t D, cudaStream_t st) {
-  const ep::MarchLayout& L = s->ml;
+  ep::MarchLayout& L = s->ml;
   if (!s->march_up) {
-    CU(upload(s->d_mpart, L.part));
-    CU(upload(s->d_mhalo, L.halo));
-    CU(upload(s->d_mtab, L.tab));
-    CU(upload(s->d_ment, L.ent));
-    CU(upload(s->d_mwmap, L.wmap));
-    CU(upload(s->d_mrec, L.rec_of));
+    CU(hand_over(s->d_mpart, L.part));
+    CU(hand_over(s->d_mhalo, L.halo));
+    CU(hand_over(s->d_mtab, L.tab));
+    CU(hand_over(s->d_ment, L.ent));
+    CU(hand_over(s->d_mwmap, L.wmap));
+    CU(hand_over(s->d_mrec, L.rec_of));
     s->march_up = true;
     s->march_dirty = true;
   }
-  const size_t ex_bytes = 2 * (size_t)L.n_rec * ep::dev::ex_chunks(D) * 16;
+  const size_t ex_bytes = march_ex_bytes(s, D);
   if (ex_bytes > s->ws_mex.bytes || D != s->march_D) s->march_dirty = true;  // other records
   s->march_D = D;
   CU(s->ws_mex.ensure(ex_bytes));
@@ -526,7 +562,7 @@ int ensure_march(ep_schedule* s, int32_t D, cudaStream_t st) {
 }
 
 int ensure_march_grad(ep_schedule* s) {
-  if (!s->d_mgslot.p) CU(upload(s->d_mgslot, s->ml.gslot));
+  if (!s->d_mgslot.p) CU(hand_over(s->d_mgslot, s->ml.gslot));
   return EP_OK;
 }
 
@@ -793,7 +829,7 @@ int fill_partition(ep_schedule* s, const int32_t* src, const int32_t* dst, int64
     if (stop && stop->load()) return fail(EP_ECANCELED, "partition cancelled");
     std::string err = ep::build_schedule(h, threads);
     if (!err.empty()) return fail(EP_EINVAL, "%s", err.c_str());
-    s->march = ep::build_march(h, kMarchParts, threads, s->ml);
+    s->march_threads = threads;
   } catch (const std::bad_alloc&) {
     return fail(EP_ENOMEM, "out of host memory");
   }
@@ -1026,7 +1062,6 @@ int ep_batch(ep_schedule* const* parts, int32_t count, ep_schedule** out) {
       delete s;
       return fail(EP_EINVAL, "%s", err.c_str());
     }
-    s->march = ep::build_march(h, kMarchParts, 0, s->ml);
   } catch (const std::bad_alloc&) {
     delete s;
     return fail(EP_ENOMEM, "out of host memory");
@@ -1272,6 +1307,23 @@ int ep_run(ep_schedule* s, int32_t kernel, float* x, const float* w, float* out,
 
 namespace {
 
+bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &c) != cudaSuccess) {
+    cudaGetLastError();  // the legacy stream beside a capture
+    return true;
+  }
+  return c != cudaStreamCaptureStatusNone;
+}
+
+// Whether a resident run finds all it uses allocated and uploaded; inside a
+// stream capture, where neither is possible, a run takes the step kernels otherwise.
+bool march_in_place(const ep_schedule* s, int32_t D, bool out) {
+  const size_t state = (size_t)s->ml.n_rec * D * sizeof(float);
+  return s->march_up && s->ws_mex.bytes >= march_ex_bytes(s, D) && s->ws_mx.bytes >= state && s->ws_mw.p &&
+         (!out || s->ws_mout.bytes >= state);
+}
+
 // A resident run: the state in and out through the march layout's records.
 int run_march(ep_schedule* s, const ep::dev::MarchPlan& P, int32_t D, int32_t steps, float tau, float* x,
               const float* w, float* out, bool from_host, cudaStream_t st) {
@@ -1312,21 +1364,21 @@ int run_flux(ep_schedule* s, int32_t D, int32_t steps, float tau, float* x, cons
   }
   fresh_state(s);
   if (int rc = ensure_bacc(s, D, st)) return rc;
-  // every workspace of either path now, whatever `steps`: a later call inside
-  // a stream capture may take the other one
-  ep::dev::MarchPlan P;
-  P.parts = 0;
-  if (march_wanted(s))
-    if (int rc = march_plan_of(s, D, false, P)) return rc;
-  if (P.parts) {
-    if (int rc = ensure_march(s, D, st)) return rc;
-    CU(s->ws_mx.ensure((size_t)s->ml.n_rec * D * sizeof(float)));
-    CU(s->ws_mw.ensure((size_t)s->ml.n_col * 64 * sizeof(float)));
-    if (out) CU(s->ws_mout.ensure((size_t)s->ml.n_rec * D * sizeof(float)));
-  }
+  // the step kernels' workspace whatever `steps`: a later call inside a stream
+  // capture may take them
   CU(s->ws_w.ensure((size_t)wlen_of(s) * sizeof(float)));
   if (int rc = ensure_host_maps(s)) return rc;
-  if (P.parts && steps > 1) return run_march(s, P, D, steps, tau, x, w, out, from_host, st);
+  if (steps > 1 && march_wanted(s)) {
+    ep::dev::MarchPlan P;
+    if (int rc = march_plan_of(s, D, false, P)) return rc;
+    if (P.parts && (march_in_place(s, D, out != nullptr) || !capturing(st))) {
+      if (int rc = ensure_march(s, D, st)) return rc;
+      CU(s->ws_mx.ensure((size_t)s->ml.n_rec * D * sizeof(float)));
+      CU(s->ws_mw.ensure((size_t)s->ml.n_col * 64 * sizeof(float)));
+      if (out) CU(s->ws_mout.ensure((size_t)s->ml.n_rec * D * sizeof(float)));
+      return run_march(s, P, D, steps, tau, x, w, out, from_host, st);
+    }
+  }
   if (s->zeroed_x != s->ws_x.p) {  // records of no vertex stay zero
     CU(cudaMemsetAsync(s->ws_x.p, 0, s->ws_x.bytes, st));
     s->zeroed_x = s->ws_x.p;

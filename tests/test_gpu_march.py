@@ -203,3 +203,58 @@ def test_checkpoints_hold_one_state_each(n, D, steps, every):
     check_state(got, dx_ref, g, steps, "dx0")
     check_field(dw, dw_ref, "dw")
     assert S.check_errors() == 0
+
+
+def test_single_steps_make_no_resident_layout():
+    """One-step runs and single steps allocate nothing for resident runs; the first run of
+    several steps does (a state and the weights at the least)."""
+    n, D = 200003, 5
+    src, dst = W.knn_mesh(n, 4, 8)
+    S = E.Schedule.partition(src, dst, n, 512)
+    x0, w = W.flux_state(n, D, 8), W.flux_weights(src.size, 8)
+    x, wd = cuda(x0), cuda(w)
+    out = torch.zeros_like(x)
+
+    def free():
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    S.run(x, wd, out, steps=1, tau=1e-2)
+    before = free()
+    for _ in range(2):
+        S.run(x, wd, out, steps=1, tau=1e-2)
+    assert free() == before
+    S.run(x, wd, out, steps=2, tau=1e-2)
+    after = free()
+    ns, nw = S.grad_sizes(D)
+    assert before - after >= 4 * (ns + nw)
+    xT, fT = O.flux_steps(src, dst, x0, w, 5, 1e-2)
+    check_state(x, xT, x0, 5, "x")
+    check_field(out, fT, "out")
+
+
+def test_run_captured_before_any_eager_one():
+    """A run of several steps captured after single steps only: nothing can be allocated or
+    uploaded there, so it takes the step kernels; captured again after an eager run."""
+    n, D = 30011, 5
+    src, dst = W.knn_mesh(n, 4, 9)
+    S = E.Schedule.partition(src, dst, n, 512)
+    x0, w = W.flux_state(n, D, 9), W.flux_weights(src.size, 9)
+    x, wd = cuda(x0), cuda(w)
+    out = torch.zeros_like(x)
+    S.run(x, wd, out, steps=1, tau=1e-3)
+    for eager in (False, True):
+        if eager:
+            S.run(x, wd, out, steps=4, tau=1e-3)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            S.run(x, wd, out, steps=4, tau=1e-3)
+        x.copy_(cuda(x0))
+        for _ in range(3):
+            g.replay()
+        torch.cuda.synchronize()
+        xT, fT = O.flux_steps(src, dst, x0, w, 12, 1e-3)
+        check_state(x, xT, x0, 12, "x")
+        check_field(out, fT, "out")
+    assert S.check_errors() == 0
