@@ -258,3 +258,59 @@ def test_run_captured_before_any_eager_one():
         check_state(x, xT, x0, 12, "x")
         check_field(out, fT, "out")
     assert S.check_errors() == 0
+
+
+SMEM = 227 * 1024 - 512  # what a block of the resident kernels may ask for
+
+
+def slots_from_l2(S, D, grad):
+    """True where a part cannot keep its slots and weights in shared memory beside its
+    state (and cotangent): the mean part's need is above the limit, so the largest's is.
+    A state has D floats a record, a weight buffer 64 a column (entries and weights 384 bytes)."""
+    ns, nw = S.grad_sizes(1)
+    assert ns > 0 and S.n >= 152 * 64  # 152 parts
+    return (2 if grad else 1) * 4 * D * ns / 152 + 384 * nw / 64 / 152 > SMEM
+
+
+@pytest.fixture(scope="module")
+def large_mesh():
+    """(n, default order) -> (src, dst, schedule), one mesh kept at a time."""
+    kept = {}
+
+    def get(n, default_order):
+        if (n, default_order) not in kept:
+            kept.clear()
+            src, dst = W.knn_mesh(n, 4, 2)
+            kept[n, default_order] = src, dst, E.Schedule.partition(src, dst, n, 1024, default_order=default_order)
+        return kept[n, default_order]
+
+    yield get
+    kept.clear()
+
+
+# the forward kernel's variants: 512 threads (D = 5 in input order), 1024 (more
+# than 128 slices a part) and the widths with one thread count; g: gradients; r: the
+# mean part fits, so slots stay in shared memory with 1024 threads (D = 3) and 512
+@pytest.mark.parametrize("n,default_order,what", [
+    (400001, True, "f5"), (400001, False, "g6"), (520001, False, "f7 f8 g4 g5"), (640001, False, "r3 f5 f6 g3"),
+    (1 << 20, False, "f1 f2 f3 f4 g1 g2"), (320000, False, "r5 g8"),
+])
+def test_slots_read_from_the_l2(large_mesh, n, default_order, what):
+    from paper_1605_02043_gb300.autograd import flux_steps
+
+    src, dst, S = large_mesh(n, default_order)
+    w = W.flux_weights(src.size, 1)
+    for kind, D in ((k[0], int(k[1])) for k in what.split()):
+        assert slots_from_l2(S, D, kind == "g") == (kind != "r")
+        if kind != "g":
+            assert run_against_oracle(S, src, dst, n, D, 2, D) == 1
+            continue
+        assert S.grad_sizes(D)[0] > 0
+        x0, g, tau = W.flux_state(n, D, D), W.loss_weights(n, D, 1), 1e-2
+        x, wt = cuda(x0).requires_grad_(True), cuda(w).requires_grad_(True)
+        xT = flux_steps(x, wt, S, 3, tau, 2)
+        xT.backward(cuda(g))
+        dx_ref, dw_ref = O.flux_adjoint(src, dst, x0, w, 3, tau, g)
+        check_state(x.grad, dx_ref, g, 3, f"dx0 D={D}")
+        check_field(wt.grad, dw_ref, f"dw D={D}")
+    assert S.check_errors() == 0
