@@ -5,7 +5,6 @@
 #include <climits>
 #include <cstddef>
 #include <cstdint>
-#include <functional>
 #include <string>
 #include <vector>
 
@@ -53,9 +52,8 @@ constexpr uint32_t kColMask = 0xffffu;
 constexpr uint32_t kEntRow = 1u;  // device entries: 4 * x record, plus 1 on the first entry of a row
 
 // SpMV kernels (bipartite): x records are read only, y records accumulate.
-// x positions: [0, n_xo) the run x_lo.., then n_xf ids from xlist[fx0..]; the x
-// records are ordered by how many blocks use them, so the run is empty (n_xo =
-// 0) and every position is listed.
+// x positions: n_xf ids from xlist[fx0..] (x records are ordered by how many
+// blocks use them, so a block has no run of its own: x_lo = n_xo = 0).
 // y positions: [0, n_yi) the single-block rows yi_lo.., [n_yi, n_yi + n_yob)
 // the run yb_lo.. of shared rows first touched here, then n_yf ids from
 // ylist[fy0..]; within each class rows are ordered by descending list length.
@@ -118,8 +116,7 @@ struct HostSchedule {
   std::vector<SpmvDesc> sdesc;
   std::vector<int32_t> xlist, ylist;
   std::vector<uint32_t> sent;   // SpMV entries (padded runs, see SpmvDesc)
-  int32_t max_nx = 0, max_ny = 0;
-  int32_t max_nxy = 0;  // largest x + y positions of a block, each rounded up to 4
+  int32_t max_ny = 0;   // most y positions of a block
   int32_t spmv_u = 0;   // entries per lane (every block: 32 * spmv_u slots)
 };
 
@@ -142,9 +139,7 @@ bool partition_edges(const int32_t* src, const int32_t* dst, int64_t m, int64_t 
 
 // schedule.cpp: everything after the partition (Definition 4, vertex lists,
 // cpack, cost, kernel layout).  Returns an empty string or an error message.
-// `ordered`, if given, is called once the schedule itself stands (everything
-// but the kernel layout).
-std::string build_schedule(HostSchedule& s, int threads, const std::function<void()>& ordered = {});
+std::string build_schedule(HostSchedule& s, int threads);
 // The flux layout again (after `halo` changed); non-bipartite schedules only.
 std::string rebuild_flux_layout(HostSchedule& s);
 

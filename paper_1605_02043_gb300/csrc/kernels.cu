@@ -418,8 +418,7 @@ __global__ void spmv_entries_kernel(const SpmvDesc* __restrict__ desc, int64_t k
     uint32_t v = 0;
     if (t < d.ne) {
       const uint32_t e = src[j], row = e >> kRowShift;
-      const int col = (int)(e & kColMask);
-      v = 4u * (uint32_t)(col < d.n_xo ? d.x_lo + col : xlist[d.fx0 + col - d.n_xo]);
+      v = 4u * (uint32_t)xlist[d.fx0 + (int)(e & kColMask)];
       if (t == 0 || src[spmv_slot(t - 1, d.u)] >> kRowShift != row) v |= kEntRow;
       if (t % d.u == 0) row0[32 * b + t / d.u] = (uint16_t)row;
     } else if (t % d.u == 0) {

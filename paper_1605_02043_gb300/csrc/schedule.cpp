@@ -465,7 +465,7 @@ std::string spmv_layout(HostSchedule& s) {
   s.ylist.clear();
   s.sent.clear();
   s.wmap.clear();
-  s.max_nx = s.max_ny = s.max_nxy = 0;
+  s.max_ny = 0;
   std::vector<int32_t> pos(s.nd, -1), cnt;
   // one entry run of 32 * u slots per block (u from the largest block), so
   // that block b's run starts at slot 32 * u * b
@@ -500,12 +500,10 @@ std::string spmv_layout(HostSchedule& s) {
     }
     d.n_yf = nyf;
     for (int64_t i = s.vert_ptr[b]; i < s.vert_ptr[b + 1]; ++i) deg[s.vert_list[i]] = 0;
-    const int32_t nxs = d.n_xo + nxf, nys = d.n_yi + d.n_yob + nyf;
-    if (nxs > (int32_t)kColMask + 1 || nys > (int32_t)kColMask + 1)
+    const int32_t nys = d.n_yi + d.n_yob + nyf;
+    if (nxf > (int32_t)kColMask + 1 || nys > (int32_t)kColMask + 1)
       return "block touches too many vertices";
-    s.max_nx = std::max(s.max_nx, nxs);
     s.max_ny = std::max(s.max_ny, nys);
-    s.max_nxy = std::max(s.max_nxy, ((nxs + 3) & ~3) + ((nys + 3) & ~3));
     // entries sorted by row position (a counting sort; schedule order within
     // a row), each lane of the kernel's warp taking u consecutive ones
     cnt.assign(nys + 1, 0);
@@ -540,7 +538,7 @@ std::string rebuild_flux_layout(HostSchedule& s) {
   return flux_layout(s, (int)std::max(1u, std::thread::hardware_concurrency()));
 }
 
-std::string build_schedule(HostSchedule& s, int threads, const std::function<void()>& ordered) {
+std::string build_schedule(HostSchedule& s, int threads) {
   if (threads <= 0) threads = (int)std::max(1u, std::thread::hardware_concurrency());
   threads = (int)std::max<int64_t>(1, std::min<int64_t>(threads, s.k));
   // reconstruction (Definition 4): counting sort by block keeps ascending ids
@@ -558,7 +556,6 @@ std::string build_schedule(HostSchedule& s, int threads, const std::function<voi
   }
   vertex_lists(s, threads);
   cpack(s);
-  if (ordered) ordered();
   return (s.flags & 1u) ? spmv_layout(s) : flux_layout(s, threads);
 }
 
