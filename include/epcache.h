@@ -434,7 +434,9 @@ int ep_timing_read(ep_schedule *s, int32_t kernel_class, double *total_ms, int64
  * stages twice the state per kernel block and does about twice the arithmetic
  * per task, so fewer CUDA blocks fit an SM and each wants more warps).
  * EP_EINVAL for a count out of range.  Does not change results beyond FP32
- * rounding order. */
+ * rounding order.  Runs that stay on the chip (ep_run and ep_run_host with two
+ * or more steps, ep_run_adjoint, the ep_grad_* calls) have a thread count of
+ * their own, and take neither of these nor the stages of ep_set_pipeline. */
 int ep_set_threads(ep_schedule *s, int32_t threads);
 int ep_set_adjoint_threads(ep_schedule *s, int32_t threads);
 

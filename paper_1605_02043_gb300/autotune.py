@@ -15,6 +15,11 @@ do not fit in the L2:
 2. confirmation: the `confirm` fastest screening rows are timed again the same
    way on the whole set of graphs, and the fastest of those wins.
 
+What is timed, and so what is tuned, are the step kernels: single steps, and
+runs and gradients of batches that do not fit the chip.  Where a batch does fit
+(Schedule.grad_sizes(D) is not zero) its runs and gradients take neither stages
+nor threads from here, and C only sets the order that the parts are cut from.
+
 Results are cached in a JSON file keyed by a hash of the graphs and the
 candidate lists, so a rerun skips the search.
 """

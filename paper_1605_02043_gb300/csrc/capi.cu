@@ -143,8 +143,8 @@ struct ep_schedule {
   // workspace
   DBuf ws_x, ws_out, ws_w, ws_bacc, ws_lam, ws_gw, ws_hist, ws_flags, ws_cnt;
   DBuf ws_hx, ws_hw, ws_hout;
-  // vertex-ordered maps for inputs read from host memory (built on first use):
-  // records of every vertex (CSR) and the weight slots of every task (2 each)
+  // vertex-ordered maps (built on first use): records of every vertex (CSR, a
+  // state in) and the weight slots of every task (2 each, weights in host memory)
   DBuf d_hptr, d_hrec, d_tslot;
   bool host_maps = false, task_slots = false;
   // shard halo (ep_set_halo): shared id of every halo vertex here, -1 if untouched

@@ -18,7 +18,8 @@ namespace ep {
 //              the state record rec_lo + p and a block's vertex set is one
 //              contiguous run; sid_list[h0 + p - ni] is the shared id h that
 //              indexes the accumulators (kSidFirst marks the first copy of h).
-// Within each class positions are ordered by descending in-block degree.
+// Within each class positions are ordered by descending in-block degree, but for
+// swaps inside octets of eight positions that even out the banks (banks.h).
 // Incidence in sliced-ELL form: slice j holds the positions [32 j, 32 j + 32);
 // its incidence entries occupy K_j = soff[q0 + j + 1] - soff[q0 + j] columns
 // of 32 slots, slot = s0 + 32 * soff[q0 + j] + 32 * column + lane, so that a

@@ -3,10 +3,12 @@
 // A run of several explicit steps keeps the whole mesh on the chip: the data
 // vertices, in the order of first appearance over the schedule's blocks
 // (cpack, Section 4.1, the locality the partition made), are cut into one
-// contiguous part per CUDA block.  A part owns its vertices: it computes the
-// whole flux of each of them (pull form, every task at both endpoints, as the
-// step kernels do), so nothing is accumulated across parts; what a part needs
-// from the others is the value of the neighbours it does not own (its halo).
+// part per CUDA block, and vertices that have most of their neighbours in
+// another part then move there (march.cpp, smooth_parts).  A part owns its
+// vertices: it computes the whole flux of each of them (pull form, every task at
+// both endpoints, as the step kernels do), so nothing is accumulated across
+// parts; what a part needs from the others is the value of the neighbours it
+// does not own (its halo).
 #pragma once
 
 #include <cstdint>
@@ -19,16 +21,19 @@ namespace ep {
 
 // One part.  Positions [0, own): its vertices, the boundary ones (in some
 // other part's halo) first, each class by descending degree; positions
-// [hbase, hbase + nh): the halo, ascending by record.  Position p is the state
-// record lo + p, own or halo, so a part's image is one run of records; halo[h0
-// + j] is the record where halo position j is its owner's.  Slices of 32
-// positions are dealt to `warps` warps, slice j to warp j % warps; the pair
-// columns (32 lanes of two slots each) of one warp's slices follow each other,
-// so that a warp reads its columns as one stream: warp v's start at column s0 +
-// tab[q0 + v], and slice j has tab[q0 + warps + j] of them.  Entry pair 32 *
-// column + lane holds two 16-bit entries (position of the other endpoint,
-// kSlotSrc on the task's first endpoint) and two weights.  An unused slot names
-// the lane's own position with weight 0 (its difference is zero by itself).
+// [hbase, hbase + nh): the halo, ascending by record; both but for swaps inside
+// the octets of eight positions, which even out the banks (banks.h).  Position p
+// is the state record lo + p, own or halo, so a part's image is one run of
+// records; halo[h0 + j] is the record where halo position j is its owner's.
+// Slices of 32 positions are dealt to `warps` warps, slice j to warp j % warps;
+// the pair columns (32 lanes of two slots each) of one warp's slices follow each
+// other, so that a warp reads its columns as one stream: warp v's start at
+// column s0 + tab[q0 + v], and slice j has tab[q0 + warps + j] of them.  Entry
+// pair 32 * column + lane holds two 16-bit entries (position of the other endpoint,
+// kSlotSrc on the task's first endpoint) and two weights.  An unused slot has
+// weight 0 and names the lane's own position or one of its neighbours, whichever
+// costs the fewest bank conflicts: its term is zero whenever the lane's used
+// slots are finite.  A lane of no vertex names what another lane reads.
 struct MarchPart {
   int32_t lo, own, nb, nsl;
   int32_t hbase, nh, h0, q0;
