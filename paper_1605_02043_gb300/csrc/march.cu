@@ -328,7 +328,7 @@ __device__ __forceinline__ void forward_slices(const MarchArgs& a, const MarchPa
     for (int c = 0; c < D; ++c) acc[c] = 0.f;
   };
   auto take = [&](uint32_t e, float2 w, int) {  // acc += w (x_o - x_p) / (1 + |x_o - x_p|^2), two slots
-    float d0[D], d1[D], q0 = 0.f, q1 = 0.f;
+    float d0[D], d1[D], q0 = kDenStart<D>, q1 = kDenStart<D>;
     rec_load<D>(xs, npos, e & kSlotPos, d0);
     rec_load<D>(xs, npos, (e >> 16) & kSlotPos, d1);
 #pragma unroll
@@ -336,7 +336,7 @@ __device__ __forceinline__ void forward_slices(const MarchArgs& a, const MarchPa
       d0[c] -= xp[c], d1[c] -= xp[c];
       q0 = fmaf(d0[c], d0[c], q0), q1 = fmaf(d1[c], d1[c], q1);
     }
-    const float f0 = w.x * rcp_approx(1.f + q0), f1 = w.y * rcp_approx(1.f + q1);
+    const float f0 = w.x * rcp_den<D>(q0), f1 = w.y * rcp_den<D>(q1);
 #pragma unroll
     for (int c = 0; c < D; ++c) acc[c] = fmaf(f1, d1[c], fmaf(f0, d0[c], acc[c]));
   };
@@ -480,7 +480,7 @@ __device__ __forceinline__ void adjoint_slices(const MarchArgs& a, const MarchPa
     for (int c = 0; c < D; ++c) acc[c] = 0.f;
   };
   auto one = [&](uint32_t e, float w, float* g) {
-    float dx[D], dl[D], q = 0.f, dg = 0.f;
+    float dx[D], dl[D], q = kDenStart<D>, dg = 0.f;
     rec_load<D>(S.x, npos, e & kSlotPos, dx);
     rec_load<D>(S.lam, npos, e & kSlotPos, dl);
 #pragma unroll
@@ -490,7 +490,7 @@ __device__ __forceinline__ void adjoint_slices(const MarchArgs& a, const MarchPa
       q = fmaf(dx[c], dx[c], q);
       dg = fmaf(dx[c], dl[c], dg);
     }
-    const float inv = rcp_approx(1.f + q), s = dg * inv, two = 2.f * s * inv;
+    const float inv = rcp_den<D>(q), s = dg * inv, two = 2.f * s * inv;
 #pragma unroll
     for (int c = 0; c < D; ++c) acc[c] -= w * (dl[c] * inv - two * dx[c]);
     if (e & kSlotSrc) {  // one lane's slot throughout: no reader before the next launch

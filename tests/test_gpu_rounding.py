@@ -43,7 +43,7 @@ def rms(got, ref):
     return float(np.sqrt(np.mean(((got - ref)[ok] / ref[ok]) ** 2)))
 
 
-@pytest.mark.parametrize("D", [5, 8])
+@pytest.mark.parametrize("D", [1, 5, 8])
 @pytest.mark.parametrize("path", ["run", "pipelined", "one block", "read-only"])
 def test_forward_term(D, path):
     S, src, dst, x, _, term = matching(D, D)
@@ -61,7 +61,7 @@ def test_forward_term(D, path):
     assert S.check_errors() == 0
 
 
-@pytest.mark.parametrize("D", [5, 8])
+@pytest.mark.parametrize("D", [1, 5, 8])
 @pytest.mark.parametrize("path", ["run", "pipelined", "one block"])
 def test_adjoint_term(D, path):
     # a cotangent of one component at the first endpoints: the weight gradient
